@@ -4,39 +4,29 @@
 //
 // GB300 design (the paper's one 64-thread block per MCU with a 32-lane code compare,
 // Sec. 5.2, is prior art here):
-//  * persistent grid; each warp takes batches of m_eff work items (one per lane), m_eff the
-//    smallest power of two up to M (4, 8, 16 or 32, the buffer width) that covers the list
-//    in one batch per warp, and a long list fills the lanes. A short list (a frame under
-//    motion with a warm block cache: at most kWarpMcuMax MCUs per warp) goes one MCU at a
-//    time, each decoded by the whole warp (decode_mcu_warp, mcu_warp_pixels), spread first
-//    over the SMs. The first batch of each warp is fixed by its rank, later ones come from a
-//    device counter, so uneven MCU sizes balance dynamically and the count never goes to
-//    the host;
-//  * entropy phase: lane m < m_eff runs MCU m's serial entropy chain over all its data
-//    units from a byte-swapped copy of its words staged in shared memory (a per-warp pool
-//    shared out by a prefix sum). Per symbol: one funnel shift of a two-word window, one
-//    10-bit LUT read (16-bit entries: code length, value size, run) together with an
-//    independent read of the second-level entry for codes longer than 10 bits, the value
-//    cut from the same window without a branch, and a select to advance the window. The
-//    quantised coefficients go in zig-zag order into a per-warp buffer coef[du][k][m]
-//    (int16). Nothing but the LUT and the stream is read on this serial chain:
-//    dequantisation waits for the IDCT phase;
-//  * IDCT phase: the batch's data units are shared out over all 32 lanes, one (data unit,
-//    MCU) pair per lane and round; lanes of one round read consecutive columns of the
-//    buffer (conflict-free), and all zig-zag positions are compile-time constants. Columns
-//    are dequantised on load with the MCU's quantisation table (read through L1); even/odd
-//    butterflies give an exact integer factorisation of the matrix product of the decode
-//    spec; the row pass writes each row's pixels in place over the slots it just read;
-//  * colour phase: 4:2:0 tiles are shared out as (MCU, group of four texels) pairs, 16-byte
-//    stores; 4:4:4 and reduced-resolution tiles are written by the MCU's own lane.
-//    The buffers per MCU are 768 B of coefficients plus 128 B of staged words, so up to
-//    seven 32-MCU warps fit on an SM.
+//  * persistent grid; each warp takes batches of m_eff <= M work items (M = 4, 8, 16 or 32, the
+//    buffer width), chosen from the list's length on the device, so the count never goes to
+//    the host. The first batch of each warp is fixed, later ones come from a device counter,
+//    so uneven MCU sizes balance dynamically;
+//  * entropy phase: lane m < m_eff runs MCU m's serial chain over all its data units from a
+//    byte-swapped copy of its words staged in shared memory (a per-warp pool shared out by a
+//    prefix sum). The chain bounds the pass (it ends with the heaviest MCU), so a symbol's
+//    dependent path is kept to one table read and a few ALU operations (entropy_fast);
+//  * pixel phase: the warp takes its MCUs one by one. Both IDCT passes of an 8x8 data unit
+//    are one mma.sync each (an 8x8 by 8x8 product, exact in fp32: see idct_pass), the
+//    fragment layouts make the first product's output the second one's input without a
+//    shuffle, and a lane ends up with two pixels of every data unit of the MCU in registers,
+//    which it colour-converts in packed 16-bit pairs and stores as 32-byte rows of texels.
+//    Nothing goes through memory between the coefficients and the tile.
 //
 // Decode spec (identical in the oracle): dequantised d = clamp16(q * Q); column pass
 // t = clamp16(floor((sum_v K[y][v] d[v][u] + 2^8) / 2^9)); row pass
 // p = clamp(floor((sum_u K[x][u] t[y][u] + 2^18) / 2^19) + 128, 0, 255) with
 // K[x][u] = round(2^14 c_u cos((2x+1) u pi / 16)); JFIF colour in 16-bit fixed point;
-// 4:2:0 chroma replicated within the MCU; DC values wrap modulo 2^16.
+// 4:2:0 chroma replicated within the MCU; DC values wrap modulo 2^16. A reduced level
+// (1/2^r) uses K_N[x][u] = round(2^14 c_u cos((2x+1) u pi / (2N))) on the N x N lowest
+// frequencies, N = 8 >> r, with the same rounding.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <cstddef>
@@ -45,6 +35,8 @@
 
 namespace jt {
 namespace {
+
+extern __shared__ __align__(16) uint8_t smem[];
 
 // ---- integer IDCT constants: round(8192 cos(k pi / 16)), k = 1..7 ----
 constexpr int C1 = 8035, C2 = 7568, C3 = 6811, C4 = 5793, C5 = 4551, C6 = 3135, C7 = 1598;
@@ -61,741 +53,524 @@ static_assert(zz_pos(0, 0) == 0 && zz_pos(0, 1) == 1 && zz_pos(1, 0) == 2 && zz_
                   zz_pos(0, 2) == 5 && zz_pos(7, 6) == 62 && zz_pos(7, 7) == 63 && zz_pos(3, 4) == 31 && zz_pos(4, 3) == 32,
               "zig-zag positions");
 
-// 1-D 8-point IDCT: out[x] = sum_u K[x][u] in[u], K as above, by even/odd parts.
-// K[7-x][u] = (-1)^u K[x][u] exactly, so out[x] = E[x] + O[x], out[7-x] = E[x] - O[x].
-__device__ __forceinline__ void idct8(const int in[8], int out[8]) {
-  const int a0 = C4 * (in[0] + in[4]), a1 = C4 * (in[0] - in[4]);
-  const int b0 = C2 * in[2] + C6 * in[6], b1 = C6 * in[2] - C2 * in[6];
-  const int e0 = a0 + b0, e3 = a0 - b0, e1 = a1 + b1, e2 = a1 - b1;
-  const int o0 = C1 * in[1] + C3 * in[3] + C5 * in[5] + C7 * in[7];
-  const int o1 = C3 * in[1] - C7 * in[3] - C1 * in[5] - C5 * in[7];
-  const int o2 = C5 * in[1] - C1 * in[3] + C7 * in[5] + C3 * in[7];
-  const int o3 = C7 * in[1] - C5 * in[3] + C3 * in[5] - C1 * in[7];
-  out[0] = e0 + o0; out[7] = e0 - o0;
-  out[1] = e1 + o1; out[6] = e1 - o1;
-  out[2] = e2 + o2; out[5] = e2 - o2;
-  out[3] = e3 + o3; out[4] = e3 - o3;
-}
-
-__device__ __forceinline__ int sat16(int v) { return min(32767, max(-32768, v)); }
-__device__ __forceinline__ uint32_t clamp255(int v) { return (uint32_t)min(255, max(0, v)); }
-
-// N-point IDCT of the N lowest frequencies, N = 4, 2, 1 (reduced-resolution decode):
-// out[x] = sum_u K_N[x][u] in[u] with K_N[x][u] = round(2^14 c_u cos((2x+1) u pi / (2N))) and
-// the 8-point c_u. The N-point cosines are the 8-point ones at even multiples, so N = 4 is
-// the even half of idct8 (inputs at 0, 2, 4, 6), N = 2 its first butterfly, N = 1 the DC term.
-template <int N>
-__device__ __forceinline__ void idct_small(const int in[4], int out[4]) {
-  if (N == 4) {
-    const int a0 = C4 * (in[0] + in[2]), a1 = C4 * (in[0] - in[2]);
-    const int b0 = C2 * in[1] + C6 * in[3], b1 = C6 * in[1] - C2 * in[3];
-    out[0] = a0 + b0; out[1] = a1 + b1; out[2] = a1 - b1; out[3] = a0 - b0;
-  } else if (N == 2) {
-    out[0] = C4 * (in[0] + in[1]);
-    out[1] = C4 * (in[0] - in[1]);
-  } else {
-    out[0] = C4 * in[0];
-  }
+// K_N[x][u] for N = 8 >> r (zero outside N x N): the N-point cosines are the 8-point ones at
+// multiples of 8 / N.
+__device__ __forceinline__ int idct_k(int x, int u, int r) {
+  const int n = 8 >> r;
+  if (x >= n || u >= n) return 0;
+  int i = ((2 * x + 1) * u << r) & 31;  // angle in units of pi / 16
+  i = i > 16 ? 32 - i : i;
+  const int j = i > 8 ? 16 - i : i;  // 1..7 unless u = 0
+  const int c = j == 1 ? C1 : j == 2 ? C2 : j == 3 ? C3 : j == 4 ? C4 : j == 5 ? C5 : j == 6 ? C6 : C7;
+  return u == 0 ? C4 : (i > 8 ? -c : c);
 }
 
 // Words of the MCUs' entropy-coded data copied to shared memory before their serial decode
 // (random loads from HBM take thousands of cycles and would otherwise sit on the serial
 // chain once per word). A warp has kStageWords words per MCU as one pool, shared out by a
 // prefix sum over its lanes, so a long MCU can use what short ones leave (the mean MCU of a
-// scene needs about a quarter). Words are stored big-endian-swapped; a lane whose MCU does
-// not fit reads the rest from global memory.
+// scene needs about a quarter). When the batch's MCUs do not fit, each is staged in parts: its
+// chain stops short of the staged words' end and goes on when the next part is there. Words
+// are stored big-endian-swapped.
 constexpr int kStageWords = 32;
 
-// Shared memory of one warp: coefficients [6][64][M] int16 (zig-zag order k, lane m at
-// column m; after the row pass each data unit's slots hold its pixels, see below) and the
-// staged entropy-coded words [M * kStageWords].
-__host__ __device__ constexpr size_t warp_smem(int M) {
-  return (size_t)6 * 64 * M * 2 + (size_t)M * kStageWords * 4;
-}
+// Shared memory of one warp: per MCU six data units of 64 int16 coefficients in zig-zag order,
+// then the staged words [M * kStageWords]. An MCU's 772 bytes are an odd number of words,
+// so that lanes storing the same coefficient of their MCUs hit different banks; a data unit
+// is 32 words, so the pixel phase's reads of one data unit never conflict.
+constexpr int kMcuBytes = 6 * 128 + 4;
+static_assert(kMcuBytes / 4 % 2 == 1 && 4 * kMcuBytes % 16 == 0, "bank spread, and 16-byte whole for M >= 4");
+__host__ __device__ constexpr size_t warp_smem(int M) { return (size_t)M * (kMcuBytes + kStageWords * 4); }
 
 __device__ __forceinline__ uint32_t bswap(uint32_t w) { return __byte_perm(w, 0, 0x0123); }
 
-// Stream word i (relative to the lane's first staged word): from the staged copy when it is
-// there, else from global memory (past the end of the stream: 0).
-__device__ __forceinline__ uint32_t lds_u32(uint32_t saddr) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(saddr));
-  return v;
-}
-__device__ __forceinline__ uint32_t lds_u16(uint32_t saddr) {
-  uint16_t v;
-  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(saddr));
-  return v;
-}
+__device__ __forceinline__ uint32_t sm_u32(uint32_t off) { return *reinterpret_cast<const uint32_t*>(smem + off); }
+__device__ __forceinline__ int16_t& sm_i16(uint32_t off) { return *reinterpret_cast<int16_t*>(smem + off); }
 
-// Stream word i (relative to the lane's first staged word): from the staged copy (shared
-// memory address st) when it is there, else from global memory (past the end: 0).
-struct Words {
-  uint32_t st;            // shared-memory address of the staged, byte-swapped words
-  uint32_t nst;           // words staged
-  const uint32_t* gw;     // stream words from the first staged word on
-  uint32_t ngw;           // readable words from gw on
-  __device__ __forceinline__ uint32_t operator()(uint32_t i) const {
-    if (i < nst) return lds_u32(st + 4 * i);
-    return i < ngw ? bswap(__ldg(gw + i)) : 0u;
-  }
-};
-
-// Reads of the table set on the serial chain: explicit shared-memory loads for the staged
-// set (address hs_sa), generic loads through hs otherwise.
-template <bool SH>
-struct Tables {
-  const HuffTable* hs;
-  uint32_t hs_sa;
-  __device__ __forceinline__ uint32_t lut(uint32_t ti, uint32_t i) const {
-    return SH ? lds_u16(hs_sa + ti * (uint32_t)sizeof(HuffTable) + i * 2) : (uint32_t)hs[ti].lut[i];
-  }
-  __device__ __forceinline__ uint32_t lut2(uint32_t ti, uint32_t j) const {
-    return SH ? lds_u16(hs_sa + ti * (uint32_t)sizeof(HuffTable) + (uint32_t)offsetof(HuffTable, lut2) + j * 2)
-              : (uint32_t)hs[ti].lut2[j];
-  }
-  __device__ __forceinline__ uint32_t first16(uint32_t ti) const {
-    return SH ? lds_u32(hs_sa + ti * (uint32_t)sizeof(HuffTable) + (uint32_t)offsetof(HuffTable, first16))
-              : hs[ti].first16;
-  }
-  __device__ __forceinline__ uint32_t n2(uint32_t ti) const {
-    return SH ? lds_u32(hs_sa + ti * (uint32_t)sizeof(HuffTable) + (uint32_t)offsetof(HuffTable, n2)) : hs[ti].n2;
-  }
-  // table ti as a byte address (shared) or byte offset from hs (global), and reads through it
-  __device__ __forceinline__ uint32_t base(uint32_t ti) const {
-    return (SH ? hs_sa : 0u) + ti * (uint32_t)sizeof(HuffTable);
-  }
-  __device__ __forceinline__ uint32_t lut_at(uint32_t b, uint32_t i) const {
-    return SH ? lds_u16(b + i * 2) : (uint32_t)*reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(hs) + b + i * 2);
-  }
-  __device__ __forceinline__ uint32_t lut2_at(uint32_t b, uint32_t j) const {
-    const uint32_t o = b + (uint32_t)offsetof(HuffTable, lut2) + j * 2;
-    return SH ? lds_u16(o) : (uint32_t)*reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(hs) + o);
-  }
-};
-
-// Symbol entry by the MAXCODE walk (T.81 F.2.2.3), or 0 for an invalid code or a symbol
-// invalid for the table's class. Only codes without a LUT entry come here.
-__device__ __noinline__ uint32_t walk_symbol(const HuffTable* t, uint32_t w, bool dc) {
+// Symbol entry by the MAXCODE walk (T.81 F.2.2.3), or kNoEntry for an invalid code or a symbol
+// invalid for the table's class. Only codes without a table entry come here.
+__device__ __noinline__ uint32_t walk_symbol(const HuffWalk* t, uint32_t w, bool dc) {
   const uint32_t top = w >> 16;
 #pragma unroll 1
   for (int l = 1; l <= 16; ++l) {
     const int code = (int)(top >> (16 - l));
     if (code <= t->maxcode[l]) {
       const int vi = code + t->valoff[l];
-      if (vi < 0 || vi > 255) return 0;
+      if (vi < 0 || vi > 255) return kNoEntry;
       const uint32_t sym = t->vals[vi];
       const uint32_t r = dc ? 0 : sym >> 4, s = dc ? sym : sym & 15;
-      if (s > (dc ? 11u : 10u)) return 0;
-      if (!dc && s == 0) return r == 0 ? huff_entry(l, 0, kRunEob) : (r == 15 ? huff_entry(l, 0, 15) : 0u);
+      if (s > (dc ? 11u : 10u)) return kNoEntry;
+      if (!dc && s == 0) return r == 0 ? huff_entry(l, 0, kRunEob) : (r == 15 ? huff_entry(l, 0, 15) : kNoEntry);
       return huff_entry(l, s, r);
     }
   }
-  return 0;
+  return kNoEntry;
 }
 
-// Entropy-decodes all data units of one MCU into coef[(du * 64 + k) * M] (quantised, zig-zag
-// k; the buffer must be zero on entry). One symbol per iteration, on a short dependent
-// chain: a funnel shift cuts the next 32 bits from the two-word window (hi:lo), one LUT
-// read gives (l, s, r), the s value bits are cut from the same window (T.81 EXTEND without
-// a branch), and the window advances by a select; the next stream word is read ahead. The
-// move to the next data unit (predictor save/restore, table choice) is also branch-free.
-// hs: the lane's tables (shared or global memory). CPT: the compact form, where the first
-// luma data unit and the chroma data units carry no DC difference and their DCs are
-// p0, p1, p2 as given. Returns the bit position after the MCU relative to the first staged
-// word, or 0xFFFFFFFF on an invalid coding.
-template <int M, bool SH, bool CPT>
-__device__ __forceinline__ uint32_t decode_mcu(const Words& W, uint32_t bit0, const Tables<SH>& T, int ndu,
-                                               int16_t& p0, int16_t& p1, int16_t& p2, int16_t* coef) {
-  constexpr bool cpt = CPT;
-  uint32_t widx = bit0 >> 5, pos = bit0 & 31;
-  uint32_t hi = W(widx), lo = W(widx + 1), nx = W(widx + 2);
-  // second-level ranges of the four tables, held in registers so that no table read other
-  // than the two LUT entries sits on the chain
-  const uint32_t F0 = T.first16(0), F1 = T.first16(1), F2 = T.first16(2), F3 = T.first16(3);
-  const uint32_t N0 = T.n2(0), N1 = T.n2(1), N2 = T.n2(2), N3 = T.n2(3);
-  int du = 0, k = cpt ? 1 : 0, comp = 0, pc = p0, q0 = p0, q1 = p1, q2 = p2;
-  // the table of the symbol being decoded (0 DC luma, 1 AC luma, 2 DC chroma, 3 AC chroma),
-  // its address and second-level range. The two possible successors (the next data unit's
-  // first table, or this one's AC table) are prepared before the symbol is read, so the
-  // symbol only has to select between them: a short dependent chain from one LUT read to the
-  // next.
-  uint32_t tcur = cpt ? 1u : 0u;
-  uint32_t bcur = T.base(tcur), fcur = cpt ? F1 : F0, ncur = cpt ? N1 : N0;
-  uint32_t boff = 0;
-  if (cpt) coef[0] = (int16_t)pc;
-  bool bad = false;
-#pragma unroll 1
-  for (int it = 0; it < 64 * 6; ++it) {  // at most 64 symbols per data unit
-    // successors, off the chain: the next data unit's component and first table, and the
-    // AC table of this data unit
-    const int cn1 = du + 1 < ndu - 2 ? 0 : (du + 1 == ndu - 2 ? 1 : 2);
-    const uint32_t tA = cn1 ? (cpt ? 3u : 2u) : 0u, tB = tcur | 1u;
-    const uint32_t bA = T.base(tA), bB = T.base(tB);
-    const uint32_t fA = cn1 ? (cpt ? F3 : F2) : F0, fB = (tcur & 2u) ? F3 : F1;
-    const uint32_t nA = cn1 ? (cpt ? N3 : N2) : N0, nB = (tcur & 2u) ? N3 : N1;
-    const int lim = 63 - k;  // the data unit ends when the run reaches it
-    const bool dc = k == 0;
-
-    const uint32_t w = __funnelshift_l(lo, hi, pos);
-    // both levels read at once (independent loads): the first-level entry when the code is
-    // short, else the second-level entry of the 16-bit prefix
-    const uint32_t e1 = T.lut_at(bcur, w >> (32 - kLutBits));
-    const uint32_t j = (w >> 16) - fcur;
-    const uint32_t e2 = T.lut2_at(bcur, min(j, (uint32_t)kLut2Size - 1u));
-    uint32_t e = (e1 & 31u) ? e1 : (j < ncur ? e2 : 0u);
-    if (e == 0) {  // no table entry: the MAXCODE walk decodes or rejects it
-      e = walk_symbol(T.hs + tcur, w, dc);
-      if (e == 0) {
-        bad = true;
-        break;
-      }
-    }
-    const uint32_t l = e & 31u, sz = (e >> 5) & 15u, r = e >> 9;
-    const bool done = (int)r >= lim;  // data unit complete
-    tcur = done ? tA : tB;
-    bcur = done ? bA : bB;
-    fcur = done ? fA : fB;
-    ncur = done ? nA : nB;
-    const uint32_t tw = w << l;
-    // EXTEND: the s bits after the code; a leading 0 bit makes the value negative
-    int v = (int)__funnelshift_l(tw, 0u, sz) + (int)(~((int)tw >> 31) & (int)(1u - (1u << sz)));
-    pos += l + sz;
-    const bool step = pos >= 32;
-    hi = step ? lo : hi;
-    lo = step ? nx : lo;
-    pos = step ? pos - 32 : pos;
-    widx += step ? 1u : 0u;
-    nx = W(widx + 2);
-    const int dcv = (int16_t)(uint16_t)(pc + v);  // DC values wrap modulo 2^16
-    v = dc ? dcv : v;
-    pc = dc ? dcv : pc;
-    const int kst = k + (int)r;
-    bad |= sz != 0 && kst > 63;
-    coef[(boff + (uint32_t)min(kst, 63)) * M] = (int16_t)v;
-    q0 = done && comp == 0 ? pc : q0;
-    q1 = done && comp == 1 ? pc : q1;
-    q2 = done && comp == 2 ? pc : q2;
-    du += done ? 1 : 0;
-    pc = done ? (cn1 == 0 ? q0 : (cn1 == 1 ? q1 : q2)) : pc;
-    comp = done ? cn1 : comp;
-    boff += done ? 64u : 0u;
-    k = done ? ((cpt && cn1 != 0) ? 1 : 0) : kst + 1;
-    if (du == ndu || bad) break;
-    if (cpt && done && cn1 != 0) coef[boff * M] = (int16_t)pc;  // compact form: a stored chroma DC
-  }
-  p0 = (int16_t)q0;
-  p1 = (int16_t)q1;
-  p2 = (int16_t)q2;
-  return (bad || du != ndu) ? 0xFFFFFFFFu : widx * 32 + pos;
+// Signed value of a symbol with entry e whose code starts at the top of w (T.81 EXTEND; 0
+// without value bits).
+__device__ __forceinline__ int symbol_value(uint32_t w, uint32_t e) {
+  const int m = (int)(0xFFFFFFFFu << ((e >> 5) & 15u));      // -2^s
+  const int raw = (int)(__funnelshift_l(w, 0u, e) & ~m);     // (shifts by the low five bits of e)
+  return raw + (2 * raw + m < 0 ? m + 1 : 0);
 }
 
-// Entropy-decodes one data unit of component comp (0 luma, else chroma) from bit0 into
-// coef[k * M] (zig-zag k; zero on entry); its DC slot receives the DC *difference* (the
-// caller chains it). Same symbol step as decode_mcu, without data-unit transitions: the DC
-// table for the first symbol, then the AC table. Returns the bit position after the unit
-// relative to the first staged word, or 0xFFFFFFFF on an invalid coding.
-template <int M, bool SH>
-__device__ __forceinline__ uint32_t decode_unit(const Words& W, uint32_t bit0, const Tables<SH>& T, int comp,
-                                                int16_t* coef) {
-  uint32_t widx = bit0 >> 5, pos = bit0 & 31;
-  uint32_t hi = W(widx), lo = W(widx + 1), nx = W(widx + 2);
-  const uint32_t tdc = comp ? 2u : 0u, tac = tdc | 1u;
-  const uint32_t bac = T.base(tac), fac = T.first16(tac), nac = T.n2(tac);
-  uint32_t tcur = tdc, bcur = T.base(tdc), fcur = T.first16(tdc), ncur = T.n2(tdc);
-  int k = 0;
-  bool bad = false;
-#pragma unroll 1
-  for (int it = 0; it < 64; ++it) {  // every symbol advances k by at least one
-    const uint32_t w = __funnelshift_l(lo, hi, pos);
-    const uint32_t e1 = T.lut_at(bcur, w >> (32 - kLutBits));
-    const uint32_t j = (w >> 16) - fcur;
-    const uint32_t e2 = T.lut2_at(bcur, min(j, (uint32_t)kLut2Size - 1u));
-    uint32_t e = (e1 & 31u) ? e1 : (j < ncur ? e2 : 0u);
-    if (e == 0) {
-      e = walk_symbol(T.hs + tcur, w, k == 0);
-      if (e == 0) {
-        bad = true;
-        break;
-      }
-    }
-    const uint32_t l = e & 31u, sz = (e >> 5) & 15u, r = e >> 9;
-    const uint32_t tw = w << l;
-    const int v = (int)__funnelshift_l(tw, 0u, sz) + (int)(~((int)tw >> 31) & (int)(1u - (1u << sz)));
-    pos += l + sz;
-    const bool step = pos >= 32;
-    hi = step ? lo : hi;
-    lo = step ? nx : lo;
-    pos = step ? pos - 32 : pos;
-    widx += step ? 1u : 0u;
-    nx = W(widx + 2);
-    const int kst = k + (int)r;
-    bad |= sz != 0 && kst > 63;
-    coef[min(kst, 63) * M] = (int16_t)v;
-    k = kst + 1;
-    tcur = tac;
-    bcur = bac;
-    fcur = fac;
-    ncur = nac;
-    if (k >= 64 || bad) break;
-  }
-  return (bad || k < 64) ? 0xFFFFFFFFu : widx * 32 + pos;
+// Stores a coefficient when c holds: a predicated store, never a branch.
+__device__ __forceinline__ void store_if(bool c, uint32_t off, int v) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.shared.u16 [%0], %1;\n\t}" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(smem) + off),
+               "h"((int16_t)v), "r"((uint32_t)c)
+               : "memory");
 }
 
-// ---- one MCU decoded by a whole warp (short work lists) ----
+// Reads a table record when c holds: predicated loads, which nothing waits for where they are
+// not made.
+template <bool CAP>
+__device__ __forceinline__ void load_if(bool p, uint32_t off, uint4& t, uint4& c) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(smem) + off;
+  if (CAP)
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %9, 0;\n\t@q ld.shared.v4.u32 {%0, %1, %2, %3}, [%8];\n\t"
+                 "@q ld.shared.v4.u32 {%4, %5, %6, %7}, [%8+16];\n\t}"
+                 : "+r"(t.x), "+r"(t.y), "+r"(t.z), "+r"(t.w), "+r"(c.x), "+r"(c.y), "+r"(c.z), "+r"(c.w)
+                 : "r"(a), "r"((uint32_t)p));
+  else
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %6, 0;\n\t@q ld.shared.v4.u32 {%0, %1, %2, %3}, [%5];\n\t"
+                 "@q ld.shared.u32 %4, [%5+16];\n\t}"
+                 : "+r"(t.x), "+r"(t.y), "+r"(t.z), "+r"(t.w), "+r"(c.x)
+                 : "r"(a), "r"((uint32_t)p));
+}
+__device__ __forceinline__ void load_if(bool p, const char* a, uint4& t, uint4& c) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %9, 0;\n\t@q ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%8];\n\t"
+               "@q ld.global.nc.v4.u32 {%4, %5, %6, %7}, [%8+16];\n\t}"
+               : "+r"(t.x), "+r"(t.y), "+r"(t.z), "+r"(t.w), "+r"(c.x), "+r"(c.y), "+r"(c.z), "+r"(c.w)
+               : "l"(a), "r"((uint32_t)p));
+}
+
+constexpr uint32_t kNoSet = 0xFFFFFFFFu;
+constexpr uint32_t kBusyWarps = 12;         // three per SM sub-partition
+constexpr uint32_t kInvalid = 0x80000000u;  // an invalid coding (bit positions stay far below)
+constexpr uint32_t kSizeMask = 15u << 5;
+constexpr uint32_t kPast = (64u << kRunShift) - (1u << (kRunShift - 1));  // k + entry past slot 63, or kNoEntry at any k
+static_assert((63u << kRunShift) + kSizeMask + 31u < kPast && kNoEntry >= kPast, "the last valid place, and no entry");
+constexpr uint32_t kSlackBytes = 1344;      // shared memory a chain may read past its staged words
+
+// Entropy-decodes the `ndu` data units of one MCU (or one data unit) from words staged whole at
+// shared offset st (nst of them) into coef (shared offset; [du][k] int16 in zig-zag order,
+// zero on entry), with the tables of record seq of the set (SH: the staged set 0, else
+// `set`). DC slots receive the DC *difference*.
 //
-// A warp that holds a single MCU would run its serial chain on one lane, and every step of
-// that chain (window cut, LUT read, length, position, coefficient store) waits for the one
-// before. Here the 32 lanes instead decode, for every bit offset of a 256-bit window of the
-// stream, the AC symbol that would start there (entries independent of each other, 8 per
-// lane, loads issued before any store), and the chain that remains is one shared-memory read
-// per one or two symbols: the slot at the current position holds the byte offset of the slot
-// after its symbol (code + value bits), its run and its value, and the same for the symbol
-// after it, so a read serves two symbols unless the first ends the data unit. All lanes follow the chain in
-// step, so its state is warp-uniform; symbol s of a data unit is kept in registers by lane
-// s mod 32, and the coefficients are stored once the data unit ends (a store on the chain
-// would hold the next table read behind it). The DC symbol of each data unit is decoded
-// directly on the chain. The window is rebuilt when the position leaves it or the component
-// class (luma, chroma) changes.
-constexpr int kWinBits = 256;    // window of symbol entries, bits (128 when the buffer is 4 MCUs wide)
-constexpr int kWarpMcuMax = 4;   // lists of at most this many MCUs per warp are decoded MCU by MCU
+// The serial chain per symbol bounds the pass: it ends with the heaviest MCU, decoded by a
+// warp with few other lanes left, which issues in order, so what counts is the number of
+// instructions per symbol and that none of them is a branch (a branch costs a lone warp 20
+// to 30 cycles; the loop's back edge is taken once per kSymbols symbols). One table read
+// serves codes of any length (see HuffSet). The bits behind the 32-bit window are cut from
+// the staged words again for every symbol, which is cheaper than refilling a buffer. Data-unit
+// bookkeeping is a record pointer: the tables come from the record, and a chain past its
+// last data unit reads a table of zeros (a symbol without value or length). Measured on the
+// heaviest 4:2:0 MCU of a 1080p frame (193 symbols): 360 cycles a symbol with the same work in
+// branches, 208 with a buffer refilled by selects and a two-level table, 133 with both
+// successors' entries read and one selected.
+//
+// Runs from ch.pos to the end of the chain or to the first group of kSymbols symbols that starts
+// at bit `limit` (of shared memory) or later; returns false for a symbol without a table entry
+// or past the data unit's end. Bits past the staged words are whatever lies there (at most 384
+// symbols of 27 bits on, inside the allocation with its slack): the caller redoes the MCU with
+// entropy_any when it consumed any, or for false.
+constexpr int kSymbols = 4;
+constexpr uint32_t kGroupBits = kSymbols * 27 + 64;  // a group consumes and looks ahead at most this far
 
-// LUT entry of the code at the top of w in table ti (0 when it has none).
-template <bool SH>
-__device__ __forceinline__ uint32_t lut_entry(const Tables<SH>& T, uint32_t ti, uint32_t f, uint32_t n, uint32_t w) {
-  const uint32_t b = T.base(ti);
-  const uint32_t e1 = T.lut_at(b, w >> (32 - kLutBits));
-  const uint32_t j = (w >> 16) - f;
-  const uint32_t e2 = T.lut2_at(b, min(j, (uint32_t)kLut2Size - 1u));
-  return (e1 & 31u) ? e1 : (j < n ? e2 : 0u);
+struct Chain {
+  uint32_t pos;      // bit position in the stream (of the symbol of e)
+  uint32_t e;        // its entry (kFresh: not read yet)
+  uint32_t k;        // k << kRunShift
+  uint32_t q, qend;  // table record of the data unit, the record past the last
+  uint32_t coef;     // shared offset of the data unit's coefficients
+};
+constexpr uint32_t kFresh = 0xFFFFFFFFu;
+
+// Byte offset in a table of the entry for window w (see HuffSet).
+template <bool CAP>
+__device__ __forceinline__ uint32_t table_index(uint32_t w, int d, int cap) {
+  const int t = (int)(w >> 16), i = (int)(w >> (32 - kLutBits));
+  return 2u * (uint32_t)(CAP ? max(__viaddmin_s32(t, d, cap), i) : __viaddmax_s32(t, d, i));
 }
 
-// Signed value of the sz bits after the l-bit code at the top of w (T.81 EXTEND).
-__device__ __forceinline__ int symbol_value(uint32_t w, uint32_t l, uint32_t sz) {
-  const uint32_t tw = w << l;
-  return (int)__funnelshift_l(tw, 0u, sz) + (int)(~((int)tw >> 31) & (int)(1u - (1u << sz)));
+// SH: the tables staged in shared memory; CAP: a set that needs its tables' caps.
+template <bool SH, bool CAP>
+__device__ __forceinline__ bool entropy_fast(Chain& ch, uint32_t st, uint32_t w0, uint32_t limit, const HuffSet* set) {
+  const char* gt = reinterpret_cast<const char*>(set);
+  auto entry = [&](uint32_t o) {
+    return SH ? (uint32_t)*reinterpret_cast<const uint16_t*>(smem + o)
+              : (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(gt + o));
+  };
+  auto rec = [&](uint32_t o) {
+    return SH ? *reinterpret_cast<const uint4*>(smem + o) : __ldg(reinterpret_cast<const uint4*>(gt + o));
+  };
+  uint32_t q = ch.q, coef = ch.coef, k = ch.k, e = ch.e;
+  const uint32_t qend = ch.qend;
+  // AC table, next first table; next first k << kRunShift, their caps
+  uint4 t = rec(q), c = rec(q + 16);
+  uint32_t p = 8 * st + (ch.pos - 32 * w0);  // in bits of shared memory (stages are 16-byte aligned)
+  uint32_t o = (p >> 3) & ~3u;
+  const uint32_t x0 = sm_u32(o), x1 = sm_u32(o + 4), x2 = sm_u32(o + 8);
+  uint32_t b0 = __funnelshift_l(x1, x0, p), b1 = __funnelshift_l(x2, x1, p);
+  if (e == kFresh) {
+    const uint4 t0 = rec(q + 32);
+    k = t0.z;
+    e = entry(t0.x + table_index<CAP>(b0, (int)t0.y, (int)t0.w));
+  }
+  uint32_t bad = 0;
+#pragma unroll 1
+  do {
+#pragma unroll
+    for (int i = 0; i < kSymbols; ++i) {
+      // the next symbol's read
+      const uint32_t kr = k + e;
+      const bool done = kr >= (63u << kRunShift);  // the run reaches slot 63
+      const uint32_t w = b0;
+      b0 = __funnelshift_l(b1, b0, e);
+      const uint32_t en = entry((done ? t.z : t.x) +
+                                table_index<CAP>(b0, (int)(done ? t.w : t.y), (int)(done ? c.z : c.y)));
+      p += e & 31u;
+      o = (p >> 3) & ~3u;
+      b1 = __funnelshift_l(sm_u32(o + 8), sm_u32(o + 4), p);
+      // the current one's value and place
+      const bool past = kr >= kPast, val = (e & kSizeMask) != 0;
+      store_if(val & !past, coef + (kr >> (kRunShift - 1)), symbol_value(w, e));
+      bad = val & past ? 1u : bad;
+      k = done ? c.x : (kr | ((1u << kRunShift) - 1u)) + 1u;
+      coef += done ? 128u : 0u;
+      q += done ? (uint32_t)sizeof(HuffSeq) : 0u;
+      if (SH)
+        load_if<CAP>(done, q, t, c);
+      else
+        load_if(done, gt + q, t, c);
+      e = en;
+    }
+  } while ((q != qend) & (bad == 0) & (p < limit));
+  ch.pos = p - 8 * st + 32 * w0;
+  ch.e = e;
+  ch.k = k;
+  ch.q = q;
+  ch.coef = coef;
+  return bad == 0;
 }
 
-// Window slot of symbol entry e read at w, window offset o, in a window of WIN bits (16-byte
-// slots). First word: byte offset in the window of the slot after the symbol, clamped to the
-// last slot (bits 0-11), run (12-17), value bits present (18), the next symbol starts past
-// the window (19), the next symbol's window offset (20-28); 0 for no symbol (an invalid
-// code), never 0 otherwise (the next offset is at least 1). Second word: the value.
-template <int WIN>
-__device__ __forceinline__ uint2 win_entry(uint32_t e, uint32_t w, uint32_t o) {
-  const uint32_t l = e & 31u, sz = (e >> 5) & 15u, r = e >> 9, nx = o + l + sz;
-  const uint32_t x = (min(nx, (uint32_t)WIN - 1u) * 16u) | (r << 12) | (sz ? 1u << 18 : 0u) |
-                     (nx >= (uint32_t)WIN ? 1u << 19 : 0u) | (nx << 20);
-  return e ? make_uint2(x, (uint32_t)symbol_value(w, l, sz)) : make_uint2(0u, 0u);
+// The general form of entropy_fast from global memory, and the last word on invalid codings:
+// `gw` are the stream's words from the MCU's first one on (ngw readable, zeros past them),
+// bit0 its first bit there. Returns the bit position after the last symbol, or kInvalid plus the
+// number of data units whose DC was reached (the coefficients decoded before the invalid
+// symbol stay). nl: luma data units (0 for a chroma unit of its own); cpt: the compact form.
+// Out of line: a rare path.
+__device__ __noinline__ uint32_t entropy_any(const uint32_t* gw, uint32_t ngw, uint32_t bit0, const HuffSet* set,
+                                             int ndu, int nl, bool cpt, uint32_t coef) {
+  for (int i = 0; i < 32 * ndu; ++i) *reinterpret_cast<uint32_t*>(smem + coef + 4 * i) = 0;
+  auto word = [&](uint32_t i) { return i < ngw ? bswap(__ldg(gw + i)) : 0u; };
+  uint32_t pos = bit0;
+  int du = 0, k = cpt ? 1 : 0;
+#pragma unroll 1
+  for (int it = 0; it < 64 * 6; ++it) {  // at most 64 symbols per data unit: each advances k
+    const HuffWalk* t = set->walk + (k == 0 ? 0 : 1) + (du < nl ? 0 : 2);
+    const uint32_t w = __funnelshift_l(word((pos >> 5) + 1), word(pos >> 5), pos & 31u);
+    const uint32_t x = (uint32_t)max(min((int)(w >> 16) + __ldg(&t->d), __ldg(&t->cap)), (int)(w >> (32 - kLutBits)));
+    uint32_t e = __ldg(reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(set) + __ldg(&t->base)) + x);
+    if (e == kNoEntry) e = walk_symbol(t, w, k == 0);
+    if (e == kNoEntry) return kInvalid + (uint32_t)(du + (k > 0 ? 1 : 0));
+    const bool val = (e & kSizeMask) != 0;
+    const int kst = k + (int)(e >> kRunShift);
+    if (val) sm_i16(coef + (uint32_t)(du * 128 + 2 * min(kst, 63))) = (int16_t)symbol_value(w, e);
+    if (val && kst > 63) return kInvalid + (uint32_t)(du + 1);
+    pos += e & 31u;
+    k = kst + 1;
+    if (kst >= 63) {
+      ++du;
+      if (du == ndu) return pos;
+      k = cpt && du >= nl ? 1 : 0;
+    }
+  }
+  return kInvalid + (uint32_t)ndu;  // (not reached)
 }
 
-__device__ __forceinline__ uint2 lds_u64(uint32_t saddr) {
-  uint2 v;
-  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(saddr));
-  return v;
-}
-__device__ __forceinline__ uint4 lds_u128(uint32_t saddr) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(saddr));
-  return v;
-}
+// ---- pixel phase ----
 
-// Stream words of a warp-decoded MCU that is staged whole (every word its symbols can reach
-// is in shared memory): reads need no bounds branch; an index past the stage (only an invalid
-// coding gets there) is clamped into the stage.
-struct StagedWords {
-  uint32_t st, last;  // shared address of the staged words, index of the last one
-  __device__ __forceinline__ uint32_t operator()(uint32_t i) const { return lds_u32(st + 4 * min(i, last)); }
+// An 8x8 transform pass of a data unit is one tensor-core product with exact results.
+//
+// D = K X with K the 14-bit integer matrix and X 16-bit integers. K is split as Kh 2^7 + Kl
+// (|Kh| <= 63, -64 <= Kl < 64), X as Xh 2^8 + Xl (Xh a signed, Xl an unsigned byte); every
+// part is exact in fp16, the products are exact, and the sums are exact in fp32. The 16 x 16
+// operand A holds Kh 2^7 in rows 0-7 and Kl in rows 8-15, columns 0-7 meeting Xh and columns
+// 8-15 (scaled by 2^-8) meeting Xl in the 16 x 8 operand B, so D's rows 0-7 are
+// (Kh 2^7) X 2^-8, multiples of 2^-1 below 2^23 in magnitude, and rows 8-15 are Kl X 2^-8,
+// multiples of 2^-8 below 2^16. A lane (g = lane / 4, t = lane % 4) gets both parts of the
+// elements (g, 2t) and (g, 2t + 1); the accumulators of the high parts start at the pass's
+// rounding constant. The parts' sum rounded down, scaled and rounded down again onto
+// 1.5 * 2^23 is the pass's floor (every threshold is representable), in the low mantissa bits.
+// The first product's output elements are the second one's B elements of the same lane, so
+// the row pass computes the transposed product K T^T and nothing moves between lanes.
+struct Frag {
+  uint32_t h0, l0, h1, l1;  // A: Kh 2^7, Kl, Kh 2^-1, Kl 2^-8, each the columns 2t, 2t + 1 of row g
 };
 
-// The 32 stream bits from bit position p on (relative to the first staged word).
-template <class WS>
-__device__ __forceinline__ uint32_t bits32w(const WS& W, uint32_t p) {
-  return __funnelshift_l(W((p >> 5) + 1), W(p >> 5), p & 31u);
+__device__ __forceinline__ uint32_t h2_bits(__half2 h) { return *reinterpret_cast<uint32_t*>(&h); }
+__device__ __forceinline__ __half2 bits_h2(uint32_t w) { return *reinterpret_cast<__half2*>(&w); }
+
+__device__ __forceinline__ Frag idct_frag(int r, int lane) {
+  const int g = lane >> 2, t = lane & 3;
+  const int ka = idct_k(g, 2 * t, r), kb = idct_k(g, 2 * t + 1, r);
+  const int ha = (ka + 64) >> 7, hb = (kb + 64) >> 7;
+  const float la = (float)(ka - ha * 128), lb = (float)(kb - hb * 128);
+  Frag f;
+  f.h0 = h2_bits(__floats2half2_rn(ha * 128.f, hb * 128.f));
+  f.l0 = h2_bits(__floats2half2_rn(la, lb));
+  f.h1 = h2_bits(__floats2half2_rn(ha * 0.5f, hb * 0.5f));
+  f.l1 = h2_bits(__floats2half2_rn(la * (1.f / 256), lb * (1.f / 256)));
+  return f;
 }
 
-// Entropy-decodes all data units of one MCU with the whole warp (every lane calls it with the
-// same arguments). Coefficients go to cc[du * 64 + k] (contiguous, zig-zag k; zero on entry);
-// tbl_sa is the 16-byte aligned shared address of WIN 16-byte slots of scratch. Slot o holds
-// the symbol starting at window offset o and, when it stays in the window, the symbol right
-// after it, so one read serves two symbols unless the first ends the data unit. Same
-// results and the same invalid codings as decode_mcu. Returns the bit position after the
-// MCU relative to the first staged word, or 0xFFFFFFFF on an invalid coding.
-template <bool SH, bool CPT, int WIN, class WS>
-__device__ __forceinline__ uint32_t decode_mcu_warp(const WS& W, uint32_t bit0, const Tables<SH>& T, int ndu,
-                                                    int p0, int p1, int p2, int16_t* cc, uint32_t tbl_sa,
-                                                    int lane) {
-  constexpr int J = WIN / 32;  // slots per lane
-  const uint32_t F0 = T.first16(0), F1 = T.first16(1), F2 = T.first16(2), F3 = T.first16(3);
-  const uint32_t N0 = T.n2(0), N1 = T.n2(1), N2 = T.n2(2), N3 = T.n2(3);
-  int pred0 = p0, pred1 = p1, pred2 = p2;
-  uint32_t pos = bit0, wb = 0;
-  int wcls = -1;  // component class of the window's entries (none yet)
-  bool bad = false;
-#pragma unroll 1
-  for (int du = 0; du < ndu && !bad; ++du) {
-    const int comp = du < ndu - 2 ? 0 : (du == ndu - 2 ? 1 : 2);
-    const int cls = comp ? 1 : 0;
-    const uint32_t tdc = cls ? 2u : 0u, tac = tdc | 1u;
-    const uint32_t fdc = cls ? F2 : F0, ndc = cls ? N2 : N0, fac = cls ? F3 : F1, nac = cls ? N3 : N1;
-    int16_t* cd = cc + du * 64;
-    int pv = comp == 0 ? pred0 : (comp == 1 ? pred1 : pred2);
-    if (!(CPT && (du == 0 || comp != 0))) {  // the compact form stores these DCs, no difference
-      const uint32_t w = bits32w(W, pos);
-      uint32_t e = lut_entry(T, tdc, fdc, ndc, w);
-      if (e == 0) e = walk_symbol(T.hs + tdc, w, true);
-      if (e == 0) {
-        bad = true;
-        break;
-      }
-      const uint32_t l = e & 31u, sz = (e >> 5) & 15u;
-      pv = (int16_t)(uint16_t)(pv + symbol_value(w, l, sz));  // DC values wrap modulo 2^16
-      pos += l + sz;
-    }
-    pred0 = comp == 0 ? pv : pred0;
-    pred1 = comp == 1 ? pv : pred1;
-    pred2 = comp == 2 ? pv : pred2;
-    // AC symbols: symbol s of the unit is kept by lane s % 32 as k << 16 | value (0: none)
-    uint32_t keep0 = 0, keep1 = 0;
-    int k = 1, s = 0, kst = 0;
-#pragma unroll 1
-    while (true) {
-      if (wcls != cls || pos - wb >= (uint32_t)WIN) {
-        // rebuild the window at pos: every lane's loads first, then its entries
-        __syncwarp();  // every lane has read the old window
-        wb = pos;
-        wcls = cls;
-        uint32_t w[J], e[J];
+constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
+
+// K X of the lane's B elements (rows 2t, 2t + 1 of column g) given as packed int16 plus 2^15,
+// plus bias, times 2^-8: the two parts of elements (g, 2t), (g, 2t + 1).
+__device__ __forceinline__ float4 idct_product(const Frag& f, uint32_t x, float bias) {
+  const uint32_t xl = h2_bits(__hsub2(bits_h2(__byte_perm(x, 0x64646464u, 0x4240)), bits_h2(0x64006400u)));
+  const uint32_t xh = h2_bits(__hsub2(bits_h2(__byte_perm(x, 0x64646464u, 0x4341)), bits_h2(0x64806480u)));
+  float4 c = make_float4(bias, bias, 0.f, 0.f);
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(c.x), "+f"(c.y), "+f"(c.z), "+f"(c.w)
+      : "r"(f.h0), "r"(f.l0), "r"(f.h1), "r"(f.l1), "r"(xh), "r"(xl));
+  return c;
+}
+
+// Row pass from the lane's column-pass results (row g, columns 2t, 2t + 1, packed int16 plus
+// 2^15): clamp(floor((sum + 2^18) / 2^19) + 128, 0, 255) of its pixels (rows 2t, 2t + 1,
+// column g) in the halves of a word. The saturating multiply clamps to [0, 256], the packed
+// minimum to 255.
+__device__ __forceinline__ uint32_t row_pass(const Frag& f, uint32_t t) {
+  const float4 c = idct_product(f, t, 1024.0f + 262144.0f);
+  const float a = __saturatef(__fadd_rd(c.x, c.z) * (1.0f / 524288)), b = __saturatef(__fadd_rd(c.y, c.w) * (1.0f / 524288));
+  const uint32_t p = __byte_perm(__float_as_uint(__fmaf_rd(a, 256.0f, kMagic)),
+                                 __float_as_uint(__fmaf_rd(b, 256.0f, kMagic)), 0x5410);
+  return __viaddmin_s16x2(p, 0u, 0x00FF00FFu);
+}
+
+__device__ __forceinline__ int sat16(int v) { return min(32767, max(-32768, v)); }
+
+// Column pass of any coefficients: t = clamp16(floor((sum + 2^8) / 2^9)) of d = clamp16(q Q);
+// q, Q: the lane's two coefficients and their steps.
+__device__ __forceinline__ uint32_t column_pass_any(const Frag& f, int qa, int qb, int Qa, int Qb) {
+  const uint32_t x = __byte_perm((uint32_t)(sat16(qa * Qa) + 32768), (uint32_t)(sat16(qb * Qb) + 32768), 0x5410);
+  const float4 c = idct_product(f, x, 1.0f);
+  const float a = fminf(fmaxf(__fadd_rd(c.x, c.z), -65536.0f), 65535.99609375f);
+  const float b = fminf(fmaxf(__fadd_rd(c.y, c.w), -65536.0f), 65535.99609375f);
+  return __byte_perm(__float_as_uint(__fmaf_rd(a, 0.5f, kMagic + 32768.0f)),
+                     __float_as_uint(__fmaf_rd(b, 0.5f, kMagic + 32768.0f)), 0x5410);
+}
+
+// Column pass of small dequantised coefficients, exact in fp16 as they are (one product of
+// depth 8, no split of X): |DC| <= kSmallDc, |AC| <= kSmallAc, so that |t| <=
+// (5793 * 1200 + 37491 * 256) / 2^9 < 2^15 needs no clamp and every sum stays below 2^24.
+constexpr float kSmallDc = 1200.0f, kSmallAc = 256.0f;
+__device__ __forceinline__ uint32_t column_pass_small(const Frag& f, __half2 x) {
+  float4 c = make_float4(256.0f, 256.0f, 0.f, 0.f);
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%0, %1, %2, %3};"
+      : "+f"(c.x), "+f"(c.y), "+f"(c.z), "+f"(c.w)
+      : "r"(f.h0), "r"(f.l0), "r"(h2_bits(x)));
+  return __byte_perm(__float_as_uint(__fmaf_rd(c.x + c.z, 1.0f / 512, kMagic + 32768.0f)),
+                     __float_as_uint(__fmaf_rd(c.y + c.w, 1.0f / 512, kMagic + 32768.0f)), 0x5410);
+}
+
+// What a lane needs of an MCU's quantisation tables: the steps of its two coefficients (luma,
+// chroma), as integers and as fp16 pairs.
+struct Steps {
+  int la, lb, ca, cb;
+  __half2 l, c;
+};
+
+// Pixels (rows 2t, 2t + 1, column g) of an MCU's NDU data units, coefficients at shared offset
+// coef. Data units go through the small form when all of the MCU's do: quantised values in
+// [-512, 511] (so that 1536 + q is exact in fp16 and its exponent field says so) and the
+// bounds of column_pass_small (a step above 2048 is infinite or inexact in fp16, and any
+// product with it then fails the bound; with q = 0 a finite step gives 0).
+template <int NDU>
+__device__ __forceinline__ void mcu_idct(const Frag& f, uint32_t coef, uint32_t oa, uint32_t ob, const Steps& Q,
+                                         __half2 bound, uint32_t (&p)[NDU]) {
+  __half2 x[NDU], worst = __float2half2_rn(0.f);
+  uint32_t odd = 0;
 #pragma unroll
-        for (int j = 0; j < J; ++j) w[j] = bits32w(W, wb + (uint32_t)(lane + 32 * j));
-        bool none = false;
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-          e[j] = lut_entry(T, tac, fac, nac, w[j]);
-          none |= e[j] == 0;
-        }
-        if (none) {  // codes without a LUT entry: the MAXCODE walk decodes or rejects them
-#pragma unroll
-          for (int j = 0; j < J; ++j)
-            if (e[j] == 0) e[j] = walk_symbol(T.hs + tac, w[j], false);
-        }
-        uint2 we[J];
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-          const uint32_t o = (uint32_t)(lane + 32 * j);
-          we[j] = win_entry<WIN>(e[j], w[j], o);
-          asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(tbl_sa + 16 * o), "r"(we[j].x), "r"(we[j].y));
-        }
-        __syncwarp();
-        // second halves: the symbol after each slot's symbol, when it starts in the window
-        uint2 nb[J];
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-          const bool in = we[j].x != 0 && (we[j].x & (1u << 19)) == 0;
-          nb[j] = lds_u64(tbl_sa + (we[j].x & 4095u));  // a slot in the window either way
-          nb[j] = in ? nb[j] : make_uint2(0u, 0u);
-        }
-#pragma unroll
-        for (int j = 0; j < J; ++j)
-          asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(tbl_sa + 16 * (uint32_t)(lane + 32 * j) + 8),
-                       "r"(nb[j].x), "r"(nb[j].y));
-        __syncwarp();
-      }
-      // symbols while the position stays in the window, one or two per read; the next
-      // slot's read goes out before this one is taken apart (a lone warp issues in order);
-      // a read past the window is clamped into it and dropped
-      uint4 ent = lds_u128(tbl_sa + 16 * (pos - wb));
-      uint32_t nofs = pos - wb;  // window offset of the next symbol
-      bool more;
-      do {
-        const int kstA = k + (int)((ent.x >> 12) & 63u);
-        const bool two = kstA < 63 && ent.z != 0;  // the second symbol belongs to this unit
-        const uint4 nxt = lds_u128(tbl_sa + ((two ? ent.z : ent.x) & 4095u));
-        const bool valA = (ent.x & (1u << 18)) != 0, valB = (ent.z & (1u << 18)) != 0;
-        const int kstB = kstA + 1 + (int)((ent.z >> 12) & 63u);
-        const uint32_t kvA = valA ? ((uint32_t)kstA << 16) | (ent.y & 0xFFFFu) : 0u;
-        const uint32_t kvB = (two && valB) ? ((uint32_t)kstB << 16) | (ent.w & 0xFFFFu) : 0u;
-        keep0 = s == lane ? kvA : (s + 1 == lane ? kvB : keep0);
-        keep1 = s == lane + 32 ? kvA : (s + 1 == lane + 32 ? kvB : keep1);
-        bad |= ent.x == 0 || (valA && kstA > 63) || (two && valB && kstB > 63);
-        kst = two ? kstB : kstA;
-        s += two ? 2 : 1;
-        k = kst + 1;
-        const uint32_t last = two ? ent.z : ent.x;
-        nofs = last >> 20;
-        more = kst < 63 && !bad && (last & (1u << 19)) == 0;
-        ent = nxt;
-      } while (more);
-      pos = wb + nofs;
-      if (kst >= 63 || bad) break;
-    }
-    if (lane == 0) cd[0] = (int16_t)pv;
-    if (keep0 != 0 && (keep0 >> 16) <= 63u) cd[keep0 >> 16] = (int16_t)(keep0 & 0xFFFFu);
-    if (keep1 != 0 && (keep1 >> 16) <= 63u) cd[keep1 >> 16] = (int16_t)(keep1 & 0xFFFFu);
+  for (int d = 0; d < NDU; ++d) {
+    const uint32_t q = __byte_perm((uint32_t)(uint16_t)sm_i16(coef + 128 * d + oa), (uint32_t)(uint16_t)sm_i16(coef + 128 * d + ob), 0x5410);
+    const uint32_t h = __viaddmax_s16x2(q, 0x66006600u, 0x80008000u);  // 1536 + q
+    odd |= h ^ 0x64006400u;
+    x[d] = __hmul2(__hsub2(bits_h2(h), bits_h2(0x66006600u)), d < NDU - 2 ? Q.l : Q.c);
+    worst = __hmax2_nan(worst, __habs2(x[d]));
   }
-  return bad ? 0xFFFFFFFFu : pos;
-}
-
-__device__ __forceinline__ uint32_t ycc_pixel(uint32_t Y, int ro, int go, int bo) {
-  return clamp255((int)Y + ro) | (clamp255((int)Y + go) << 8) | (clamp255((int)Y + bo) << 16) | 0xFF000000u;
-}
-
-__device__ __forceinline__ void chroma_offsets(uint32_t cb8, uint32_t cr8, int& ro, int& go, int& bo) {
-  const int cb = (int)cb8 - 128, cr = (int)cr8 - 128;
-  ro = (91881 * cr + 32768) >> 16;
-  go = (-22554 * cb - 46802 * cr + 32768) >> 16;
-  bo = (116130 * cb + 32768) >> 16;
-}
-
-
-// Pixels after the row pass, in place: the row pass of data unit d, row y has just read
-// the 8 slots zz_pos(y, 0..7) (no other row reads them) and writes pixels x = 2i, 2i+1 as the
-// low and high byte of slot zz_pos(y, i), i < 4. pixel2(d, y, i) reads that pair.
-template <int M>
-__device__ __forceinline__ uint32_t pixel2(const int16_t* col, int d, int y, int i) {
-  return (uint16_t)col[(d * 64 + zz_pos(y, i)) * M];
-}
-
-// Reduced-resolution IDCT of one data unit (N = 8 >> R) in place over the buffer: the same
-// dequantisation and rounding as the full transform on the N x N lowest frequencies; the
-// row pass leaves pixel pairs (x = 2i, 2i+1) in slots zz_pos(y, i), i < N/2 (N = 1: the
-// pixel in the low byte of slot 0), which pixel2() reads as for the full size.
-template <int M, int R>
-__device__ __forceinline__ void idct_reduced(int16_t* blk, const uint16_t* Qd) {
-  constexpr int N = 8 >> R;
+  const bool small = (odd & 0xFC00FC00u) == 0 && __hble2(worst, bound);
+  if (__all_sync(0xFFFFFFFFu, small)) {
 #pragma unroll
-  for (int u = 0; u < N; ++u) {
-    int in[4] = {0, 0, 0, 0}, out[4];
+    for (int d = 0; d < NDU; ++d) p[d] = row_pass(f, column_pass_small(f, x[d]));
+  } else {
 #pragma unroll
-    for (int v = 0; v < N; ++v) {
-      const int k = zz_pos(v, u);
-      in[v] = sat16(blk[k * M] * (int)__ldg(Qd + k));
-    }
-    idct_small<N>(in, out);
-#pragma unroll
-    for (int y = 0; y < N; ++y) blk[zz_pos(y, u) * M] = (int16_t)sat16((out[y] + 256) >> 9);
-  }
-#pragma unroll
-  for (int y = 0; y < N; ++y) {
-    int in[4] = {0, 0, 0, 0}, out[4];
-#pragma unroll
-    for (int x = 0; x < N; ++x) in[x] = blk[zz_pos(y, x) * M];
-    idct_small<N>(in, out);
-    if (N == 1) {
-      blk[zz_pos(y, 0) * M] = (int16_t)clamp255(((out[0] + (1 << 18)) >> 19) + 128);
-    } else {
-#pragma unroll
-      for (int i = 0; i < N / 2; ++i)
-        blk[zz_pos(y, i) * M] = (int16_t)(clamp255(((out[2 * i] + (1 << 18)) >> 19) + 128) |
-                                          (clamp255(((out[2 * i + 1] + (1 << 18)) >> 19) + 128) << 8));
-    }
+    for (int d = 0; d < NDU; ++d)
+      p[d] = row_pass(f, column_pass_any(f, sm_i16(coef + 128 * d + oa), sm_i16(coef + 128 * d + ob),
+                                         d < NDU - 2 ? Q.la : Q.ca, d < NDU - 2 ? Q.lb : Q.cb));
   }
 }
 
-// Colour conversion of a reduced tile ((mw >> r)^2 texels, mw = 16 at 4:2:0, 8 at 4:4:4),
-// chroma replicated 2x2 at 4:2:0 as at full size; one 4-byte store per texel.
-template <int M>
-__device__ __noinline__ void colour_reduced(const int16_t* col, bool s420, int red, uint32_t* tile) {
-  const int n = 8 >> red, tw = (s420 ? 16 : 8) >> red;
-  auto pix = [&](int d, int y, int x) { return (pixel2<M>(col, d, y, x >> 1) >> (8 * (x & 1))) & 255u; };
-#pragma unroll 1
-  for (int ty = 0; ty < tw; ++ty)
-#pragma unroll 1
-    for (int tx = 0; tx < tw; ++tx) {
-      uint32_t Y, cb, cr;
-      if (s420) {
-        Y = pix((ty / n) * 2 + tx / n, ty % n, tx % n);
-        cb = pix(4, ty >> 1, tx >> 1);
-        cr = pix(5, ty >> 1, tx >> 1);
-      } else {
-        Y = pix(0, ty, tx);
-        cb = pix(1, ty, tx);
-        cr = pix(2, ty, tx);
-      }
-      int ro, go, bo;
-      chroma_offsets(cb, cr, ro, go, bo);
-      tile[ty * tw + tx] = ycc_pixel(Y, ro, go, bo);
-    }
+// RGBA8 of two texels: luma and offsets in the halves of y, ro, go, bo.
+__device__ __forceinline__ uint2 texel_pair(uint32_t y, uint32_t ro, uint32_t go, uint32_t bo) {
+  const uint32_t m = 0x00FF00FFu;
+  const uint32_t r = __viaddmin_s16x2_relu(y, ro, m), g = __viaddmin_s16x2_relu(y, go, m),
+                 b = __viaddmin_s16x2_relu(y, bo, m);
+  const uint32_t rg = __byte_perm(r, g, 0x6240), ba = __byte_perm(b, 0xFFFFFFFFu, 0x4240);
+  return make_uint2(__byte_perm(rg, ba, 0x5410), __byte_perm(rg, ba, 0x7632));
 }
 
-// Full-size IDCT of one data unit in place over the buffer: column pass with dequantisation
-// on load, t = clamp16(floor((sum_v K[y][v] clamp16(q Q) + 2^8) / 2^9)), then the row pass
-// p = clamp(floor((sum_u K[x][u] t[y][u] + 2^18) / 2^19) + 128, 0, 255), whose pixel pairs
-// land in the slots the row just read (see pixel2).
-template <int M>
-__device__ __forceinline__ void idct_full(int16_t* blk, const uint16_t* Qd) {
-#pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    int in[8], out[8];
-#pragma unroll
-    for (int v = 0; v < 8; ++v) {
-      const int k = zz_pos(v, u);
-      in[v] = sat16(blk[k * M] * (int)__ldg(Qd + k));
-    }
-    idct8(in, out);
-#pragma unroll
-    for (int y = 0; y < 8; ++y) blk[zz_pos(y, u) * M] = (int16_t)sat16((out[y] + 256) >> 9);
-  }
-#pragma unroll
-  for (int y = 0; y < 8; ++y) {
-    int in[8], out[8];
-#pragma unroll
-    for (int x = 0; x < 8; ++x) in[x] = blk[zz_pos(y, x) * M];
-    idct8(in, out);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      blk[zz_pos(y, i) * M] = (int16_t)(clamp255(((out[2 * i] + (1 << 18)) >> 19) + 128) |
-                                        (clamp255(((out[2 * i + 1] + (1 << 18)) >> 19) + 128) << 8));
-  }
+// (R, G, B) offsets of one chroma pair times 2^16 (JFIF in 16-bit fixed point; the upper half
+// of each word is the offset).
+__device__ __forceinline__ void chroma_offsets(int cb, int cr, uint32_t& r, uint32_t& g, uint32_t& b) {
+  r = (uint32_t)(91881 * cr + (32768 - 91881 * 128));
+  g = (uint32_t)(-22554 * cb - 46802 * cr + (32768 + (22554 + 46802) * 128));
+  b = (uint32_t)(116130 * cb + (32768 - 116130 * 128));
 }
 
-// IDCT and colour of one full-size MCU held by a whole warp (after decode_mcu_warp): the
-// column passes are shared out over the lanes as (data unit, column) pairs, the row passes as
-// (data unit, row) pairs, the tile as half rows of texels; same arithmetic as idct_full and
-// the per-MCU colour stores. cc: quantised coefficients [ndu][64] in zig-zag order; tmp
-// (16-byte aligned, [ndu][64] int16) and pix ([ndu][64] bytes) are scratch in natural order;
-// Q: the MCU's quantisation tables (luma, then chroma, zig-zag order); tile: its cache block.
-__device__ __forceinline__ void mcu_warp_pixels(const int16_t* cc, int16_t* tmp, uint8_t* pix, int ndu, bool s420,
-                                                const uint16_t* Q, uint8_t* tile, int lane) {
-  const int nluma = s420 ? 4 : 1;
-#pragma unroll 1
-  for (int q = lane; q < 8 * ndu; q += 32) {  // column u of data unit d, dequantised on load
-    const int d = q >> 3, u = q & 7;
-    const uint16_t* Qd = Q + (d < nluma ? 0 : 64);
-    int in[8], out[8];
+// IDCT, colour and tile of one MCU by the whole warp. coef: shared offset of its
+// coefficients; tile: its cache block, (mw >> r)^2 texels. RED: a reduced level, only pixels
+// below N = 8 >> r of each data unit exist.
+template <bool S420, bool RED>
+__device__ __forceinline__ void mcu_pixels(const Frag& f, uint32_t coef, uint32_t oa, uint32_t ob, const Steps& Q,
+                                           __half2 bound, int r, uint32_t* tile, int lane) {
+  const int g = lane >> 2, t = lane & 3;
+  const int n = RED ? 8 >> r : 8;
+  const bool in0 = !RED || (g < n && 2 * t < n), in1 = !RED || (g < n && 2 * t + 1 < n);
+  if (S420) {
+    uint32_t p[6];
+    mcu_idct<6>(f, coef, oa, ob, Q, bound, p);
+    const uint32_t cc = __byte_perm(p[4], p[5], 0x6420);  // Cb of rows 2t and 2t + 1, then Cr
 #pragma unroll
-    for (int v = 0; v < 8; ++v) {
-      const int k = zz_pos(v, u);
-      in[v] = sat16(cc[d * 64 + k] * (int)__ldg(Qd + k));
+    for (int d = 0; d < 4; ++d) {
+      // texels (di n + 2t + e, dj n + g) use chroma sample (row, col) = half of that
+      const int di = d >> 1, dj = d & 1;
+      const int row = (di * n >> 1) + t, col = (dj * n >> 1) + (g >> 1);
+      const uint32_t w = __shfl_sync(0xFFFFFFFFu, cc, (col * 4 + (row >> 1)) & 31);
+      const uint32_t sel = 0x4440u + (uint32_t)(row & 1);
+      uint32_t ro, go, bo;
+      chroma_offsets((int)__byte_perm(w, 0, sel), (int)__byte_perm(w, 0, sel + 2), ro, go, bo);
+      const uint2 px = texel_pair(p[d], __byte_perm(ro, 0, 0x3232), __byte_perm(go, 0, 0x3232), __byte_perm(bo, 0, 0x3232));
+      uint32_t* o = tile + (di * n + 2 * t) * (2 * n) + dj * n + g;
+      if (in0) o[0] = px.x;
+      if (in1) o[2 * n] = px.y;
     }
-    idct8(in, out);
-#pragma unroll
-    for (int v = 0; v < 8; ++v) tmp[d * 64 + v * 8 + u] = (int16_t)sat16((out[v] + 256) >> 9);
-  }
-  __syncwarp();
-#pragma unroll 1
-  for (int q = lane; q < 8 * ndu; q += 32) {  // row y of data unit d
-    const int d = q >> 3, y = q & 7;
-    const uint4 r = *reinterpret_cast<const uint4*>(tmp + d * 64 + y * 8);
-    const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
-    int in[8], out[8];
-#pragma unroll
-    for (int x = 0; x < 8; ++x) in[x] = (int16_t)(uint16_t)(rw[x >> 1] >> (16 * (x & 1)));
-    idct8(in, out);
-    uint32_t lo = 0, hi = 0;
-#pragma unroll
-    for (int x = 0; x < 4; ++x) {
-      lo |= clamp255(((out[x] + (1 << 18)) >> 19) + 128) << (8 * x);
-      hi |= clamp255(((out[x + 4] + (1 << 18)) >> 19) + 128) << (8 * x);
-    }
-    *reinterpret_cast<uint2*>(pix + d * 64 + y * 8) = make_uint2(lo, hi);
-  }
-  __syncwarp();
-  if (s420) {  // 16 x 16 texels: lane = (row ty, half h), texels x = 8h .. 8h + 7
-    const int ty = lane >> 1, h = lane & 1;
-    const uint2 yv = *reinterpret_cast<const uint2*>(pix + ((ty >> 3) * 2 + h) * 64 + (ty & 7) * 8);
-    const uint32_t cbv = *reinterpret_cast<const uint32_t*>(pix + 4 * 64 + (ty >> 1) * 8 + 4 * h);
-    const uint32_t crv = *reinterpret_cast<const uint32_t*>(pix + 5 * 64 + (ty >> 1) * 8 + 4 * h);
-    uint32_t o[8];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {  // chroma sample c covers texels 2c, 2c + 1
-      int ro, go, bo;
-      chroma_offsets((cbv >> (8 * c)) & 255u, (crv >> (8 * c)) & 255u, ro, go, bo);
-      const uint32_t yw = c < 2 ? yv.x : yv.y;
-      o[2 * c] = ycc_pixel((yw >> (16 * (c & 1))) & 255u, ro, go, bo);
-      o[2 * c + 1] = ycc_pixel((yw >> (16 * (c & 1) + 8)) & 255u, ro, go, bo);
-    }
-    uint4* dst = reinterpret_cast<uint4*>(tile + (ty * 16 + 8 * h) * 4);
-    dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-    dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
-  } else {  // 8 x 8 texels, Y Cb Cr data units 0 1 2: lane = (row ty, texels x0, x0 + 1)
-    const int ty = lane >> 2, x0 = (lane & 3) * 2;
-    uint32_t o[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int i = ty * 8 + x0 + e;
-      int ro, go, bo;
-      chroma_offsets(pix[64 + i], pix[128 + i], ro, go, bo);
-      o[e] = ycc_pixel(pix[i], ro, go, bo);
-    }
-    *reinterpret_cast<uint2*>(tile + (ty * 8 + x0) * 4) = make_uint2(o[0], o[1]);
+  } else {
+    uint32_t p[3];
+    mcu_idct<3>(f, coef, oa, ob, Q, bound, p);
+    uint32_t r0, g0, b0, r1, g1, b1;
+    chroma_offsets((int)(p[1] & 255u), (int)(p[2] & 255u), r0, g0, b0);
+    chroma_offsets((int)(p[1] >> 16), (int)(p[2] >> 16), r1, g1, b1);
+    const uint2 px = texel_pair(p[0], __byte_perm(r0, r1, 0x7632), __byte_perm(g0, g1, 0x7632), __byte_perm(b0, b1, 0x7632));
+    uint32_t* o = tile + 2 * t * n + g;
+    if (in0) o[0] = px.x;
+    if (in1) o[n] = px.y;
   }
 }
 
 // UNITS: the variant for contexts with data-unit starts. Each MCU of a batch then takes six
 // lanes, lane 6m + d decoding data unit d of MCU m from its own start (levels without
 // starts are decoded whole by lane 6m); MCUs per batch are at most 4.
-// SHORT: the variant that decodes short lists MCU by MCU with whole warps (a separate kernel,
-// so that the lane-per-MCU variant is compiled without that code).
-template <int M, bool UNITS, bool SHORT>
-__global__ void k_decode(const __grid_constant__ DecodeArgs a) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  HuffSet* sh = reinterpret_cast<HuffSet*>(smem);
+template <bool UNITS>
+__global__ void __launch_bounds__(512, 1) k_decode(const __grid_constant__ DecodeArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint8_t* wbase = smem + sizeof(HuffSet) + 64 + (size_t)warp * warp_smem(M);
-  int16_t* coef = reinterpret_cast<int16_t*>(wbase);                    // [6][64][M]
-  uint32_t* stage = reinterpret_cast<uint32_t*>(wbase + 6 * 64 * M * 2);  // [M * kStageWords]
+  const int M = a.mcus_per_warp;
+  const uint32_t coef0 = kStagedTables + (uint32_t)warp * (uint32_t)warp_smem(M);
+  const uint32_t stage0 = coef0 + (uint32_t)(M * kMcuBytes);
   // this lane's MCU slot and data unit (the whole MCU outside the unit variant)
   const int lm = UNITS ? lane / 6 : lane, ld = UNITS ? lane % 6 : 0;
-  int16_t* col = coef + (lm < M ? lm : 0);  // this lane's MCU column
-  constexpr int kMaxBatch = UNITS ? (M < 4 ? M : 4) : M;
+  const uint32_t mine = coef0 + (uint32_t)((lm < M ? lm : 0) * kMcuBytes);
+  const int max_batch = UNITS ? min(M, 4) : M;
 
-  {  // stage Huffman set 0 (written at upload, so before the wait for the kernel before)
-    const uint4* src = reinterpret_cast<const uint4*>(a.huff);
-    uint4* dst = reinterpret_cast<uint4*>(sh);
-    for (int i = threadIdx.x; i < (int)(sizeof(HuffSet) / 16); i += blockDim.x) dst[i] = __ldg(src + i);
-  }
+  // stages set i of the Huffman tables when it fits; kNoSet when it does not
+  auto stage_set = [&](uint32_t i) {
+    const uint32_t used = __ldg(&a.huff[i].used);
+    if (used > kStagedTables) return kNoSet;
+    for (uint32_t j = threadIdx.x; j < (used + 15) / 16; j += blockDim.x)
+      reinterpret_cast<uint4*>(smem)[j] = __ldg(reinterpret_cast<const uint4*>(a.huff + i) + j);
+    return i;
+  };
+  // a context's only set is staged before the wait for the kernel before (it was written at
+  // upload)
+  uint32_t staged = a.nsets == 1 ? stage_set(0) : kNoSet;
+  // the lane's two coefficients of a data unit and its transform fragments
+  const int fg = lane >> 2, ft = lane & 3;
+  const uint32_t oa = 2 * (uint32_t)zz_pos(2 * ft, fg), ob = 2 * (uint32_t)zz_pos(2 * ft + 1, fg);
+  const Frag f8 = idct_frag(0, lane);
+  const __half2 bound = __floats2half2_rn(lane == 0 ? kSmallDc : kSmallAc, kSmallAc);
   __syncthreads();
   pdl_wait();  // the work list, slots and counts come from the compaction or the cache update
 
   const uint32_t count = min(*(volatile uint32_t*)&a.state->count, a.work_cap);
   bool any_bad = false;
-  // MCUs per batch: the smallest power of two <= M that covers the list in one batch per
-  // warp, so short lists spread one MCU per warp (latency) and long ones fill the lanes
-  const uint32_t total_warps = gridDim.x * (blockDim.x >> 5);
-  const uint32_t per_warp = (count + total_warps - 1) / total_warps;
-  // (up to kWarpMcuMax MCUs per warp they go one at a time, each decoded by the whole warp:
-  // a lone lane's chain is several times longer than the warp's)
-  int lmeff = 0;
-  if (!SHORT || M < 4 || per_warp > (uint32_t)kWarpMcuMax)
-    while ((1u << lmeff) < per_warp && (1 << lmeff) < kMaxBatch) ++lmeff;
-  const int meff = 1 << lmeff;
-  // first batch by rank, interleaved over the CTAs (one warp per SM first), then dynamic
-  const uint32_t wrank = (uint32_t)warp * gridDim.x + blockIdx.x;
+  // MCUs per batch: the smallest power of two <= M that covers the list in one batch for each
+  // of kBusyWarps warps of a CTA: short lists spread one MCU per warp (latency), long ones fill
+  // the lanes, and between them few warps with more lanes beat more warps (their chains share
+  // the issue slots): 27 MCUs per SM took 59.5 us a frame with 7 warps of 4 against 61.2 with 14 of 2.
+  // The first batches are fixed: dealt warp by warp over the CTAs, so that neighbours (alike in
+  // length) fall on different SMs, or, with several sets of Huffman tables, in runs of
+  // neighbours, so that a CTA's MCUs mostly share a texture and with it the staged set. What
+  // they leave of a long list is handed out by a counter.
+  const uint32_t warps = blockDim.x >> 5, run = (count + gridDim.x - 1) / gridDim.x;
+  const uint32_t busy = min(warps, kBusyWarps), per_warp = (run + busy - 1) / busy;
+  int meff = 1;
+  while ((uint32_t)meff < per_warp && meff < max_batch) meff *= 2;
+  const bool runs = a.nsets > 1;
+  const uint32_t span = runs ? min(run, warps * (uint32_t)meff) : warps * (uint32_t)meff;
+  const uint32_t first = blockIdx.x * span;
+  if (runs) {  // stage the set of the CTA's first MCU
+    uint32_t i = kNoSet;
+    if (first < count) {
+      const uint32_t d = __ldg(a.desc_of_gid + __ldg(a.work + first));
+      if (d < a.ndesc) i = a.descs[d].hset;
+    }
+    if (i != kNoSet) staged = stage_set(i);
+    __syncthreads();
+  }
+  const bool staged_cap = staged != kNoSet && __ldg(&a.huff[staged].capped) != 0;
 
 #pragma unroll 1
   for (uint32_t it = 0;; ++it) {
-    uint32_t base = wrank * (uint32_t)meff;
+    uint32_t base = runs ? first + (uint32_t)(warp * meff) : ((uint32_t)warp * gridDim.x + blockIdx.x) * (uint32_t)meff;
+    uint32_t limit = runs ? min(first + span, count) : count;
     if (it != 0) {
+      if (run <= span) break;  // the first batches covered the list
       uint32_t b = 0;
       if (lane == 0) b = atomicAdd(&a.state->decode_next, (uint32_t)meff);
-      base = __shfl_sync(0xFFFFFFFFu, b, 0) + total_warps * (uint32_t)meff;
+      base = __shfl_sync(0xFFFFFFFFu, b, 0) + gridDim.x * span;
+      limit = count;
     }
-    if (base >= count) break;
+    if (base >= limit) break;
 
-    {  // clear the coefficient buffer (768 M bytes; a warp-decoded MCU needs only its
-       // contiguous 768 B: every other byte it reads is written first)
-      uint4* z = reinterpret_cast<uint4*>(coef);
-      const int nz = (SHORT && M >= 4 && meff == 1) ? 48 : 48 * M;
+    {  // clear the batch's coefficients
+      uint4* z = reinterpret_cast<uint4*>(smem + coef0);
+      const int nz = (meff * kMcuBytes + 15) / 16;
 #pragma unroll 4
       for (int i = lane; i < nz; i += 32) z[i] = make_uint4(0, 0, 0, 0);
     }
 
     // ---- set-up: lanes of MCU slot m < m_eff take item base + m ----
     const uint32_t item = base + lm;
-    bool act = lm < meff && item < count;
+    bool act = lm < meff && item < limit;
     bool unit = false;  // this lane decodes data unit ld only
     const uint32_t gid = act ? __ldg(a.work + item) : 0u;
     const uint32_t di = act ? __ldg(a.desc_of_gid + gid) : 0u;
     int ndu = 0;
     bool s420 = true, store = false;
-    uint32_t off = 0, nbits = 0, bitpos = 0, endbit = 0, w0 = 0, want = 0, nwords = 0;
+    uint32_t off = 0, nbits = 0, bitpos = 0, endbit = 0, nwords = 0;
     bool cpt = false;
     int red = 0;  // reduced-resolution level: 1/2^red
     const uint32_t* words = nullptr;
-    uint32_t qs = 0;  // the MCU's quantisation table set (zig-zag order, read through L1)
+    uint32_t qs = 0;  // the MCU's quantisation table set
     int16_t pr0 = 0, pr1 = 0, pr2 = 0;
-    const HuffTable* hs = sh->t;
+    const HuffSet* hs = a.huff;
+    bool staged_set = false;  // its Huffman tables are the staged ones
     if (act && di < a.ndesc) {
       const DevDesc d = a.descs[di];
       const uint32_t mcu = gid - d.gid_base;
@@ -847,233 +622,142 @@ __global__ void k_decode(const __grid_constant__ DecodeArgs a) {
         words = d.stream;
         nwords = d.nwords;
         nbits = d.nbits;
-        // the MCU's words: from its first word (16 B aligned) to the next MCU's start plus
-        // the window's look-ahead (3 words)
-        w0 = (bitpos >> 5) & ~3u;
-        want = (max(endbit, bitpos) >> 5) + 3 - w0;
-        want = (want + 3) & ~3u;
-        if (w0 + want > nwords) want = nwords > w0 ? (nwords - w0) & ~3u : 0u;
-        if (d.hset != 0) hs = a.huff[d.hset].t;
+        hs = a.huff + d.hset;
+        staged_set = d.hset == staged;
         qs = d.qset;
       }
     } else {
       act = false;
     }
-    if (!act) want = 0;
-    // share the warp's stage pool out by a prefix sum of the lanes' word counts
-    uint32_t sbeg = want;
-#pragma unroll
-    for (int dlt = 1; dlt < 32; dlt <<= 1) {
-      const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, sbeg, dlt);
-      if (lane >= dlt) sbeg += o;
-    }
-    sbeg -= want;  // exclusive
-    constexpr uint32_t kPool = (uint32_t)kStageWords * M;
-    const uint32_t nst = sbeg >= kPool ? 0u : min(want, kPool - sbeg);
-    if (act) {
-      const uint4* src4 = reinterpret_cast<const uint4*>(words + w0);
-      uint4* dst4 = reinterpret_cast<uint4*>(stage + sbeg);
-#pragma unroll 1
-      for (uint32_t j = 0; j < nst / 4; j += 4) {
-        uint4 r[4];
-#pragma unroll
-        for (int t = 0; t < 4; ++t) r[t] = j + t < nst / 4 ? __ldg(src4 + j + t) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-        for (int t = 0; t < 4; ++t)
-          if (j + t < nst / 4) dst4[j + t] = make_uint4(bswap(r[t].x), bswap(r[t].y), bswap(r[t].z), bswap(r[t].w));
-      }
-    }
-    __syncwarp();
-
     // ---- entropy phase: each active lane decodes all data units of its MCU (or, with
-    // data-unit starts, one data unit) ----
-    if (act && unit) {
-      const Words W{(uint32_t)__cvta_generic_to_shared(stage + sbeg), nst, words + w0,
-                    nwords > w0 ? nwords - w0 : 0u};
-      const int comp = ld < ndu - 2 ? 0 : 1;
-      const uint32_t b0 = bitpos - w0 * 32;
-      int16_t* cu = col + ld * 64 * M;
-      const uint32_t end = hs == sh->t
-                               ? decode_unit<M, true>(W, b0, Tables<true>{hs, (uint32_t)__cvta_generic_to_shared(sh->t)},
-                                                      comp, cu)
-                               : decode_unit<M, false>(W, b0, Tables<false>{hs, 0u}, comp, cu);
-      // a data unit must end at or before the next one's start
-      if (end == 0xFFFFFFFFu || (uint64_t)w0 * 32 + end > endbit) any_bad = true;
+    // data-unit starts, one data unit), in rounds of staging and decoding (one round unless
+    // the batch's words exceed the pool) ----
+    int nd = ndu, nl = ndu - 2, seq = s420 ? (cpt ? kSeqCompact420 : kSeq420) : (cpt ? kSeqCompact444 : kSeq444);
+    uint32_t dst = mine;
+    if (UNITS && unit) {
+      nl = ld < nl ? 1 : 0;
+      nd = 1;
+      seq = nl ? kSeqLuma : kSeqChroma;
+      dst += 128 * (uint32_t)ld;
     }
-    bool warp_done = false;  // the MCU's tile was written by the whole warp
-    if (SHORT && !UNITS && M >= 4 && meff == 1) {
-      // one MCU per warp: the whole warp runs lane 0's chain (coefficients contiguous in
-      // the buffer's first 768 B, the window's slots after them); a full-size tile
-      // is then transformed and stored by the whole warp, any other is scattered into lane
-      // 0's column for the per-lane passes
-      if (__shfl_sync(0xFFFFFFFFu, act ? 1 : 0, 0)) {
-        const Words W{(uint32_t)__cvta_generic_to_shared(stage), __shfl_sync(0xFFFFFFFFu, nst, 0),
-                      reinterpret_cast<const uint32_t*>(
-                          __shfl_sync(0xFFFFFFFFu, reinterpret_cast<unsigned long long>(words + w0), 0)),
-                      __shfl_sync(0xFFFFFFFFu, nwords > w0 ? nwords - w0 : 0u, 0)};
-        const HuffTable* hw = reinterpret_cast<const HuffTable*>(
-            __shfl_sync(0xFFFFFFFFu, reinterpret_cast<unsigned long long>(hs), 0));
-        const uint32_t b0 = __shfl_sync(0xFFFFFFFFu, bitpos - w0 * 32, 0);
-        const int nd = __shfl_sync(0xFFFFFFFFu, ndu, 0);
-        const bool cw = __shfl_sync(0xFFFFFFFFu, cpt ? 1 : 0, 0) != 0;
-        const int q0 = __shfl_sync(0xFFFFFFFFu, (int)pr0, 0), q1 = __shfl_sync(0xFFFFFFFFu, (int)pr1, 0),
-                  q2 = __shfl_sync(0xFFFFFFFFu, (int)pr2, 0);
-        const uint32_t tsa = (uint32_t)__cvta_generic_to_shared(coef) + 768u;
-        constexpr int kWin = M >= 8 ? kWinBits : kWinBits / 2;  // 16 B slots after the 768 B of coefficients
-        static_assert(768 + 16 * kWin <= 768 * M || M < 4, "window slots fit the coefficient buffer");
-        const Tables<true> TS{hw, (uint32_t)__cvta_generic_to_shared(sh->t)};
-        const Tables<false> TG{hw, 0u};
-        // staged whole: every word up to the next MCU's start plus the look-ahead
-        const uint32_t nst0 = __shfl_sync(0xFFFFFFFFu, nst, 0);
-        const bool whole = nst0 > 0 && nst0 >= __shfl_sync(0xFFFFFFFFu, want, 0);
-        const StagedWords SW{W.st, nst0 - 1};
-        uint32_t end;
-        if (whole && hw == sh->t)
-          end = cw ? decode_mcu_warp<true, true, kWin>(SW, b0, TS, nd, q0, q1, q2, coef, tsa, lane)
-                   : decode_mcu_warp<true, false, kWin>(SW, b0, TS, nd, q0, q1, q2, coef, tsa, lane);
-        else if (whole)
-          end = cw ? decode_mcu_warp<false, true, kWin>(SW, b0, TG, nd, q0, q1, q2, coef, tsa, lane)
-                   : decode_mcu_warp<false, false, kWin>(SW, b0, TG, nd, q0, q1, q2, coef, tsa, lane);
-        else if (hw == sh->t)
-          end = cw ? decode_mcu_warp<true, true, kWin>(W, b0, TS, nd, q0, q1, q2, coef, tsa, lane)
-                   : decode_mcu_warp<true, false, kWin>(W, b0, TS, nd, q0, q1, q2, coef, tsa, lane);
-        else
-          end = cw ? decode_mcu_warp<false, true, kWin>(W, b0, TG, nd, q0, q1, q2, coef, tsa, lane)
-                   : decode_mcu_warp<false, false, kWin>(W, b0, TG, nd, q0, q1, q2, coef, tsa, lane);
-        if (lane == 0 && (end == 0xFFFFFFFFu || (uint64_t)w0 * 32 + end > (cpt ? endbit : nbits))) any_bad = true;
-        __syncwarp();
-        if (__shfl_sync(0xFFFFFFFFu, (red == 0 && store) ? 1 : 0, 0)) {
-          const bool s4 = __shfl_sync(0xFFFFFFFFu, s420 ? 1 : 0, 0) != 0;
-          const uint32_t qs0 = __shfl_sync(0xFFFFFFFFu, qs, 0), off0 = __shfl_sync(0xFFFFFFFFu, off, 0);
-          mcu_warp_pixels(coef, coef + 384, reinterpret_cast<uint8_t*>(coef) + 1536, nd, s4,
-                          a.quant + (size_t)qs0 * 128, a.cache + (size_t)off0 * kUnitBytes, lane);
-          warp_done = true;
-        } else {
-          int16_t v[12];
+    Chain ch{bitpos, kFresh, 0u, (uint32_t)(seq * sizeof(HuffSeq)), (uint32_t)((seq + nd) * sizeof(HuffSeq)), dst};
+    int reached = ndu;  // data units whose DC difference was decoded
+    bool more = act;
+    const uint32_t pool = (uint32_t)(kStageWords * M);
+#pragma unroll 1
+    do {
+      // the chain's words: from its next one (16 B aligned) to the next MCU's start plus the
+      // window's look-ahead (3 words)
+      const uint32_t w0 = (ch.pos >> 5) & ~3u;
+      uint32_t all = (max(endbit, ch.pos) >> 5) + 3 - w0;
+      all = (all + 3) & ~3u;
+      if (w0 + all > nwords) all = nwords > w0 ? (nwords - w0) & ~3u : 0u;
+      if (!more) all = 0;
+      // share the warp's stage pool out by a prefix sum of the lanes' word counts, in equal
+      // shares when they exceed it (at least 12 words: a group of symbols from any bit of the
+      // first four ends inside them, so the first unfinished chain always advances)
+      uint32_t want = all;
+      if (__reduce_add_sync(0xFFFFFFFFu, all) > pool)
+        want = min(all, max(pool / (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, all != 0)) & ~3u, 12u));
+      uint32_t sbeg = want;
 #pragma unroll
-          for (int i = 0; i < 12; ++i) v[i] = coef[lane + 32 * i];
-          __syncwarp();
+      for (int dlt = 1; dlt < 32; dlt <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, sbeg, dlt);
+        if (lane >= dlt) sbeg += o;
+      }
+      sbeg -= want;  // exclusive
+      const uint32_t nst = sbeg >= pool ? 0u : min(want, pool - sbeg);
+      if (more) {
+        const uint4* src4 = reinterpret_cast<const uint4*>(words + w0);
+        uint4* dst4 = reinterpret_cast<uint4*>(smem + stage0 + 4 * sbeg);
+#pragma unroll 1
+        for (uint32_t j = 0; j < nst / 4; j += 4) {
+          uint4 r[4];
 #pragma unroll
-          for (int i = 0; i < 12; ++i) coef[(lane + 32 * i) * M] = v[i];
+          for (int t = 0; t < 4; ++t) r[t] = j + t < nst / 4 ? __ldg(src4 + j + t) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+            if (j + t < nst / 4) dst4[j + t] = make_uint4(bswap(r[t].x), bswap(r[t].y), bswap(r[t].z), bswap(r[t].w));
         }
       }
-    } else if (act && !unit) {
-      const Words W{(uint32_t)__cvta_generic_to_shared(stage + sbeg), nst, words + w0,
-                    nwords > w0 ? nwords - w0 : 0u};
-      const Tables<true> TS{hs, (uint32_t)__cvta_generic_to_shared(sh->t)};
-      const Tables<false> TG{hs, 0u};
-      const uint32_t b0 = bitpos - w0 * 32;
-      uint32_t end;
-      if (hs == sh->t)
-        end = cpt ? decode_mcu<M, true, true>(W, b0, TS, ndu, pr0, pr1, pr2, col)
-                  : decode_mcu<M, true, false>(W, b0, TS, ndu, pr0, pr1, pr2, col);
-      else
-        end = cpt ? decode_mcu<M, false, true>(W, b0, TG, ndu, pr0, pr1, pr2, col)
-                  : decode_mcu<M, false, false>(W, b0, TG, ndu, pr0, pr1, pr2, col);
-      // a compact MCU must also end inside its own bytes
-      if (end == 0xFFFFFFFFu || (uint64_t)w0 * 32 + end > (cpt ? endbit : nbits)) any_bad = true;
-    }
-
-    if (UNITS) {  // chain the data units' DC differences (first lane of each MCU)
       __syncwarp();
-      if (act && unit && ld == 0) {
-        int c0 = pr0;
-#pragma unroll 1
-        for (int du = 0; du < ndu - 2; ++du) {  // luma: each unit's difference to the previous
-          int16_t* dcp = col + du * 64 * M;
-          c0 = (int16_t)(uint16_t)(c0 + (int)*dcp);  // modulo 2^16
-          *dcp = (int16_t)c0;
+      const bool whole = nst >= all;  // staged to its end
+      if (more && (whole || nst >= 12)) {
+        const uint32_t st = stage0 + 4 * sbeg, limit = whole ? 0xFFFFFFFFu : 8 * st + 32 * nst - kGroupBits;
+        bool ok = all != 0;
+        if (ok)
+          ok = !staged_set  ? entropy_fast<false, true>(ch, st, w0, limit, hs)
+               : staged_cap ? entropy_fast<true, true>(ch, st, w0, limit, hs)
+                            : entropy_fast<true, false>(ch, st, w0, limit, hs);
+        more = ok && ch.q != ch.qend;
+        if (!more) {
+          uint64_t end = 32ull * w0 + (ch.pos - 32 * w0);  // after the last symbol
+          // an invalid symbol, or bits past the stage: from the start again, word by word
+          if (!ok || ch.pos - 32 * w0 + 32 > 32 * nst) {
+            const uint32_t f = (bitpos >> 5) & ~3u;
+            const uint32_t r = entropy_any(words + f, nwords > f ? nwords - f : 0u, bitpos - 32 * f, hs, nd, nl, cpt, dst);
+            ok = r < kInvalid;
+            end = 32ull * f + r;
+            if (!ok && !unit) reached = (int)(r - kInvalid);
+          }
+          // the coding must be valid and end inside the stream; a compact MCU inside its own
+          // bytes, a data unit at or before the next one's start
+          if (!ok || end > ((cpt || unit) ? endbit : nbits)) any_bad = true;
         }
-        int16_t* cb = col + (ndu - 2) * 64 * M;
-        int16_t* cr = col + (ndu - 1) * 64 * M;
-        *cb = (int16_t)(uint16_t)((int)pr1 + (int)*cb);
-        *cr = (int16_t)(uint16_t)((int)pr2 + (int)*cr);
       }
+      __syncwarp();
+    } while (__any_sync(0xFFFFFFFFu, more));
+    __syncwarp();
+    if (act && ld == 0) {  // chain the DC differences (modulo 2^16)
+      uint32_t o = mine;
+      int c0 = pr0;
+#pragma unroll 1
+      for (int d = 0; d < min(ndu - 2, reached); ++d, o += 128) {
+        c0 = (int16_t)(uint16_t)(c0 + (int)sm_i16(o));
+        sm_i16(o) = (int16_t)c0;
+      }
+      if (reached > ndu - 2) sm_i16(o) = (int16_t)(uint16_t)((int)pr1 + (int)sm_i16(o));
+      if (reached > ndu - 1) sm_i16(o + 128) = (int16_t)(uint16_t)((int)pr2 + (int)sm_i16(o + 128));
     }
-
-    // ---- IDCT: the batch's data units are shared out over the warp: pair q = (d, m) (data
-    // unit d of MCU m) goes to lane q % 32 in round q / 32, which runs the column and the
-    // row pass of that data unit. MCU m's set-up values come from its first lane.
-    const uint32_t minfo =
-        (act ? 1u : 0u) | (s420 ? 2u : 0u) | ((uint32_t)red << 2) | (store ? 16u : 0u) | (qs << 8);
+    // ---- pixel phase: the warp takes the batch's MCUs one by one ----
+    const uint32_t minfo = (act && store ? 1u : 0u) | (s420 ? 2u : 0u) | ((uint32_t)red << 2) | (qs << 8);
     __syncwarp();  // every lane's coefficients are visible to the warp
+    Steps Q{};
+    Frag fr = f8;  // fragments of the last reduced level
+    int rcur = 0;
+    uint32_t qcur = 0xFFFFFFFFu;
 #pragma unroll 1
-    for (int r0 = 0; r0 < (warp_done ? 0 : 6 * meff); r0 += 32) {
-      const int q = r0 + lane;
-      const int d = q >> lmeff, m = q & (meff - 1);
-      const uint32_t im = __shfl_sync(0xFFFFFFFFu, minfo, UNITS ? 6 * m : m);
-      if (q < 6 * meff && (im & 1u) && d < ((im & 2u) ? 6 : 3)) {
-        const uint16_t* Qd = a.quant + (size_t)(im >> 8) * 128 + (d < ((im & 2u) ? 4 : 1) ? 0 : 64);
-        int16_t* blk = coef + d * 64 * M + m;
-        const int rm = (int)((im >> 2) & 3u);
-        if (rm == 0)
-          idct_full<M>(blk, Qd);
-        else if (rm == 1)
-          idct_reduced<M, 1>(blk, Qd);
-        else if (rm == 2)
-          idct_reduced<M, 2>(blk, Qd);
-        else
-          idct_reduced<M, 3>(blk, Qd);
-      }
-    }
-    __syncwarp();  // every data unit's pixels are visible to the warp
-
-    // ---- colour conversion + tile stores. Full-size 4:2:0 tiles are shared out as pairs
-    // (MCU m, column group c2 of 4 texels), 16-byte stores; 4:4:4 and reduced tiles are
-    // written by their own lane ----
-#pragma unroll 1
-    for (int r0 = 0; r0 < (warp_done ? 0 : 4 * meff); r0 += 32) {
-      const int q = r0 + lane;
-      const int m = (q >> 2) & (meff - 1), c2 = q & 3;
+    for (int m = 0; m < meff; ++m) {
       const uint32_t im = __shfl_sync(0xFFFFFFFFu, minfo, UNITS ? 6 * m : m);
       const uint32_t om = __shfl_sync(0xFFFFFFFFu, off, UNITS ? 6 * m : m);
-      if (q < 4 * meff && (im & 0x1Fu) == (1u | 2u | 16u)) {  // active, 4:2:0, full size, stored
-        const int16_t* cm = coef + m;
-        uint8_t* tile = a.cache + (size_t)om * kUnitBytes;
-        // chroma sample (cx, cy) covers texels 2cx..2cx+1, 2cy..2cy+1; texels x = 4 c2 .. 4 c2 + 3
-#pragma unroll 1
-        for (int cy = 0; cy < 8; ++cy) {
-          const uint32_t cb2 = pixel2<M>(cm, 4, cy, c2), cr2 = pixel2<M>(cm, 5, cy, c2);
-          int ro[2], go[2], bo[2];
-          chroma_offsets(cb2 & 255, cr2 & 255, ro[0], go[0], bo[0]);
-          chroma_offsets(cb2 >> 8, cr2 >> 8, ro[1], go[1], bo[1]);
-#pragma unroll
-          for (int dy = 0; dy < 2; ++dy) {
-            const int ty = 2 * cy + dy;
-            const int du = (ty >> 3) * 2 + (c2 >> 1), ry = ty & 7, ci = (c2 & 1) * 2;
-            const uint32_t ya = pixel2<M>(cm, du, ry, ci), yb = pixel2<M>(cm, du, ry, ci + 1);
-            uint4 o;
-            o.x = ycc_pixel(ya & 255, ro[0], go[0], bo[0]);
-            o.y = ycc_pixel(ya >> 8, ro[0], go[0], bo[0]);
-            o.z = ycc_pixel(yb & 255, ro[1], go[1], bo[1]);
-            o.w = ycc_pixel(yb >> 8, ro[1], go[1], bo[1]);
-            *reinterpret_cast<uint4*>(tile + (ty * 16 + 4 * c2) * 4) = o;
-          }
-        }
+      if (!(im & 1u)) continue;
+      if (im >> 8 != qcur) {
+        qcur = im >> 8;
+        const uint16_t* q = a.quant + (size_t)qcur * 128;
+        Q.la = __ldg(q + oa / 2);
+        Q.lb = __ldg(q + ob / 2);
+        Q.ca = __ldg(q + 64 + oa / 2);
+        Q.cb = __ldg(q + 64 + ob / 2);
+        Q.l = __floats2half2_rn(fminf((float)Q.la, 32768.f), fminf((float)Q.lb, 32768.f));
+        Q.c = __floats2half2_rn(fminf((float)Q.ca, 32768.f), fminf((float)Q.cb, 32768.f));
       }
-    }
-    if (!warp_done && act && ld == 0 && store && red != 0)
-      colour_reduced<M>(col, s420, red, reinterpret_cast<uint32_t*>(a.cache + (size_t)off * kUnitBytes));
-    if (!warp_done && act && ld == 0 && store && red == 0 && !s420) {  // 4:4:4, 8x8 texels, Y Cb Cr data units 0 1 2
-      uint8_t* tile = a.cache + (size_t)off * kUnitBytes;
-#pragma unroll 1
-      for (int ty = 0; ty < 8; ++ty) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {  // texels x = 4h .. 4h + 3
-          uint32_t o[4];
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const uint32_t y2 = pixel2<M>(col, 0, ty, 2 * h + j), b2 = pixel2<M>(col, 1, ty, 2 * h + j),
-                           r2 = pixel2<M>(col, 2, ty, 2 * h + j);
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              int ro, go, bo;
-              chroma_offsets((b2 >> (8 * e)) & 255, (r2 >> (8 * e)) & 255, ro, go, bo);
-              o[2 * j + e] = ycc_pixel((y2 >> (8 * e)) & 255, ro, go, bo);
-            }
-          }
-          *reinterpret_cast<uint4*>(tile + (ty * 8 + 4 * h) * 4) = make_uint4(o[0], o[1], o[2], o[3]);
+      const uint32_t cm = coef0 + (uint32_t)(m * kMcuBytes);
+      uint32_t* tile = reinterpret_cast<uint32_t*>(a.cache + (size_t)om * kUnitBytes);
+      const int rm = (int)((im >> 2) & 3u);
+      if (rm == 0) {
+        if (im & 2u)
+          mcu_pixels<true, false>(f8, cm, oa, ob, Q, bound, 0, tile, lane);
+        else
+          mcu_pixels<false, false>(f8, cm, oa, ob, Q, bound, 0, tile, lane);
+      } else {
+        if (rm != rcur) {
+          rcur = rm;
+          fr = idct_frag(rm, lane);
         }
+        if (im & 2u)
+          mcu_pixels<true, true>(fr, cm, oa, ob, Q, bound, rm, tile, lane);
+        else
+          mcu_pixels<false, true>(fr, cm, oa, ob, Q, bound, rm, tile, lane);
       }
     }
     __syncwarp();  // the buffers are cleared for the next items
@@ -1081,74 +765,41 @@ __global__ void k_decode(const __grid_constant__ DecodeArgs a) {
   if (any_bad) atomicOr(&a.state->err, JT_DEVERR_CORRUPT);
 }
 
-size_t smem_bytes(int warps, int M) { return sizeof(HuffSet) + 64 + (size_t)warps * warp_smem(M); }
+size_t smem_bytes(int warps, int M) { return kStagedTables + (size_t)warps * warp_smem(M) + kSlackBytes; }
 
-template <int M, bool UNITS, bool SHORT>
-int occupancy_of(int warps) {
-  const size_t smem = smem_bytes(warps, M);
-  if (smem > 227 * 1024) return 0;
-  if (cudaFuncSetAttribute(k_decode<M, UNITS, SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess) {
+template <bool UNITS>
+int occupancy_of(int warps, int M) {
+  const size_t smem_b = smem_bytes(warps, M);
+  if (smem_b > 227 * 1024) return 0;
+  if (cudaFuncSetAttribute(k_decode<UNITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_decode<M, UNITS, SHORT>, warps * 32, smem) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_decode<UNITS>, warps * 32, smem_b) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
   return n;
 }
 
-// resident CTAs per SM that every variant reaches (the launch picks one per frame)
-template <int M>
-int occupancy(int warps) {
-  return min(min(occupancy_of<M, false, false>(warps), occupancy_of<M, true, false>(warps)),
-             occupancy_of<M, false, true>(warps));
-}
-
 }  // namespace
 
 size_t decode_smem_bytes(int warps, int mcus_per_warp) { return smem_bytes(warps, mcus_per_warp); }
 
-// The dynamic shared-memory attribute of each variant is set by decode_max_ctas_per_sm(),
+// The dynamic shared-memory attribute of both variants is set by decode_max_ctas_per_sm(),
 // which the context calls for every (warps, M) on its device before the first launch.
 void launch_decode(const DecodeArgs& a, int warps, int grid, cudaStream_t s) {
-  const size_t smem = smem_bytes(warps, a.mcus_per_warp);
-  if (a.unit_mode) {
-    switch (a.mcus_per_warp) {
-      case 4: launch_pdl(k_decode<4, true, false>, grid, warps * 32, smem, s, a); break;
-      case 8: launch_pdl(k_decode<8, true, false>, grid, warps * 32, smem, s, a); break;
-      case 16: launch_pdl(k_decode<16, true, false>, grid, warps * 32, smem, s, a); break;
-      default: launch_pdl(k_decode<32, true, false>, grid, warps * 32, smem, s, a); break;
-    }
-    return;
-  }
-  if (a.short_lists) {
-    switch (a.mcus_per_warp) {
-      case 4: launch_pdl(k_decode<4, false, true>, grid, warps * 32, smem, s, a); break;
-      case 8: launch_pdl(k_decode<8, false, true>, grid, warps * 32, smem, s, a); break;
-      case 16: launch_pdl(k_decode<16, false, true>, grid, warps * 32, smem, s, a); break;
-      default: launch_pdl(k_decode<32, false, true>, grid, warps * 32, smem, s, a); break;
-    }
-    return;
-  }
-  switch (a.mcus_per_warp) {
-    case 4: launch_pdl(k_decode<4, false, false>, grid, warps * 32, smem, s, a); break;
-    case 8: launch_pdl(k_decode<8, false, false>, grid, warps * 32, smem, s, a); break;
-    case 16: launch_pdl(k_decode<16, false, false>, grid, warps * 32, smem, s, a); break;
-    default: launch_pdl(k_decode<32, false, false>, grid, warps * 32, smem, s, a); break;
-  }
+  const size_t smem_b = smem_bytes(warps, a.mcus_per_warp);
+  if (a.unit_mode)
+    launch_pdl(k_decode<true>, grid, warps * 32, smem_b, s, a);
+  else
+    launch_pdl(k_decode<false>, grid, warps * 32, smem_b, s, a);
 }
 
+// Resident CTAs per SM that both variants reach (the launch picks one per frame).
 int decode_max_ctas_per_sm(int warps, int mcus_per_warp) {
-  switch (mcus_per_warp) {
-    case 4: return occupancy<4>(warps);
-    case 8: return occupancy<8>(warps);
-    case 16: return occupancy<16>(warps);
-    case 32: return occupancy<32>(warps);
-  }
-  return 0;
+  return min(occupancy_of<false>(warps, mcus_per_warp), occupancy_of<true>(warps, mcus_per_warp));
 }
 
 void idct_constants(int out[8]) {

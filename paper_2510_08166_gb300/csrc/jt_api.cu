@@ -57,10 +57,13 @@ struct jt_ctx {
   int32_t* d_map = nullptr;
   LevelRec* d_lrec = nullptr;
   PixRec* d_prec = nullptr;
-  std::vector<HuffSet> hsets;
+  std::vector<std::vector<HuffSet>> hsets;            // one set each
+  std::vector<std::vector<jt_huff_spec>> huff_specs;  // the specs of each set, unused values zeroed
   HuffSet* d_huff = nullptr;
+  size_t huff_cap = 0, huff_have = 0;  // sets allocated, sets copied
   std::vector<std::vector<uint16_t>> qsets;  // zig-zag order, 128 entries
   uint16_t* d_quant = nullptr;
+  size_t quant_cap = 0, quant_have = 0;
   uint64_t ngid = 0;
 
   // per-frame buffers
@@ -175,18 +178,18 @@ void zigzag_natural(int nat[64]) {
     }
 }
 
-// Table entry of symbol `sym` with a code of length l (0 when the symbol is invalid for the
+// Table entry of symbol `sym` with a code of length l (kNoEntry when the symbol is invalid for the
 // table's class; the decoder's MAXCODE walk then rejects it).
 uint16_t symbol_entry(bool dc, int l, uint8_t sym) {
   const int r = dc ? 0 : sym >> 4, s = dc ? sym : sym & 15;
-  if ((dc && s > 11) || (!dc && s > 10) || (!dc && s == 0 && r != 0 && r != 15)) return 0;
+  if ((dc && s > 11) || (!dc && s > 10) || (!dc && s == 0 && r != 0 && r != 15)) return kNoEntry;
   if (!dc && s == 0) return huff_entry((uint32_t)l, 0, r == 0 ? kRunEob : 15u);
   return huff_entry((uint32_t)l, (uint32_t)s, (uint32_t)r);
 }
 
-// Canonical decode tables of one Huffman spec (T.81 Annex C code assignment).
-bool build_table(const jt_huff_spec& spec, bool dc, HuffTable& t, std::string& why) {
-  std::memset(&t, 0, sizeof t);
+// Canonical decode tables of one Huffman spec (T.81 Annex C code assignment): its entries at
+// `lut`, their count, and the walk's tables.
+bool build_table(const jt_huff_spec& spec, bool dc, uint16_t* lut, uint32_t& entries, HuffWalk& t, std::string& why) {
   int n = 0;
   uint64_t kraft = 0;
   for (int l = 1; l <= 16; ++l) {
@@ -202,11 +205,16 @@ bool build_table(const jt_huff_spec& spec, bool dc, HuffTable& t, std::string& w
     return false;
   }
   std::memcpy(t.vals, spec.vals, n);
-  // left-aligned start of the codes longer than kLutBits = Kraft mass of the shorter ones
-  uint32_t first16 = 0;
-  for (int l = 1; l <= kLutBits; ++l) first16 += (uint32_t)spec.bits[l - 1] << (16 - l);
-  t.first16 = first16;
-  t.n2 = (first16 < 65536u && 65536u - first16 <= (uint32_t)kLut2Size) ? 65536u - first16 : 0u;
+  // left-aligned start of the codes longer than kLutBits = Kraft mass of the shorter ones;
+  // 65536 (no second granularity) when they take too many prefixes
+  uint32_t first = 0;
+  for (int l = 1; l <= kLutBits; ++l) first += (uint32_t)spec.bits[l - 1] << (16 - l);
+  const uint32_t end = std::min<uint32_t>((uint32_t)kraft + 1, 65536u);  // one entry past the last code stays empty
+  if (kraft <= first || end - first > (uint32_t)kLut2Size) first = 65536u;
+  t.d = (int32_t)(first >> 6) - (int32_t)first;
+  entries = (first >> 6) + (first < 65536u ? end - first : 0u);
+  t.cap = (int32_t)entries - 1;
+  std::fill(lut, lut + entries, kNoEntry);
   int code = 0, k = 0;
   for (int l = 1; l <= 16; ++l) {
     const int nl = spec.bits[l - 1];
@@ -218,11 +226,11 @@ bool build_table(const jt_huff_spec& spec, bool dc, HuffTable& t, std::string& w
       for (int i = 0; i < nl; ++i, ++k, ++code) {
         const uint16_t e = symbol_entry(dc, l, spec.vals[k]);
         if (l <= kLutBits) {
-          const int first = code << (kLutBits - l), cnt = 1 << (kLutBits - l);
-          for (int j = 0; j < cnt; ++j) t.lut[first + j] = e;
-        } else if (t.n2) {
-          const uint32_t first = ((uint32_t)code << (16 - l)) - first16, cnt = 1u << (16 - l);
-          for (uint32_t j = 0; j < cnt; ++j) t.lut2[first + j] = e;
+          const uint32_t at = (uint32_t)code << (kLutBits - l), cnt = 1u << (kLutBits - l);
+          for (uint32_t j = 0; j < cnt; ++j) lut[at + j] = e;
+        } else if (first < 65536u) {
+          const uint32_t at = (uint32_t)((int32_t)((uint32_t)code << (16 - l)) + t.d), cnt = 1u << (16 - l);
+          for (uint32_t j = 0; j < cnt; ++j) lut[at + j] = e;
         }
       }
       t.maxcode[l] = code - 1;
@@ -230,6 +238,47 @@ bool build_table(const jt_huff_spec& spec, bool dc, HuffTable& t, std::string& w
     code <<= 1;
   }
   t.maxcode[0] = -1;
+  return true;
+}
+
+// The decode tables of four specs (DC luma, AC luma, DC chroma, AC chroma).
+bool build_set(const jt_huff_spec huff[4], HuffSet& hs, std::string& why) {
+  std::memset(&hs, 0, sizeof hs);
+  uint32_t at = 0;
+  for (int t = 0; t < 4; ++t) {
+    uint32_t entries = 0;
+    if (!build_table(huff[t], t % 2 == 0, hs.lut + at, entries, hs.walk[t], why)) {
+      why = "Huffman table " + std::to_string(t) + ": " + why;
+      return false;
+    }
+    hs.walk[t].base = (uint32_t)offsetof(HuffSet, lut) + 2 * at;
+    at += entries;
+  }
+  hs.used = (uint32_t)offsetof(HuffSet, lut) + 2 * at;
+  for (const HuffWalk& w : hs.walk) hs.capped |= 65535 + w.d > w.cap ? 1u : 0u;
+  // data unit i of a chain of nl luma and nc chroma units, then the record past the end
+  HuffWalk none{};
+  none.base = (uint32_t)offsetof(HuffSet, none);
+  none.d = (65536 >> 6) - 65536;
+  none.cap = kLutSize - 1;
+  auto chain = [&](int first, int nl, int nc, bool compact) {
+    auto ac = [&](int i) { return i < nl ? 1 : 3; };
+    auto apart = [&](int i) { return compact && (i == 0 || i >= nl); };  // DC not in the stream
+    auto head = [&](int i) { return apart(i) ? ac(i) : ac(i) - 1; };
+    for (int i = 0; i <= nl + nc; ++i) {
+      HuffSeq& q = hs.seq[first + i];
+      const bool over = i == nl + nc, final = i + 1 >= nl + nc;
+      const HuffWalk &a = over ? none : hs.walk[ac(i)], &n = final ? none : hs.walk[head(i + 1)], &o = hs.walk[head(i)];
+      q = HuffSeq{a.base, a.d, n.base, n.d, (!final && apart(i + 1) ? 1u : 0u) << kRunShift, a.cap, n.cap, 0u,
+                  o.base, o.d, (apart(i) ? 1u : 0u) << kRunShift, o.cap};
+    }
+  };
+  chain(kSeq420, 4, 2, false);
+  chain(kSeq444, 1, 2, false);
+  chain(kSeqCompact420, 4, 2, true);
+  chain(kSeqCompact444, 1, 2, true);
+  chain(kSeqLuma, 1, 0, false);
+  chain(kSeqChroma, 0, 1, false);
   return true;
 }
 
@@ -285,18 +334,32 @@ jt_status sync_descs(jt_ctx* c) {
   return JT_OK;
 }
 
-jt_status sync_tables(jt_ctx* c) {
+// Device copies of the Huffman sets and quantisation tables: grown by doubling, and only the
+// sets added since the last call are copied.
+template <typename T, typename V>
+jt_status sync_sets(jt_ctx* c, T*& dev, size_t& cap, size_t& have, const V& sets, size_t bytes) {
+  const size_t n = sets.size();
+  if (dev && have == n) return JT_OK;
   ++c->generation;
-  dev_free(c->d_huff);
-  jt_status s = dev_alloc(c, &c->d_huff, std::max<size_t>(1, c->hsets.size()) * sizeof(HuffSet));
-  if (s != JT_OK) return s;
-  if (!c->hsets.empty())
-    JT_CUDA(c, cudaMemcpy(c->d_huff, c->hsets.data(), c->hsets.size() * sizeof(HuffSet), cudaMemcpyHostToDevice));
-  dev_free(c->d_quant);
-  if ((s = dev_alloc(c, &c->d_quant, std::max<size_t>(1, c->qsets.size()) * 256)) != JT_OK) return s;
-  for (size_t i = 0; i < c->qsets.size(); ++i)
-    JT_CUDA(c, cudaMemcpy(c->d_quant + i * 128, c->qsets[i].data(), 256, cudaMemcpyHostToDevice));
+  if (!dev || n > cap) {
+    dev_free(dev);
+    have = 0;
+    cap = std::max<size_t>({n, 2 * cap, 1});
+    jt_status s = dev_alloc(c, &dev, cap * bytes);
+    if (s != JT_OK) {
+      cap = 0;
+      return s;
+    }
+  }
+  for (; have < n; ++have)
+    JT_CUDA(c, cudaMemcpy(reinterpret_cast<uint8_t*>(dev) + have * bytes, sets[have].data(), bytes,
+                          cudaMemcpyHostToDevice));
   return JT_OK;
+}
+
+jt_status sync_tables(jt_ctx* c) {
+  jt_status s = sync_sets(c, c->d_huff, c->huff_cap, c->huff_have, c->hsets, sizeof(HuffSet));
+  return s != JT_OK ? s : sync_sets(c, c->d_quant, c->quant_cap, c->quant_have, c->qsets, 256);
 }
 
 bool pow2(uint32_t v) { return v && !(v & (v - 1)); }
@@ -462,8 +525,8 @@ jt_status enqueue_decode(jt_ctx* c, cudaStream_t s) {
   a.desc_of_gid = c->d_desc_of_gid;
   a.mcus_per_warp = c->tuning.decode_mcus_per_warp;
   a.unit_mode = c->unit_mode ? 1 : 0;
-  a.short_lists = c->tuning.decode_short_lists < 0 ? (c->persistent ? 1 : 0) : c->tuning.decode_short_lists;
   a.huff = c->d_huff;
+  a.nsets = (uint32_t)c->hsets.size();
   a.quant = c->d_quant;
   a.work = c->work;
   a.work_cap = (uint32_t)c->gid_cap;
@@ -630,9 +693,11 @@ jt_status jt_create(jt_ctx** out, int device, uint64_t max_cache_blocks) {
   for (int M : kMcusPerWarp)
     for (int W = 1; W <= 16; ++W) c->decode_occ[M][W] = decode_max_ctas_per_sm(W, M);
   cudaGetLastError();
-  c->tuning.decode_mcus_per_warp = 32;
-  c->tuning.decode_warps = 4;
-  c->tuning.decode_ctas_per_sm = std::max(1, c->decode_occ[32][4]);
+  // the widest shape that fills an SM's shared memory at 16 MCUs per warp: of the shapes tried
+  // it was the fastest or within 3 % of it on lists of 2 to 9000 MCUs per SM
+  c->tuning.decode_mcus_per_warp = 16;
+  c->tuning.decode_warps = 14;
+  c->tuning.decode_ctas_per_sm = std::max(1, c->decode_occ[16][14]);
   c->tuning.pixel_threads = 256;
   c->tuning.pixel_ctas_per_sm = 8;
   c->tuning.decode_short_lists = -1;
@@ -786,14 +851,22 @@ static jt_status upload_level(jt_ctx* c, int tex_id, int level, int width, int h
   if (!g.ok) return fail(c, JT_ERR_CUDA, "cannot select device %d", c->device);
 
   // decode tables (deduplicated by content)
-  HuffSet hs;
-  std::string why;
-  for (int t = 0; t < 4; ++t)
-    if (!build_table(huff[t], t % 2 == 0, hs.t[t], why))
-      return fail(c, JT_ERR_INVALID_ARG, "Huffman table %d: %s", t, why.c_str());
+  std::vector<jt_huff_spec> specs(huff, huff + 4);
+  for (jt_huff_spec& h : specs) {
+    int n = 0;
+    for (int l = 0; l < 16; ++l) n += h.bits[l];
+    for (int i = n; i < 256; ++i) h.vals[i] = 0;
+  }
+  auto same = [&](const std::vector<jt_huff_spec>& o) { return std::memcmp(o.data(), specs.data(), 4 * sizeof(jt_huff_spec)) == 0; };
   int hset = -1;
-  for (size_t i = 0; i < c->hsets.size(); ++i)
-    if (std::memcmp(&c->hsets[i], &hs, sizeof hs) == 0) hset = (int)i;
+  for (size_t i = 0; i < c->huff_specs.size(); ++i)
+    if (same(c->huff_specs[i])) hset = (int)i;
+  std::vector<HuffSet> hs;
+  std::string why;
+  if (hset < 0) {
+    hs.resize(1);
+    if (!build_set(huff, hs[0], why)) return fail(c, JT_ERR_INVALID_ARG, "%s", why.c_str());
+  }
   int nat[64];
   zigzag_natural(nat);
   std::vector<uint16_t> qz(128);
@@ -805,7 +878,8 @@ static jt_status upload_level(jt_ctx* c, int tex_id, int level, int width, int h
   bool tables_changed = false;
   if (hset < 0) {
     if (c->hsets.size() >= 255) return fail(c, JT_ERR_UNSUPPORTED, "more than 255 distinct Huffman table sets");
-    c->hsets.push_back(hs);
+    c->hsets.push_back(std::move(hs));
+    c->huff_specs.push_back(specs);
     hset = (int)c->hsets.size() - 1;
     tables_changed = true;
   }

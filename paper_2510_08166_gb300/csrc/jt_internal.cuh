@@ -6,7 +6,7 @@
 //   desc_map   int32[ntex * 16]      (tex_id, level) -> desc index, -1 when absent
 //   streams    per level: uint32 words of the unstuffed entropy stream + >= 64 zero bytes
 //   index      per level: packed 10-byte {bit_offset, dc_pred[3]} entries
-//   huff       HuffSet[nh]           decode LUTs, deduplicated by content
+//   huff       HuffSet[nh]           decode tables, deduplicated by content
 //   quant      uint16[nq][2][64]     quantisation tables in zig-zag order
 //   flags      uint8[ngid]           per-frame marks: cache units of the MCU (4, 1) or 0
 //   slot       uint32[ngid]          cache-unit offset of each needed gid
@@ -17,6 +17,7 @@
 
 #include <cuda_runtime.h>
 
+#include <cstddef>
 #include <cstdint>
 
 #include "jt.h"
@@ -54,46 +55,91 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 
 constexpr int kLutBits = 10;                 // first-level Huffman LUT: next 10 bits
 constexpr int kLutSize = 1 << kLutBits;
-constexpr int kLut2Size = 1024;              // second-level LUT for longer codes
+constexpr int kLut2Size = 4096;              // entries for longer codes, at most
 constexpr int kStreamPadBytes = 64;          // zero padding after each entropy stream
 constexpr uint32_t kUnitBytes = 256;         // cache unit
 constexpr int kSampling420 = 0, kSampling444 = 1, kSamplingCoef = 2;
 
-// Decode tables of one Huffman spec (T.81 Annex C canonical codes). A symbol entry is 16
-// bits: code length l (bits 0..4), value-bit count s (bits 5..8), run r (bits 9..14):
-//   AC value  (r, s)   -> store at k + r, advance k by r + 1
-//   ZRL       (15, 0)  -> advance 16 (the skipped slots are zero)
-//   EOB       (63, 0)  -> advance 64 (store a zero at slot 63, which is zero already)
-//   DC        (0, s)   -> difference, advance 1
-// The s value bits follow the code in the stream; the decoder cuts them from its 32-bit
-// window itself (T.81 EXTEND), so an entry depends on the code alone. 0 = no entry.
-//   lut[i]   entry of the code that starts the next kLutBits bits i (codes up to kLutBits)
-//   lut2[j]  entry of the longer code whose 16-bit left-aligned prefix is first16 + j: in
-//            canonical order the longer codes are the numerically largest, so they occupy
-//            the top n2 of the 65536 16-bit prefixes (n2 <= kLut2Size, else 0)
-// The decoder reads both entries for every symbol (the two reads are independent), so a
-// long code costs no branch. Codes without an entry (invalid codes, long codes of tables
-// whose range exceeds kLut2Size) and symbols invalid for the table's class (DC category >
-// 11, AC size > 10, AC size 0 with a run other than 0 or 15) go to the MAXCODE walk of
-// T.81 F.2.2.3, which decodes or rejects them.
+// Decode tables of one set of four Huffman specs (T.81 Annex C canonical codes; DC luma, AC
+// luma, DC chroma, AC chroma). A symbol entry is 16 bits:
+//   bits 0..4    code length plus value bits s (at most 27)
+//   bits 5..8    s
+//   bits 10..15  run r: AC value (r, s) -> store at k + r, advance k by r + 1; ZRL (15, 0) ->
+//                advance 16; EOB (63, 0); DC (0, s). The top field, so that an entry added to
+//                k << 10 gives the coefficient's place there.
+// The s value bits follow the code in the stream; the decoder cuts them from its window
+// itself (T.81 EXTEND), so an entry depends on the code alone. kNoEntry marks the rest: value
+// bits and a run that is past slot 63 from any k.
+//
+// A table's entries are one array over two granularities. Codes of at most kLutBits bits are
+// indexed by the next kLutBits bits w >> 22. In canonical order the longer codes are the
+// numerically largest: they start at the 16-bit left-aligned prefix `first` (a multiple of
+// 64), and their entries, one per 16-bit prefix, start where the short ones end, at
+// first >> 6. The index of any code is then max(w >> 22, (w >> 16) + d) with
+// d = (first >> 6) - first: the second term grows 64 times as fast and passes the first one
+// exactly at `first`. So a symbol is one read, without a branch or a select. Codes without
+// an entry (invalid codes, the long codes of a table where they take more than kLut2Size
+// prefixes) and symbols invalid for the table's class (DC category > 11, AC size > 10, AC
+// size 0 with a run other than 0 or 15) go to the MAXCODE walk of T.81 F.2.2.3, which decodes
+// or rejects them.
 __host__ __device__ constexpr uint16_t huff_entry(uint32_t l, uint32_t s, uint32_t r) {
-  return (uint16_t)(l | (s << 5) | (r << 9));
+  return (uint16_t)((l + s) | (s << 5) | (r << 10));
 }
 constexpr uint32_t kRunEob = 63;
-struct HuffTable {
-  uint16_t lut[kLutSize];
-  uint16_t lut2[kLut2Size];
-  uint32_t first16;     // 16-bit left-aligned value of the first code longer than kLutBits
-  uint32_t n2;          // entries of lut2 in use (0: no longer codes, or too many)
+constexpr int kRunShift = 10;
+constexpr uint16_t kNoEntry = 0xFFE0;
+
+// A code that leaves prefixes unused above its last one (`end`, 65536 for a complete code) has
+// entries up to there only, and the index of a longer code is also capped, at the table's
+// last entry (kNoEntry).
+//
+// The MAXCODE walk's tables of one spec, and where its entries are (byte offset in the set).
+struct HuffWalk {
   int32_t maxcode[17];  // -1 when no code of length l
   int32_t valoff[17];
   uint8_t vals[256];
+  uint32_t base;
+  int32_t d, cap;
+  uint32_t pad;
 };
 
-// Four tables: DC luma, AC luma, DC chroma, AC chroma.
-struct HuffSet {
-  HuffTable t[4];
+// The tables a chain of data units uses, one record per data unit and one past the last: those
+// of its AC symbols and of the next data unit's first symbol (byte offset in the set, d, cap),
+// and the next data unit's first k << kRunShift (k = 1 where the DC is stored apart).
+// The last data unit's next table and both of the record past it are the table of zeros.
+// start_*: of the data unit's own first symbol.
+struct HuffSeq {
+  uint32_t ac_base;
+  int32_t ac_d;
+  uint32_t next_base;
+  int32_t next_d;
+  uint32_t next_k;
+  int32_t ac_cap, next_cap;
+  uint32_t pad;
+  uint32_t start_base;
+  int32_t start_d;
+  uint32_t start_k;
+  int32_t start_cap;
 };
+static_assert(sizeof(HuffSeq) == 48, "read as 16-byte words");
+// records: 4:2:0 and 4:4:4 MCUs, the same in the compact form, one luma, one chroma data unit
+constexpr int kSeq420 = 0, kSeq444 = 7, kSeqCompact420 = 11, kSeqCompact444 = 18, kSeqLuma = 22, kSeqChroma = 24;
+constexpr int kSeqRecords = 26;
+constexpr int kMaxTableEntries = kLutSize + kLut2Size;
+
+struct HuffSet {
+  HuffSeq seq[kSeqRecords];
+  uint32_t used;    // bytes from the start of the set to the end of its entries
+  uint32_t capped;  // some table needs its cap
+  uint32_t pad[2];
+  uint16_t none[kLutSize];               // zeros: a symbol without value, run or length
+  uint16_t lut[4 * kMaxTableEntries];  // the four tables' entries, back to back
+  HuffWalk walk[4];
+};
+static_assert(sizeof(HuffSet) % 16 == 0 && offsetof(HuffSet, lut) % 16 == 0, "copied in 16-byte words");
+// A decode CTA stages one set in shared memory when it is at most this long (the typical tables
+// of the standard take 13,144 bytes).
+constexpr uint32_t kStagedTables = 18432;
 
 struct DevDesc {
   const uint32_t* stream;      // big-endian words (word i = bytes 4i..4i+3)
@@ -287,8 +333,8 @@ struct DecodeArgs {
   const uint32_t* desc_of_gid;  // descriptor index of each gid
   int mcus_per_warp;      // M, the buffer width: 4, 8, 16 or 32 (batches may be smaller)
   int unit_mode;          // some level has data-unit starts: the kernel that decodes them in parallel
-  int short_lists;        // the kernel that decodes short lists MCU by MCU with whole warps
-  const HuffSet* huff;    // set 0 is staged in shared memory
+  const HuffSet* huff;    // a CTA stages one of them in shared memory
+  uint32_t nsets;
   const uint16_t* quant;  // [nq][2][64] zig-zag order
   const uint32_t* work;
   uint32_t work_cap;
