@@ -8,10 +8,8 @@
 // Mark: one quad of 4 pixels per lane (32 B + 8 B + 4 B vector loads). Pixels of a tile
 // share MCUs, so Mark keeps a 1024-entry table of the gids its CTA already flagged in shared
 // memory and stores each flag about once per CTA instead of once per pixel (the byte stores
-// of every SM to the same flag lines otherwise dominate the pass). A pixel's (texture,
-// level) record is one 16-byte load, kept in registers while consecutive pixels share it;
-// levels whose sides are powers of two (all mip chains of power-of-two textures) wrap with a
-// mask, MCU coordinates are shifts.
+// of every SM to the same flag lines otherwise dominate the pass). A quad is decided at once
+// from the box of its taps (see k_mark).
 //
 // Colourise: a lane owns pixels 32 apart (lane + 32 k), so the 32 addresses of one texel
 // gather instruction are 32 consecutive pixels' taps, which fall in two or three tiles (half
@@ -372,13 +370,57 @@ __device__ __forceinline__ void load_row(const View& V, int x, int y, bool valid
 // ---------------------------------------------------------------------------------------
 constexpr int kSeen = 1024;  // per-CTA table of recently flagged gids
 
-template <int FILTER, bool MULTI>
+// Mark is bound by its instruction count (an evaluation of four taps and up to four table probes
+// per pixel ran at 72 % of the issue slots), so a lane decides its quad of four pixels at
+// once. Nearly every quad has one level, and its footprint, the box of the taps of its
+// pixels, lies in one row or one column of at most two MCUs, which are then exactly the MCUs
+// of the box's ends. Every other quad (several levels, both rows and columns, a larger box, a
+// repeat edge of a level whose sides are no powers of two, coordinates beyond 2^22, the ragged
+// end of a row) goes into the warp's queue, whose quads are taken eight at a time, a pixel
+// per lane: a few such quads in every warp cost their share and not a pass of the warp each
+// (in a branch of their own they made the kernel slower than the plain form: 50.9 against
+// 42.7 us on the 4K frame of 64 textures, bilinear). Measured: 42.7 -> 27.9 us on that frame
+// (43 % of the HBM rate, long_scoreboard first among its stalls), 395 -> 286 us for the
+// nearest texels of eight 4096^2 views (63 %).
+
+// One pixel on its own: flag(g) for every MCU its taps fall in.
+template <int FILTER, typename F>
+__device__ __forceinline__ void mark_pixel(const PixL& P, float u, float v, F&& flag) {
+  int xa, xb, ya, yb;
+  float fx, fy;
+  if (FILTER == JT_FILTER_NEAREST) {
+    if (!nearest_fast(P, u, v, xa, ya)) nearest_any(P, u, v, xa, ya);
+    flag(P.gid_base + ((uint32_t)xa >> P.shift) + ((uint32_t)ya >> P.shift) * P.mcus_x);
+    return;
+  }
+  if (!taps_fast(P, u, v, xa, xb, ya, yb, fx, fy)) taps_any(P, u, v, xa, xb, ya, yb, fx, fy);
+  const uint32_t ca = (uint32_t)xa >> P.shift, cb = (uint32_t)xb >> P.shift;
+  const uint32_t ra = P.gid_base + ((uint32_t)ya >> P.shift) * P.mcus_x, rb = P.gid_base + ((uint32_t)yb >> P.shift) * P.mcus_x;
+  flag(ra + ca);
+  if (cb != ca) flag(ra + cb);
+  if (rb != ra) {
+    flag(rb + ca);
+    if (cb != ca) flag(rb + cb);
+  }
+}
+
+constexpr int kMarkQueue = 8 + 32;  // quads waiting in a warp: fewer than eight, and one row segment's
+
+template <int FILTER>
 __global__ void k_mark(const __grid_constant__ MarkArgs a) {
+  constexpr int kTap = FILTER == JT_FILTER_NEAREST ? 0 : 1;  // the second tap's distance
+  extern __shared__ uint2 queue[];  // [warps][kMarkQueue]: first pixel in the view; view | pixels << 8
   __shared__ uint32_t seen[kSeen];
   pdl_launch_dependents();
   for (int i = threadIdx.x; i < kSeen; i += blockDim.x) seen[i] = kNoGid;
   __syncthreads();
+  const int lane = threadIdx.x & 31;
+  uint2* wq = queue + (threadIdx.x >> 5) * kMarkQueue;
+  int waiting = 0;
   bool missing = false;
+  const uint32_t kind = a.coef_mode ? kPixCoef : kPixJpeg;
+  // an empty pixel's texture, or one that is filtered out
+  auto skip = [&](uint32_t tex) { return tex == JT_EMPTY_TEXTURE || (a.only_tex >= 0 && (int)tex != a.only_tex); };
   // flags gid g unless this CTA already did (racy by design: a duplicate store writes the
   // same byte)
   auto flag = [&](uint32_t g, uint32_t units) {
@@ -388,39 +430,89 @@ __global__ void k_mark(const __grid_constant__ MarkArgs a) {
       a.flags[g] = (uint8_t)units;
     }
   };
+  // the last (at most) eight quads of the queue, a pixel per lane
+  auto drain = [&] {
+    __syncwarp();
+    const int n = min(waiting, 8);
+    waiting -= n;
+    if ((lane >> 2) < n) {
+      const uint2 e = wq[waiting + (lane >> 2)];
+      const View& V = a.views.v[e.y & 255u];
+      if ((uint32_t)(lane & 3) < e.y >> 8) {
+        const uint32_t p = e.x + (lane & 3);
+        const uint32_t tex = __ldg(V.tex + p);
+        if (!skip(tex)) {
+          const float2 uv = __ldg(reinterpret_cast<const float2*>(V.uv) + p);
+          const PixL P = pix_level(a.tl, tex | ((uint32_t)__ldg(V.mip + p) << 16));
+          if (P.info & kind)
+            mark_pixel<FILTER>(P, uv.x, uv.y, [&](uint32_t g) { flag(g, P.info & 255u); });
+          else
+            missing = true;
+        }
+      }
+    }
+    __syncwarp();
+  };
   for_each_quad(a.views, [&](const View& V, int y, int x) {
     float u[4], v[4];
     uint32_t t[4], m[4];
     const int n = load_px4(V, y, x, u, v, t, m);
-    QuadLevels q;
-    quad_levels(a.tl, n, t, m, a.only_tex, q);
-    for_quad_pixels(a.tl, q, [&](auto p2, const Lvl& L, int i) {
-      constexpr bool P2 = decltype(p2)::value;
-      const uint32_t key = q.key[i];
-      const bool ok = key < kNoKey - 1 && L.w != 0 && ((L.sampling == kSamplingCoef) == (a.coef_mode != 0));
-      missing |= key != kNoKey && !ok;
-      if (!ok) return;
-      if (FILTER == JT_FILTER_NEAREST) {
-        int tx, ty;
-        nearest_texel<P2>(u[i], v[i], L, tx, ty);
-        flag(L.gid_base + (tx >> L.shift) + (ty >> L.shift) * L.mcus_x, L.units);
-      } else {
-        int xa, xb, ya, yb;
-        float fx, fy;
-        bilinear_taps<P2>(u[i], v[i], L, xa, xb, ya, yb, fx, fy);
-        const int mxa = xa >> L.shift, mxb = xb >> L.shift;
-        const int mya = ya >> L.shift, myb = yb >> L.shift;
-        const uint32_t row_a = L.gid_base + mya * L.mcus_x;
-        flag(row_a + mxa, L.units);
-        if (mxb != mxa) flag(row_a + mxb, L.units);  // the footprint straddles MCUs (rare)
-        if (myb != mya) {
-          const uint32_t row_b = L.gid_base + myb * L.mcus_x;
-          flag(row_b + mxa, L.units);
-          if (mxb != mxa) flag(row_b + mxb, L.units);
-        }
-      }
-    });
+    const uint32_t t0 = t[0], m0 = m[0];
+    const bool one = n == 4 && ((t[1] ^ t0) | (t[2] ^ t0) | (t[3] ^ t0) | (m[1] ^ m0) | (m[2] ^ m0) | (m[3] ^ m0)) == 0;
+    const bool none = n == 0 || (one && skip(t0));
+    const PixL P = pix_level(a.tl, t0 | (m0 << 16));
+    int px[4], py[4];
+    uint32_t far = 0;  // exponents other than that of [2^23, 2^24): |coordinate| beyond 2^22
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float xs = __fmul_rn(u[i], P.wf), ys = __fmul_rn(v[i], P.hf);
+      const uint32_t bx = __float_as_uint(__fadd_rd(kTap ? __fsub_rn(xs, 0.5f) : xs, kMagic));
+      const uint32_t by = __float_as_uint(__fadd_rd(kTap ? __fsub_rn(ys, 0.5f) : ys, kMagic));
+      far |= (bx ^ 0x4B000000u) | (by ^ 0x4B000000u);
+      px[i] = (int)bx - 0x4B400000;
+      py[i] = (int)by - 0x4B400000;
+    }
+    int x0 = min(min(px[0], px[1]), min(px[2], px[3])), x1 = max(max(px[0], px[1]), max(px[2], px[3])) + kTap;
+    int y0 = min(min(py[0], py[1]), min(py[2], py[3])), y1 = max(max(py[0], py[1]), max(py[2], py[3])) + kTap;
+    bool box = one && (P.info & kind) && (far & 0xFF800000u) == 0;
+    // MCU coordinates are unwrapped up to here; powers of two wrap them with a mask
+    const uint32_t s = P.shift;
+    uint32_t cm = (P.masks & 0xFFFFu) >> s, rm = P.masks >> (16 + s);
+    if (!a.tl.all_p2 && !(P.info & kPixPow2)) {
+      // other sides: the quad moves into the level by its first pixel's repeat (any integer
+      // near the quotient will do: the box has to end up inside the level)
+      const int w = (int)(P.wh & 0xFFFFu), h = (int)(P.wh >> 16);
+      int rx = px[0] - __float2int_rd(__fdividef((float)px[0], P.wf)) * w;
+      int ry = py[0] - __float2int_rd(__fdividef((float)py[0], P.hf)) * h;
+      rx += rx < 0 ? w : rx >= w ? -w : 0;
+      ry += ry < 0 ? h : ry >= h ? -h : 0;
+      x0 += rx - px[0];
+      x1 += rx - px[0];
+      y0 += ry - py[0];
+      y1 += ry - py[0];
+      box = box && x0 >= 0 && x1 < w && y0 >= 0 && y1 < h;
+      cm = rm = 0xFFFFu;
+    }
+    const int c0 = x0 >> s, c1 = x1 >> s, r0 = y0 >> s, r1 = y1 >> s;
+    const int dc = c1 - c0, dr = r1 - r0;
+    box = box && dc + dr <= 1;  // (both are at least 0)
+    if (box && !none) {
+      const uint32_t units = P.info & 255u;
+      const uint32_t g0 = P.gid_base + ((uint32_t)r0 & rm) * P.mcus_x + ((uint32_t)c0 & cm);
+      const uint32_t g1 = P.gid_base + ((uint32_t)r1 & rm) * P.mcus_x + ((uint32_t)c1 & cm);
+      flag(g0, units);
+      if (g1 != g0) flag(g1, units);
+    }
+    const uint32_t rest = __ballot_sync(0xFFFFFFFFu, !box && !none);
+    if (rest) {
+      if (!box && !none)
+        wq[waiting + __popc(rest & ((1u << lane) - 1u))] =
+            make_uint2((uint32_t)y * (uint32_t)V.width + (uint32_t)x, (uint32_t)(&V - a.views.v) | ((uint32_t)n << 8));
+      waiting += __popc(rest);
+      while (waiting >= 8) drain();
+    }
   });
+  while (waiting > 0) drain();
   if (missing) atomicOr(&a.state->err, JT_DEVERR_MISSING);
 }
 
@@ -1078,18 +1170,11 @@ void launch_float_backward(const FloatArgs& a, int threads, int pixel_grid, int 
 
 void launch_mark(const MarkArgs& a, int threads, int grid, cudaStream_t s) {
   // the clamped filter reads only the nearest texel's MCU
-  const bool nearest = a.filter == JT_FILTER_NEAREST || a.filter == JT_FILTER_BILINEAR_CLAMP;
-  if (a.views.n > 1) {
-    if (nearest)
-      k_mark<JT_FILTER_NEAREST, true><<<grid, threads, 0, s>>>(a);
-    else
-      k_mark<JT_FILTER_BILINEAR, true><<<grid, threads, 0, s>>>(a);
-  } else {
-    if (nearest)
-      k_mark<JT_FILTER_NEAREST, false><<<grid, threads, 0, s>>>(a);
-    else
-      k_mark<JT_FILTER_BILINEAR, false><<<grid, threads, 0, s>>>(a);
-  }
+  const size_t smem = (size_t)(threads / 32) * kMarkQueue * sizeof(uint2);
+  if (a.filter == JT_FILTER_NEAREST || a.filter == JT_FILTER_BILINEAR_CLAMP)
+    k_mark<JT_FILTER_NEAREST><<<grid, threads, smem, s>>>(a);
+  else
+    k_mark<JT_FILTER_BILINEAR><<<grid, threads, smem, s>>>(a);
 }
 
 // pixels per lane per step: two (60 registers, 32 warps per SM) measured faster than four
