@@ -52,7 +52,7 @@ struct jt_ctx {
   uint64_t desc_of_gid_cap = 0;
   std::vector<int32_t> map;  // [map_ntex * 16]
   std::vector<LevelRec> lrec;  // [map_ntex * 16]
-  std::vector<PixRec> prec;    // [map_ntex * 16 + 1], the last one all zero
+  std::vector<PixRec> prec;    // [(map_ntex + 1) * kPixLevels]
   uint32_t map_ntex = 0;
   int32_t* d_map = nullptr;
   LevelRec* d_lrec = nullptr;
@@ -323,8 +323,7 @@ jt_status sync_descs(jt_ctx* c) {
   if (s != JT_OK) return s;
   if ((s = dev_alloc(c, &c->d_lrec, c->lrec.size() * sizeof(LevelRec))) != JT_OK) return s;
   dev_free(c->d_prec);
-  c->prec.resize(c->lrec.size() + 1, PixRec{});
-  c->prec.back() = PixRec{};  // the record of keys outside the table
+  c->prec.resize(((size_t)c->map_ntex + 1) * kPixLevels, PixRec{});
   if ((s = dev_alloc(c, &c->d_prec, c->prec.size() * sizeof(PixRec))) != JT_OK) return s;
   JT_CUDA(c, cudaMemcpy(c->d_prec, c->prec.data(), c->prec.size() * sizeof(PixRec), cudaMemcpyHostToDevice));
   if (!c->map.empty()) {
@@ -365,10 +364,13 @@ jt_status sync_tables(jt_ctx* c) {
 bool pow2(uint32_t v) { return v && !(v & (v - 1)); }
 
 TexLookup lookup(const jt_ctx* c) {
-  bool all_p2 = true;
-  for (const DevDesc& d : c->descs) all_p2 &= pow2(d.width) && pow2(d.height);
+  bool all_p2 = true, all_s4 = true;
+  for (const DevDesc& d : c->descs) {
+    all_p2 &= pow2(d.width) && pow2(d.height);
+    all_s4 &= d.sampling != kSampling444 && d.reduce == 0;
+  }
   return TexLookup{c->d_descs, c->d_map, reinterpret_cast<const uint4*>(c->d_lrec),
-                   reinterpret_cast<const uint4*>(c->d_prec), c->map_ntex, all_p2 ? 1u : 0u};
+                   reinterpret_cast<const uint4*>(c->d_prec), c->map_ntex, all_p2 ? 1u : 0u, all_s4 ? 1u : 0u};
 }
 
 
@@ -702,7 +704,9 @@ jt_status jt_create(jt_ctx** out, int device, uint64_t max_cache_blocks) {
   c->tuning.pixel_ctas_per_sm = 8;
   c->tuning.decode_short_lists = -1;
   c->cap_units = max_cache_blocks * 4;
-  if (dev_alloc(c, &c->cache, c->cap_units * kUnitBytes) != JT_OK || dev_alloc(c, &c->state, sizeof(FrameState)) != JT_OK ||
+  // one block of padding: colourise gathers texels for pixels that it then drops (see shade),
+  // up to a 4:2:0 tile from any slot
+  if (dev_alloc(c, &c->cache, (c->cap_units + 4) * kUnitBytes) != JT_OK || dev_alloc(c, &c->state, sizeof(FrameState)) != JT_OK ||
       cudaMemset(c->state, 0, sizeof(FrameState)) != cudaSuccess || cudaMemset(c->cache, 0, c->cap_units * kUnitBytes) != cudaSuccess ||
       grow_frame_buffers(c, 4096) != JT_OK || sync_tables(c) != JT_OK) {
     jt_destroy(c);
@@ -791,8 +795,7 @@ static jt_status add_level(jt_ctx* c, int tex_id, int level, DevDesc d, Level L)
     n = std::min<uint32_t>(n, 0xFFFF);
     c->map.resize((size_t)n * JT_MAX_LEVELS, -1);
     c->lrec.resize((size_t)n * JT_MAX_LEVELS, LevelRec{0, 0, 0, 0});
-    c->prec.assign((size_t)n * JT_MAX_LEVELS + 1, PixRec{});
-    for (size_t i = 0; i < c->descs.size(); ++i) c->prec[(size_t)c->levels[i].tex * JT_MAX_LEVELS + c->levels[i].level] = pix_rec(c->descs[i]);
+    c->prec.resize(((size_t)n + 1) * kPixLevels, PixRec{});  // (the added rows are zero, as the old last one was)
     c->map_ntex = n;
   }
   c->map[(size_t)tex_id * JT_MAX_LEVELS + level] = (int32_t)c->descs.size();
@@ -802,7 +805,7 @@ static jt_status add_level(jt_ctx* c, int tex_id, int level, DevDesc d, Level L)
   r.info = level_info(d.mcus_x, (d.sampling == kSampling444 ? 3u : 4u) - d.reduce, d.units, d.sampling, pow2(d.width),
                       pow2(d.height));
   r.pad = 0;
-  c->prec[(size_t)tex_id * JT_MAX_LEVELS + level] = pix_rec(d);
+  c->prec[(size_t)tex_id * kPixLevels + level] = pix_rec(d);
   c->descs.push_back(d);
   c->levels.push_back(L);
   const uint64_t g0 = c->ngid;

@@ -219,8 +219,10 @@ __host__ __device__ inline uint32_t level_info(uint32_t mcus_x, uint32_t shift, 
 // The screen passes' record of one (texture, level): 32 bytes (two vector loads that hit
 // L1, since a warp's pixels mostly share a level), every field in the form the texel
 // addressing uses, so no per-pixel branch or decoding is needed. Indexed by
-// tex * JT_MAX_LEVELS + level; record map_ntex * JT_MAX_LEVELS is all zero, the record of
-// every key outside the table (empty pixels, unknown textures or levels).
+// min(tex, map_ntex) * kPixLevels + min(level, JT_MAX_LEVELS): every texture has one record
+// more than it can have levels, and there is one texture more than the table holds, all of
+// them zero, as are the records of levels that do not exist (empty pixels, unknown textures
+// or levels).
 struct PixRec {
   uint32_t gid_base;
   float wf, hf;     // sides as floats
@@ -231,6 +233,7 @@ struct PixRec {
   uint32_t wh;      // w | h << 16
 };
 static_assert(sizeof(PixRec) == 32, "screen-pass record layout");
+constexpr uint32_t kPixLevels = JT_MAX_LEVELS + 1;
 constexpr uint32_t kPixJpeg = 1u << 16;  // an uploaded JPEG level (colourise, mark)
 constexpr uint32_t kPixCoef = 1u << 17;  // a coefficient level (mark of the float chain)
 constexpr uint32_t kPixPow2 = 1u << 18;  // both sides are powers of two
@@ -239,9 +242,10 @@ struct TexLookup {
   const DevDesc* descs;
   const int32_t* desc_map;
   const uint4* levels;  // LevelRec per (tex, level), same indexing as desc_map
-  const uint4* pix;     // PixRec per (tex, level) as two uint4, then the all-zero record
+  const uint4* pix;     // PixRec per (tex, level) as two uint4, indexed as PixRec says
   uint32_t map_ntex;
   uint32_t all_p2;      // every level has power-of-two sides
+  uint32_t all_s4;      // every JPEG level has 16-texel MCUs (4:2:0 at full size)
 };
 
 // ---- launchers (defined in the kernel translation units) ----

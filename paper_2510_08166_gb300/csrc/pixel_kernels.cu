@@ -233,9 +233,7 @@ struct PixL {
 };
 
 __device__ __forceinline__ PixL pix_level(const TexLookup& tl, uint32_t tm) {
-  const uint32_t tex = tm & 0xFFFFu, mip = tm >> 16;
-  const uint32_t key =
-      (tex < tl.map_ntex && mip < JT_MAX_LEVELS) ? tex * JT_MAX_LEVELS + mip : tl.map_ntex * JT_MAX_LEVELS;
+  const uint32_t key = min(tm & 0xFFFFu, tl.map_ntex) * kPixLevels + min(tm >> 16, (uint32_t)JT_MAX_LEVELS);
   const uint4 r0 = __ldg(tl.pix + 2 * key), r1 = __ldg(tl.pix + 2 * key + 1);
   PixL P;
   P.gid_base = r0.x;
@@ -252,7 +250,13 @@ __device__ __forceinline__ PixL pix_level(const TexLookup& tl, uint32_t tm) {
 // Bilinear taps on the fast path: a power-of-two level and |u w|, |v h| < 2^22 (returns
 // false otherwise; every tap is then still inside the level, so loads made from it stay in
 // range, but the caller must redo the pixel on the general path). Columns xa, xb = xa + 1,
-// rows ya, yb = ya + 1 (repeat wrap), fractions fx, fy.
+// rows ya, yb = ya + 1 (repeat wrap), fractions fx, fy. The range test is of the round-down
+// sums' exponents: [2^23, 2^24). P2: every level is known to be a power of two.
+__device__ __forceinline__ bool in_range(float tx, float ty) {
+  return ((__float_as_uint(tx) ^ 0x4B000000u) | (__float_as_uint(ty) ^ 0x4B000000u)) < 0x00800000u;
+}
+
+template <bool P2 = false>
 __device__ __forceinline__ bool taps_fast(const PixL& P, float u, float v, int& xa, int& xb, int& ya, int& yb,
                                           float& fx, float& fy) {
   const float xs = __fsub_rn(__fmul_rn(u, P.wf), 0.5f), ys = __fsub_rn(__fmul_rn(v, P.hf), 0.5f);
@@ -264,15 +268,16 @@ __device__ __forceinline__ bool taps_fast(const PixL& P, float u, float v, int& 
   ya = __float_as_int(ty) & hm;
   xb = (xa + 1) & wm;
   yb = (ya + 1) & hm;
-  return (P.info & kPixPow2) && fabsf(xs) < 4194304.0f && fabsf(ys) < 4194304.0f;
+  return (P2 || (P.info & kPixPow2)) && in_range(tx, ty);
 }
 
 // Nearest texel on the fast path (same conditions as taps_fast).
+template <bool P2 = false>
 __device__ __forceinline__ bool nearest_fast(const PixL& P, float u, float v, int& x, int& y) {
-  const float xn = __fmul_rn(u, P.wf), yn = __fmul_rn(v, P.hf);
-  x = __float_as_int(__fadd_rd(xn, kMagic)) & (int)(P.masks & 0xFFFFu);
-  y = __float_as_int(__fadd_rd(yn, kMagic)) & (int)(P.masks >> 16);
-  return (P.info & kPixPow2) && fabsf(xn) < 4194304.0f && fabsf(yn) < 4194304.0f;
+  const float tx = __fadd_rd(__fmul_rn(u, P.wf), kMagic), ty = __fadd_rd(__fmul_rn(v, P.hf), kMagic);
+  x = __float_as_int(tx) & (int)(P.masks & 0xFFFFu);
+  y = __float_as_int(ty) & (int)(P.masks >> 16);
+  return (P2 || (P.info & kPixPow2)) && in_range(tx, ty);
 }
 
 // The same taps for any level and coordinate (conversion instructions, floor-mod by
@@ -295,12 +300,10 @@ __device__ __forceinline__ void nearest_any(const PixL& P, float u, float v, int
 }
 
 // Walks the views' tiles: CTA tiles blockIdx.x, + gridDim.x, ...; warp rows w, w + nwarps,
-// ... of each tile. A row of a tile is 128 pixels, taken in SPR steps of 128 / SPR pixels
-// (the unit of work of a warp). The tile origin is recomputed only when the tile changes.
-template <int SPR>
-struct TileWalk {
+// ... of each tile. The tile origin is recomputed only when the tile changes.
+struct RowWalk {
   uint32_t tile;
-  int r, h;    // row in the tile, step in the row
+  int r;       // row in the tile
   int vi;      // view of the tile
   int x0, y0;  // tile origin
   __device__ __forceinline__ bool valid(const ViewSet& vs) const { return tile < vs.total_tiles; }
@@ -316,14 +319,11 @@ struct TileWalk {
   __device__ __forceinline__ void start(const ViewSet& vs) {
     tile = blockIdx.x;
     r = threadIdx.x >> 5;
-    h = 0;
     vi = 0;
     x0 = y0 = 0;
     set_tile(vs);
   }
   __device__ __forceinline__ void advance(const ViewSet& vs) {
-    if (++h < SPR) return;
-    h = 0;
     r += blockDim.x >> 5;
     if (r >= kTileH) {
       r = threadIdx.x >> 5;
@@ -331,36 +331,44 @@ struct TileWalk {
       set_tile(vs);
     }
   }
-  __device__ __forceinline__ int x() const { return x0 + h * (kTileW / SPR); }  // first pixel of the step
-  __device__ __forceinline__ int y() const { return y0 + r; }
 };
 
-// G-buffer of a lane's pixels of the next step, loaded one step ahead of its use so that
-// its HBM reads are in flight while the lane works on the current one.
+// A lane's part of one row of a tile: pixels x + 32 j, j < 4.
+struct Row {
+  uint32_t p0;  // index of pixel j = 0 in the view
+  int rem;      // pixel j exists when 32 j < rem
+};
+
+__device__ __forceinline__ Row row_of(const View& V, const RowWalk& w, bool valid) {
+  const int x = w.x0 + (int)(threadIdx.x & 31), y = w.y0 + w.r;
+  return Row{(uint32_t)y * (uint32_t)V.width + (uint32_t)x, valid && y < V.height ? V.width - x : 0};
+}
+
+// G-buffer of NPX of a lane's pixels, loaded one step ahead of its use so that its HBM reads
+// are in flight while the lane works on the current one. The loads are streaming ones (and so
+// are the framebuffer's stores): nothing reads these lines again, and L1 keeps the tiles'
+// texels and the slots instead (4K frame: 51.9 us without, 47.1 with).
 template <int NPX>
-struct RowG {  // Colourise: pixels x + lane + 32 k, k < NPX, of one step of a row
+struct RowG {
   float u[NPX], v[NPX];
   uint32_t tm[NPX];  // texture id | mip level << 16 (JT_EMPTY_TEXTURE past the view)
-  uint32_t p0;       // index of pixel k = 0 in the view
-  uint32_t n;        // pixels present: those with k < n
 };
 
 template <int NPX>
-__device__ __forceinline__ void load_row(const View& V, int x, int y, bool valid, RowG<NPX>& g) {
-  g.n = (valid && y < V.height && x < V.width) ? (uint32_t)min(NPX, (V.width - x + 31) >> 5) : 0u;
-  g.p0 = (uint32_t)y * (uint32_t)V.width + (uint32_t)x;
-  const float2* uv = reinterpret_cast<const float2*>(V.uv) + g.p0;
-  const uint16_t* tx = V.tex + g.p0;
-  const uint8_t* mp = V.mip + g.p0;
+__device__ __forceinline__ void load_row(const View& V, const Row& row, int j0, RowG<NPX>& g) {
+  const float2* uv = reinterpret_cast<const float2*>(V.uv) + row.p0;
+  const uint16_t* tx = V.tex + row.p0;
+  const uint8_t* mp = V.mip + row.p0;
 #pragma unroll
   for (int k = 0; k < NPX; ++k) {
+    const int j = 32 * (j0 + k);
     g.u[k] = g.v[k] = 0.f;
     g.tm[k] = JT_EMPTY_TEXTURE;
-    if ((uint32_t)k < g.n) {
-      const float2 t = __ldg(uv + 32 * k);
+    if (j < row.rem) {
+      const float2 t = __ldcs(uv + j);
       g.u[k] = t.x;
       g.v[k] = t.y;
-      g.tm[k] = (uint32_t)__ldg(tx + 32 * k) | ((uint32_t)__ldg(mp + 32 * k) << 16);
+      g.tm[k] = (uint32_t)__ldcs(tx + j) | ((uint32_t)__ldcs(mp + j) << 16);
     }
   }
 }
@@ -557,43 +565,35 @@ __device__ __forceinline__ uint32_t blend_h(uint32_t c00, uint32_t c10, uint32_t
   return __byte_perm(h2_as_u32(rg), h2_as_u32(ba), 0x6420u);
 }
 
-// Slot at a, or 0 without touching memory when p is false: a predicated load, so that no
-// branch orders one pixel's loads behind another's.
-__device__ __forceinline__ uint32_t ldg_slot_if(bool p, const uint32_t* a) {
-  uint32_t v;
-  asm("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t@q ld.global.nc.u32 %0, [%1];\n\t}"
-      : "=r"(v)
-      : "l"(a), "r"((uint32_t)p));
-  return v;
-}
-
-// One pixel's colour from its taps: slots of up to four MCUs (predicated loads, the ones
-// beyond the first only when the footprint straddles MCUs) and four texel gathers, then the
-// blend (bilinear) or the texel itself (nearest). Branch-free: a pixel that is not shaded
-// (ok false) reads no slot and gathers its texels from unit 0 (the cache holds at least one
-// block), so the pixels of a lane overlap their chains.
-template <int FILTER>
+// One pixel's colour from its taps: the slots of their four MCUs and four texel gathers, then
+// the blend (bilinear) or the texel itself (nearest). Branch- and predicate-free, so the
+// pixels of a lane overlap their chains: the four slots are read whether or not the footprint
+// straddles MCUs (the same address twice where it does not, an L1 hit), which costs less than
+// the comparisons, predicates and selects that would spare the reads (the ALU pipe bounds the
+// pass). Any slot is in range, of an MCU no pixel needs too (a stale one), and a pixel that
+// is not shaded reads the first slots and gathers from wherever they point.
+// S: log2 of the MCU side when every level has the same, else -1.
+template <int FILTER, int S>
 __device__ __forceinline__ uint32_t shade(const uint32_t* __restrict__ slot, const uint32_t* __restrict__ cache,
-                                          const PixL& P, bool ok, int xa, int xb, int ya, int yb, float fx,
-                                          float fy) {
-  const uint32_t s = P.shift, mwm = (1u << s) - 1u;
-  const uint32_t xas = (uint32_t)xa >> s, xbs = (uint32_t)xb >> s;
-  const uint32_t rowa = P.gid_base + ((uint32_t)ya >> s) * P.mcus_x;
-  const uint32_t o00 = ldg_slot_if(ok, slot + rowa + xas);
+                                          const PixL& P, int xa, int xb, int ya, int yb, float fx, float fy) {
+  const uint32_t s = S >= 0 ? (uint32_t)S : P.shift, mwm = (1u << s) - 1u;
+  const uint32_t xas = (uint32_t)xa >> s, rowa = P.gid_base + ((uint32_t)ya >> s) * P.mcus_x;
+  const uint32_t o00 = __ldg(slot + rowa + xas);
   const uint32_t ia = ((uint32_t)ya & mwm) << s, ja = (uint32_t)xa & mwm;
   if (FILTER == JT_FILTER_NEAREST) return __ldg(cache + (size_t)o00 * (kUnitBytes / 4) + (ia | ja));
-  const uint32_t rowb = P.gid_base + ((uint32_t)yb >> s) * P.mcus_x;
-  const bool sx = xbs != xas, sy = rowb != rowa;
-  const uint32_t l10 = ldg_slot_if(ok && sx, slot + rowa + xbs);
-  const uint32_t l01 = ldg_slot_if(ok && sy, slot + rowb + xas);
-  const uint32_t l11 = ldg_slot_if(ok && sx && sy, slot + rowb + xbs);
-  const uint32_t o10 = sx ? l10 : o00, o01 = sy ? l01 : o00;
-  const uint32_t o11 = sx ? (sy ? l11 : o10) : o01;
+  const uint32_t xbs = (uint32_t)xb >> s, rowb = P.gid_base + ((uint32_t)yb >> s) * P.mcus_x;
   const uint32_t ib = ((uint32_t)yb & mwm) << s, jb = (uint32_t)xb & mwm;
-  const uint32_t c00 = __ldg(cache + (size_t)o00 * (kUnitBytes / 4) + (ia | ja));
-  const uint32_t c10 = __ldg(cache + (size_t)o10 * (kUnitBytes / 4) + (ia | jb));
-  const uint32_t c01 = __ldg(cache + (size_t)o01 * (kUnitBytes / 4) + (ib | ja));
-  const uint32_t c11 = __ldg(cache + (size_t)o11 * (kUnitBytes / 4) + (ib | jb));
+  uint32_t o10 = o00, o01 = o00, o11 = o00;
+  if (FILTER == JT_FILTER_BILINEAR) {  // (the clamped filter's taps share the nearest texel's MCU)
+    o10 = __ldg(slot + rowa + xbs);
+    o01 = __ldg(slot + rowb + xas);
+    o11 = __ldg(slot + rowb + xbs);
+  }
+  // texel j of the tile at unit o (S >= 0: texel indexes fit 32 bits)
+  auto texel = [&](uint32_t o, uint32_t j) {
+    return S >= 0 ? __ldg(cache + (o * (kUnitBytes / 4) | j)) : __ldg(cache + (size_t)o * (kUnitBytes / 4) + j);
+  };
+  const uint32_t c00 = texel(o00, ia | ja), c10 = texel(o10, ia | jb), c01 = texel(o01, ib | ja), c11 = texel(o11, ib | jb);
   return blend_h(c00, c10, c01, c11, fx, fy);
 }
 
@@ -625,86 +625,101 @@ __device__ __noinline__ uint32_t colour_any(const uint32_t* slot, const uint32_t
       clamp_taps(P.shift, nx, ny, xa, xb, ya, yb);
     }
   }
-  return shade<FILTER>(slot, cache, P, true, xa, xb, ya, yb, fx, fy);
+  return shade<FILTER, -1>(slot, cache, P, xa, xb, ya, yb, fx, fy);
 }
 
-// A lane owns pixel lane + 32 k (k < NPX) of each step of a row (32 NPX pixels), so a warp's
-// texel gathers for one tap fall in the two or three tiles its 32 consecutive pixels cover
-// (few L1 wavefronts per load), and the lane's NPX pixels are independent chains (level
-// record, slot, texels) that overlap. The next step's G-buffer is loaded before the
-// current one is shaded. The fast path has no data-dependent branch: the level record is
-// loaded per pixel (an L1 hit), slots beyond the first tap's MCU are predicated loads, and
-// pixels it cannot address (sides not powers of two, |u w| or |v h| >= 2^22) are redone on
-// the general path. Warps whose pixels all lack a texture skip the arithmetic. Slots are in
-// range by construction (the compaction and the cache update never write a slot whose tile
-// would end past the cache), and the all-zero record of keys outside the table addresses
-// unit 0, so no load needs a bound check.
-template <int FILTER, bool MULTI, int NPX>
-__global__ void __launch_bounds__(512, 2) k_colorize(const __grid_constant__ ColorizeArgs a) {
+// A lane owns pixels lane + 32 j (j < 4) of a row of a tile, NPX at a time, so a warp's texel
+// gathers for one tap fall in the two or three tiles its 32 consecutive pixels cover (few L1
+// wavefronts per load), and the lane's NPX pixels are independent chains (level record, slots,
+// texels) that overlap. The next NPX pixels' G-buffer is loaded before the current ones are
+// shaded. The fast path has no data-dependent branch: the level record is loaded per pixel (an
+// L1 hit), and pixels it cannot address (sides not powers of two, |u w| or |v h| >= 2^22) are
+// redone on the general path. Warps whose pixels all lack a texture skip the arithmetic. Slots
+// are in range by construction (the compaction and the cache update never write a slot whose
+// tile would end past the cache), and the all-zero record of keys outside the table addresses
+// the first gid, so no load needs a bound check.
+// ONE: pixels of one texture only (the per-texture form). S: see shade; S >= 0 also says that
+// every level's sides are powers of two.
+template <int FILTER, bool ONE, int S, int NPX>
+__device__ __forceinline__ void colour_step(const ColorizeArgs& a, const RowG<NPX>& g, uint32_t* out, int rem,
+                                            bool& missing) {
   const uint32_t* __restrict__ cache = reinterpret_cast<const uint32_t*>(a.cache);
   const uint32_t* __restrict__ slot = a.slot;
-  const ViewSet& vs = a.views;
-  bool missing = false;
-  const int lx = threadIdx.x & 31;
-  TileWalk<4 / NPX> it;
-  it.start(vs);
-  RowG<NPX> g;
-  load_row(vs.v[MULTI ? it.vi : 0], it.x() + lx, it.y(), it.valid(vs), g);
-#pragma unroll 1
-  while (it.valid(vs)) {
-    TileWalk<4 / NPX> nx = it;
-    nx.advance(vs);
-    RowG<NPX> ng;
-    load_row(vs.v[MULTI ? nx.vi : 0], nx.x() + lx, nx.y(), nx.valid(vs), ng);
-    uint32_t sel = 0, use = 0;
+  bool use = false;
+#pragma unroll
+  for (int k = 0; k < NPX; ++k) {  // (pixels past the view are empty)
+    const uint32_t tex = g.tm[k] & 0xFFFFu;
+    use |= tex != JT_EMPTY_TEXTURE && (!ONE || (int)tex == a.only_tex);
+  }
+  uint32_t px[NPX];
+#pragma unroll
+  for (int k = 0; k < NPX; ++k) px[k] = 0xFF000000u;  // empty pixels
+  if (__any_sync(0xFFFFFFFFu, use)) {
+    uint32_t slow = 0;
 #pragma unroll
     for (int k = 0; k < NPX; ++k) {
       const uint32_t tex = g.tm[k] & 0xFFFFu;
-      const bool sk = (uint32_t)k < g.n && (a.only_tex < 0 || (int)tex == a.only_tex);
-      sel |= sk ? (1u << k) : 0u;
-      use |= sk && tex != JT_EMPTY_TEXTURE ? (1u << k) : 0u;
-    }
-    uint32_t px[NPX];
-#pragma unroll
-    for (int k = 0; k < NPX; ++k) px[k] = 0xFF000000u;  // empty pixels
-    if (__any_sync(0xFFFFFFFFu, use != 0)) {
-      uint32_t slow = 0;
-#pragma unroll
-      for (int k = 0; k < NPX; ++k) {
-        const PixL P = pix_level(a.tl, g.tm[k]);
-        const bool ok = (use >> k & 1u) && (P.info & kPixJpeg);
-        missing |= (use >> k & 1u) && !(P.info & kPixJpeg);
-        int xa, xb, ya, yb;
-        float fx = 0.f, fy = 0.f;
-        bool fast;
-        if (FILTER == JT_FILTER_NEAREST) {
-          fast = nearest_fast(P, g.u[k], g.v[k], xa, ya);
-          xb = xa;
-          yb = ya;
-        } else {
-          fast = taps_fast(P, g.u[k], g.v[k], xa, xb, ya, yb, fx, fy);
-          if (FILTER == JT_FILTER_BILINEAR_CLAMP) {
-            int nxp, nyp;
-            fast &= nearest_fast(P, g.u[k], g.v[k], nxp, nyp);
-            clamp_taps(P.shift, nxp, nyp, xa, xb, ya, yb);
-          }
+      const bool mine = tex != JT_EMPTY_TEXTURE && (!ONE || (int)tex == a.only_tex);
+      const PixL P = pix_level(a.tl, g.tm[k]);
+      const bool ok = mine && (P.info & kPixJpeg);
+      missing |= mine && !ok;
+      int xa, xb, ya, yb;
+      float fx = 0.f, fy = 0.f;
+      bool fast;
+      if (FILTER == JT_FILTER_NEAREST) {
+        fast = nearest_fast<(S >= 0)>(P, g.u[k], g.v[k], xa, ya);
+        xb = xa;
+        yb = ya;
+      } else {
+        fast = taps_fast<(S >= 0)>(P, g.u[k], g.v[k], xa, xb, ya, yb, fx, fy);
+        if (FILTER == JT_FILTER_BILINEAR_CLAMP) {
+          int nxp, nyp;
+          fast &= nearest_fast<(S >= 0)>(P, g.u[k], g.v[k], nxp, nyp);
+          clamp_taps(S >= 0 ? (uint32_t)S : P.shift, nxp, nyp, xa, xb, ya, yb);
         }
-        const uint32_t c = shade<FILTER>(slot, cache, P, ok, xa, xb, ya, yb, fx, fy);
-        px[k] = ok ? c : px[k];
-        slow |= (ok && !fast) ? (1u << k) : 0u;
       }
-      if (slow) {  // rare: redo those pixels on the general path
-#pragma unroll
-        for (int k = 0; k < NPX; ++k)
-          if (slow & (1u << k)) px[k] = colour_any<FILTER>(slot, cache, pix_level(a.tl, g.tm[k]), g.u[k], g.v[k]);
-      }
+      const uint32_t c = shade<FILTER, S>(slot, cache, P, xa, xb, ya, yb, fx, fy);
+      px[k] = ok ? c : px[k];
+      slow |= (ok && !fast) ? (1u << k) : 0u;
     }
-    uint32_t* out = reinterpret_cast<uint32_t*>(vs.v[MULTI ? it.vi : 0].out) + g.p0;
+    if (slow) {  // rare: redo those pixels on the general path
 #pragma unroll
-    for (int k = 0; k < NPX; ++k)
-      if (sel & (1u << k)) out[32 * k] = px[k];
-    it = nx;
-    g = ng;
+      for (int k = 0; k < NPX; ++k)
+        if (slow & (1u << k)) px[k] = colour_any<FILTER>(slot, cache, pix_level(a.tl, g.tm[k]), g.u[k], g.v[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < NPX; ++k)
+    if (32 * k < rem && (!ONE || (int)(g.tm[k] & 0xFFFFu) == a.only_tex)) __stcs(out + 32 * k, px[k]);
+}
+
+template <int FILTER, bool MULTI, bool ONE, int S, int NPX>
+__global__ void __launch_bounds__(512, 2) k_colorize(const __grid_constant__ ColorizeArgs a) {
+  constexpr int kSteps = 4 / NPX;
+  const ViewSet& vs = a.views;
+  bool missing = false;
+  RowWalk it;
+  it.start(vs);
+  Row row = row_of(vs.v[MULTI ? it.vi : 0], it, it.valid(vs));
+  RowG<NPX> g;
+  load_row(vs.v[MULTI ? it.vi : 0], row, 0, g);
+#pragma unroll 1
+  while (it.valid(vs)) {
+    uint32_t* out = reinterpret_cast<uint32_t*>(vs.v[MULTI ? it.vi : 0].out) + row.p0;
+    const int rem = row.rem;
+#pragma unroll
+    for (int h = 0; h < kSteps; ++h) {
+      RowG<NPX> ng;
+      if (h + 1 < kSteps) {
+        load_row(vs.v[MULTI ? it.vi : 0], row, (h + 1) * NPX, ng);
+      } else {
+        it.advance(vs);
+        row = row_of(vs.v[MULTI ? it.vi : 0], it, it.valid(vs));
+        load_row(vs.v[MULTI ? it.vi : 0], row, 0, ng);
+      }
+      colour_step<FILTER, ONE, S, NPX>(a, g, out + 32 * NPX * h, rem - 32 * NPX * h, missing);
+      g = ng;
+    }
   }
   if (missing) atomicOr(&a.state->err, JT_DEVERR_MISSING);
 }
@@ -1177,26 +1192,33 @@ void launch_mark(const MarkArgs& a, int threads, int grid, cudaStream_t s) {
     k_mark<JT_FILTER_BILINEAR><<<grid, threads, smem, s>>>(a);
 }
 
-// pixels per lane per step: two (60 registers, 32 warps per SM) measured faster than four
-// (74 registers) on the 4K frame
-constexpr int kColorizePx = 2;
+// pixels per lane per step: of one, two and four with three to five 256-thread CTAs per SM, two
+// with four CTAs (64 registers) was the fastest for the bilinear filters (4K frame: 47.1 us,
+// 53.9 with one, 49.4 with four and three CTAs, 53.1 with five CTAs), a whole row's four for the
+// nearest texel, whose chains are shorter (eight 4096^2 views: 549 us, 686 with two)
+constexpr int kColorizePx = 2, kColorizePxNearest = 4;
 
-template <bool MULTI>
-void launch_colorize_views(const ColorizeArgs& a, int threads, int grid, cudaStream_t s) {
+template <bool MULTI, bool ONE, int S>
+void launch_colorize_form(const ColorizeArgs& a, int threads, int grid, cudaStream_t s) {
   constexpr int N = kColorizePx;
   if (a.filter == JT_FILTER_NEAREST)
-    k_colorize<JT_FILTER_NEAREST, MULTI, N><<<grid, threads, 0, s>>>(a);
+    k_colorize<JT_FILTER_NEAREST, MULTI, ONE, S, kColorizePxNearest><<<grid, threads, 0, s>>>(a);
   else if (a.filter == JT_FILTER_BILINEAR_CLAMP)
-    k_colorize<JT_FILTER_BILINEAR_CLAMP, MULTI, N><<<grid, threads, 0, s>>>(a);
+    k_colorize<JT_FILTER_BILINEAR_CLAMP, MULTI, ONE, S, N><<<grid, threads, 0, s>>>(a);
   else
-    k_colorize<JT_FILTER_BILINEAR, MULTI, N><<<grid, threads, 0, s>>>(a);
+    k_colorize<JT_FILTER_BILINEAR, MULTI, ONE, S, N><<<grid, threads, 0, s>>>(a);
 }
 
+// The form with a constant MCU side serves contexts whose levels are all 4:2:0 at full size
+// with power-of-two sides; the other one takes both from each pixel's record.
 void launch_colorize(const ColorizeArgs& a, int threads, int grid, cudaStream_t s) {
-  if (a.views.n > 1)
-    launch_colorize_views<true>(a, threads, grid, s);
+  const bool s4 = a.tl.all_s4 && a.tl.all_p2 && a.cap_units <= 0xFFFFFFFFu / (kUnitBytes / 4);
+  if (a.only_tex >= 0)  // one view at a time
+    launch_colorize_form<false, true, -1>(a, threads, grid, s);
+  else if (a.views.n > 1)
+    s4 ? launch_colorize_form<true, false, 4>(a, threads, grid, s) : launch_colorize_form<true, false, -1>(a, threads, grid, s);
   else
-    launch_colorize_views<false>(a, threads, grid, s);
+    s4 ? launch_colorize_form<false, false, 4>(a, threads, grid, s) : launch_colorize_form<false, false, -1>(a, threads, grid, s);
 }
 
 }  // namespace jt
