@@ -1052,8 +1052,8 @@ jt_status jt_raster_scene(jt_ctx* c, const jt_scene* sc, const jt_gbuffer* out, 
       return fail(c, JT_ERR_INVALID_ARG, "quad %d names texture %d", n, sc->quads[n].tex);
   DeviceGuard dg(c->device);
   if (!dg.ok) return fail(c, JT_ERR_CUDA, "cannot select device %d", c->device);
-  // device copies of the texture table and the quads: [w][h][levels] x ntex, then quads
-  const size_t tbytes = (size_t)sc->ntex * 4, qoff = (3 * tbytes + 15) & ~(size_t)15;
+  // device copies of the texture table ([w, h, levels] as 16-byte records) and the quads
+  const size_t qoff = (size_t)sc->ntex * 16;
   const size_t need = qoff + (size_t)sc->nquads * sizeof(SceneQuad);
   if (need > c->raster_cap) {
     dev_free(c->raster_buf);
@@ -1064,12 +1064,15 @@ jt_status jt_raster_scene(jt_ctx* c, const jt_scene* sc, const jt_gbuffer* out, 
     c->raster_cap = need;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  JT_CUDA(c, cudaMemcpyAsync(c->raster_buf, sc->tex_w, tbytes, cudaMemcpyHostToDevice, st));
-  JT_CUDA(c, cudaMemcpyAsync(c->raster_buf + tbytes, sc->tex_h, tbytes, cudaMemcpyHostToDevice, st));
-  JT_CUDA(c, cudaMemcpyAsync(c->raster_buf + 2 * tbytes, sc->tex_levels, tbytes, cudaMemcpyHostToDevice, st));
-  if (sc->nquads)
-    JT_CUDA(c, cudaMemcpyAsync(c->raster_buf + qoff, sc->quads, (size_t)sc->nquads * sizeof(SceneQuad),
-                               cudaMemcpyHostToDevice, st));
+  // one copy of them all (pageable memory is staged before the call returns)
+  std::vector<uint8_t> host(need);
+  for (int t = 0; t < sc->ntex; ++t) {
+    const float wh[2] = {(float)sc->tex_w[t], (float)sc->tex_h[t]};
+    std::memcpy(host.data() + (size_t)t * 16, wh, 8);
+    std::memcpy(host.data() + (size_t)t * 16 + 8, &sc->tex_levels[t], 4);
+  }
+  if (sc->nquads) std::memcpy(host.data() + qoff, sc->quads, (size_t)sc->nquads * sizeof(SceneQuad));
+  JT_CUDA(c, cudaMemcpyAsync(c->raster_buf, host.data(), need, cudaMemcpyHostToDevice, st));
   RasterArgs a{};
   a.width = sc->width;
   a.height = sc->height;
@@ -1085,11 +1088,10 @@ jt_status jt_raster_scene(jt_ctx* c, const jt_scene* sc, const jt_gbuffer* out, 
   a.shift = sc->shift;
   a.cell_seed = sc->cell_seed;
   a.ntex = sc->ntex;
+  a.mod_m = sc->ntex == 1 ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / (uint64_t)sc->ntex);
   a.use_mips = sc->use_mips;
   a.nquads = sc->nquads;
-  a.tex_w = reinterpret_cast<const int32_t*>(c->raster_buf);
-  a.tex_h = reinterpret_cast<const int32_t*>(c->raster_buf + tbytes);
-  a.tex_levels = reinterpret_cast<const int32_t*>(c->raster_buf + 2 * tbytes);
+  a.sizes = reinterpret_cast<const float4*>(c->raster_buf);
   a.quads = reinterpret_cast<const SceneQuad*>(c->raster_buf + qoff);
   // the G-buffer record is declared read-only for the passes that consume it; here it is
   // the output

@@ -321,10 +321,10 @@ struct RasterArgs {
   float ax, ay, tan_x, tan_y, max_t, kx, ky, shift;
   uint64_t cell_seed;
   int32_t ntex, use_mips, nquads;
-  const int32_t* tex_w;       // device copies
-  const int32_t* tex_h;
-  const int32_t* tex_levels;
-  const SceneQuad* quads;
+  int32_t tile_x;             // columns of a CTA's tile (chosen by the launcher)
+  uint32_t mod_m;             // floor(2^32 / ntex), or 2^32 - 1 for one texture
+  const float4* sizes;        // device copies: per texture its level-0 sides and (bits of) its level count,
+  const SceneQuad* quads;     // then the quads
   float2* uv;
   uint16_t* tex;
   uint8_t* mip;
