@@ -408,7 +408,7 @@ jt_status jt_colorize_float(jt_ctx* ctx, const jt_gbuffer* g, const float* coeff
  * overwritten: zero except for the MCUs the frame touches. Recomputes the needed set
  * from the G-buffer; stores no decoded blocks and no per-texel gradients: the view's
  * pixels are bucketed under the MCUs their taps touch and each MCU gathers its bucket.
- * The bucket array (four 32-byte entries per pixel of the view) is grown on the first call
+ * The bucket array (four 16-byte entries per pixel of the view) is grown on the first call
  * with a larger view, which synchronises the stream once. */
 jt_status jt_colorize_backward(jt_ctx* ctx, const jt_gbuffer* g, const float* grad_frame, float* grad_coeffs,
                                jt_stream stream);

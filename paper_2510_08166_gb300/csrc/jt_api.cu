@@ -51,11 +51,8 @@ struct jt_ctx {
   uint32_t* d_desc_of_gid = nullptr;  // descriptor index of every gid (the decoder's lookup)
   uint64_t desc_of_gid_cap = 0;
   std::vector<int32_t> map;  // [map_ntex * 16]
-  std::vector<LevelRec> lrec;  // [map_ntex * 16]
   std::vector<PixRec> prec;    // [(map_ntex + 1) * kPixLevels]
   uint32_t map_ntex = 0;
-  int32_t* d_map = nullptr;
-  LevelRec* d_lrec = nullptr;
   PixRec* d_prec = nullptr;
   std::vector<std::vector<HuffSet>> hsets;            // one set each
   std::vector<std::vector<jt_huff_spec>> huff_specs;  // the specs of each set, unused values zeroed
@@ -89,10 +86,10 @@ struct jt_ctx {
   int coef_first = -1, coef_count = 0, coef_w = 0, coef_h = 0;
   uint32_t coef_gid_base = 0;
   uint32_t float_tile_cap = 0;     // needed coefficient MCUs a float pass can serve
-  uint32_t* bucket_cnt = nullptr;   // [float_tile_cap + 1], cleared at the start of each backward call
-  uint32_t* bucket_off = nullptr;   // [float_tile_cap + 1]
-  uint32_t* bucket_bsum = nullptr;  // one per kBucketScan counts
-  uint32_t* bucket = nullptr;       // [bucket_cap] 32-byte entries
+  uint32_t* float_cursor = nullptr;   // [coefficient MCUs], zero between passes
+  uint32_t* float_offset = nullptr;   // [coefficient MCUs]
+  uint64_t* float_sums = nullptr;     // one per kFloatScan counts
+  uint4* bucket = nullptr;            // [bucket_cap] entries
   uint64_t bucket_cap = 0;
   cudaStream_t capture_stream = nullptr;
 
@@ -317,19 +314,11 @@ jt_status sync_descs(jt_ctx* c) {
     c->d_descs_cap = cap;
   }
   JT_CUDA(c, cudaMemcpy(c->d_descs, c->descs.data(), c->descs.size() * sizeof(DevDesc), cudaMemcpyHostToDevice));
-  dev_free(c->d_map);
-  dev_free(c->d_lrec);
-  jt_status s = dev_alloc(c, &c->d_map, c->map.size() * 4);
-  if (s != JT_OK) return s;
-  if ((s = dev_alloc(c, &c->d_lrec, c->lrec.size() * sizeof(LevelRec))) != JT_OK) return s;
   dev_free(c->d_prec);
   c->prec.resize(((size_t)c->map_ntex + 1) * kPixLevels, PixRec{});
-  if ((s = dev_alloc(c, &c->d_prec, c->prec.size() * sizeof(PixRec))) != JT_OK) return s;
+  jt_status s = dev_alloc(c, &c->d_prec, c->prec.size() * sizeof(PixRec));
+  if (s != JT_OK) return s;
   JT_CUDA(c, cudaMemcpy(c->d_prec, c->prec.data(), c->prec.size() * sizeof(PixRec), cudaMemcpyHostToDevice));
-  if (!c->map.empty()) {
-    JT_CUDA(c, cudaMemcpy(c->d_map, c->map.data(), c->map.size() * 4, cudaMemcpyHostToDevice));
-    JT_CUDA(c, cudaMemcpy(c->d_lrec, c->lrec.data(), c->lrec.size() * sizeof(LevelRec), cudaMemcpyHostToDevice));
-  }
   return JT_OK;
 }
 
@@ -369,8 +358,7 @@ TexLookup lookup(const jt_ctx* c) {
     all_p2 &= pow2(d.width) && pow2(d.height);
     all_s4 &= d.sampling != kSampling444 && d.reduce == 0;
   }
-  return TexLookup{c->d_descs, c->d_map, reinterpret_cast<const uint4*>(c->d_lrec),
-                   reinterpret_cast<const uint4*>(c->d_prec), c->map_ntex, all_p2 ? 1u : 0u, all_s4 ? 1u : 0u};
+  return TexLookup{reinterpret_cast<const uint4*>(c->d_prec), c->map_ntex, all_p2 ? 1u : 0u, all_s4 ? 1u : 0u};
 }
 
 
@@ -427,7 +415,7 @@ jt_status check_launch(jt_ctx* c, const char* what) {
   return JT_OK;
 }
 
-jt_status enqueue_mark(jt_ctx* c, const ViewSet& vs, int filter, int only_tex, int coef_mode, cudaStream_t s) {
+jt_status enqueue_mark(jt_ctx* c, const ViewSet& vs, int filter, int only_tex, cudaStream_t s) {
   if (c->descs.empty()) return fail(c, JT_ERR_STATE, "no textures uploaded");
   MarkArgs a{};
   a.views = vs;
@@ -436,7 +424,6 @@ jt_status enqueue_mark(jt_ctx* c, const ViewSet& vs, int filter, int only_tex, i
   a.state = c->state;
   a.filter = filter;
   a.only_tex = only_tex;
-  a.coef_mode = coef_mode;
   launch_mark(a, c->tuning.pixel_threads, pixel_grid(c, vs), s);
   return check_launch(c, "mark");
 }
@@ -566,7 +553,7 @@ jt_status enqueue_frame(jt_ctx* c, const ViewSet& vs, int filter, cudaStream_t s
     if (c->profiling) cudaEventRecordWithFlags(c->prof[i], s, rec_flags);
   };
   mark_time(0);
-  if ((st = enqueue_mark(c, vs, filter, -1, 0, s)) != JT_OK) return st;
+  if ((st = enqueue_mark(c, vs, filter, -1, s)) != JT_OK) return st;
   mark_time(1);
   if ((st = enqueue_compact(c, s)) != JT_OK) return st;
   mark_time(2);
@@ -612,9 +599,11 @@ jt_status float_setup(jt_ctx* c, const jt_gbuffer* g, const float* in, const flo
   a.coef_gid_base = c->coef_gid_base;
   a.coef_mcus = (uint32_t)((uint64_t)c->coef_count * (c->coef_w / 16) * (c->coef_h / 16));
   a.tile_cap = c->float_tile_cap;
-  a.bucket_cnt = c->bucket_cnt;
-  a.bucket_off = c->bucket_off;
-  a.bucket_bsum = c->bucket_bsum;
+  a.work_cap = (uint32_t)c->gid_cap;
+  a.cap_units = (uint32_t)c->cap_units;
+  a.cursor = c->float_cursor;
+  a.offset = c->float_offset;
+  a.block_sum = c->float_sums;
   a.state = c->state;
   // orthonormal 8-point DCT-III basis, A[x][u] = C(u)/2 cos((2x+1) u pi / 16)
   const double pi = 3.14159265358979323846;
@@ -624,24 +613,20 @@ jt_status float_setup(jt_ctx* c, const jt_gbuffer* g, const float* in, const flo
   return JT_OK;
 }
 
-// Needed set of the coefficient textures (bilinear taps) and its compaction, then the
-// buckets' room (a pixel's taps touch at most four MCUs; grown, stream-ordered, when a larger
-// view comes) and their zeroed counts.
-jt_status enqueue_float_needed(jt_ctx* c, FloatArgs& a, cudaStream_t st) {
-  jt_status s;
+// The entries' room (a pixel's taps touch at most four MCUs; grown, stream-ordered, when a larger
+// view comes).
+jt_status float_bucket(jt_ctx* c, FloatArgs& a, cudaStream_t st) {
   const uint64_t need = 4ull * a.views.v[0].width * a.views.v[0].height;
   if (need > c->bucket_cap) {
     JT_CUDA(c, cudaStreamSynchronize(st));
     dev_free(c->bucket);
     c->bucket_cap = 0;
-    if ((s = dev_alloc(c, &c->bucket, std::max<uint64_t>(need, 1) * 32)) != JT_OK) return s;
+    jt_status s = dev_alloc(c, &c->bucket, std::max<uint64_t>(need, 1) * sizeof(uint4));
+    if (s != JT_OK) return s;
     c->bucket_cap = need;
   }
   a.bucket = c->bucket;
   a.bucket_cap = (uint32_t)std::min<uint64_t>(c->bucket_cap, 0xFFFFFFFFull);
-  if ((s = enqueue_mark(c, a.views, JT_FILTER_BILINEAR, -1, 1, st)) != JT_OK) return s;
-  if ((s = enqueue_scan(c, c->coef_gid_base, (uint64_t)c->coef_gid_base + a.coef_mcus, st)) != JT_OK) return s;
-  JT_CUDA(c, cudaMemsetAsync(c->bucket_cnt, 0, ((size_t)c->float_tile_cap + 1) * 4, st));
   return JT_OK;
 }
 
@@ -731,8 +716,6 @@ jt_status jt_destroy(jt_ctx* c) {
     if (l.du_mem) cudaFree(l.du_mem);
   }
   dev_free(c->d_descs);
-  dev_free(c->d_map);
-  dev_free(c->d_lrec);
   dev_free(c->d_prec);
   dev_free(c->d_huff);
   dev_free(c->d_quant);
@@ -744,9 +727,9 @@ jt_status jt_destroy(jt_ctx* c) {
   dev_free(c->d_desc_of_gid);
   cache_free(c);
   dev_free(c->state);
-  dev_free(c->bucket_cnt);
-  dev_free(c->bucket_off);
-  dev_free(c->bucket_bsum);
+  dev_free(c->float_cursor);
+  dev_free(c->float_offset);
+  dev_free(c->float_sums);
   dev_free(c->bucket);
   dev_free(c->raster_buf);
   if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
@@ -794,17 +777,10 @@ static jt_status add_level(jt_ctx* c, int tex_id, int level, DevDesc d, Level L)
     uint32_t n = std::max<uint32_t>((uint32_t)tex_id + 1, c->map_ntex * 2);
     n = std::min<uint32_t>(n, 0xFFFF);
     c->map.resize((size_t)n * JT_MAX_LEVELS, -1);
-    c->lrec.resize((size_t)n * JT_MAX_LEVELS, LevelRec{0, 0, 0, 0});
     c->prec.resize(((size_t)n + 1) * kPixLevels, PixRec{});  // (the added rows are zero, as the old last one was)
     c->map_ntex = n;
   }
   c->map[(size_t)tex_id * JT_MAX_LEVELS + level] = (int32_t)c->descs.size();
-  LevelRec& r = c->lrec[(size_t)tex_id * JT_MAX_LEVELS + level];
-  r.gid_base = d.gid_base;
-  r.wh = (uint32_t)d.width | ((uint32_t)d.height << 16);
-  r.info = level_info(d.mcus_x, (d.sampling == kSampling444 ? 3u : 4u) - d.reduce, d.units, d.sampling, pow2(d.width),
-                      pow2(d.height));
-  r.pad = 0;
   c->prec[(size_t)tex_id * kPixLevels + level] = pix_rec(d);
   c->descs.push_back(d);
   c->levels.push_back(L);
@@ -1114,7 +1090,7 @@ jt_status jt_mark(jt_ctx* c, const jt_gbuffer* g, int filter, jt_stream stream) 
   if (s != JT_OK) return s;
   DeviceGuard dg(c->device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if ((s = enqueue_mark(c, vs, filter, -1, 0, st)) != JT_OK) return s;
+  if ((s = enqueue_mark(c, vs, filter, -1, st)) != JT_OK) return s;
   c->phase = Phase::Marked;
   c->last_stream = st;
   return JT_OK;
@@ -1290,7 +1266,7 @@ jt_status jt_frame_plain(jt_ctx* c, const jt_view* views, int nviews, int filter
     if ((s = make_views(c, views + v, 1, true, one)) != JT_OK) return s;
     if ((s = enqueue_colorize(c, one, filter, JT_EMPTY_TEXTURE, st)) != JT_OK) return s;
     for (const auto& kv : ranges) {
-      if ((s = enqueue_mark(c, one, filter, kv.first, 0, st)) != JT_OK) return s;
+      if ((s = enqueue_mark(c, one, filter, kv.first, st)) != JT_OK) return s;
       if ((s = enqueue_scan(c, kv.second.first, kv.second.second, st)) != JT_OK) return s;
       if ((s = enqueue_decode(c, st)) != JT_OK) return s;
       if ((s = enqueue_colorize(c, one, filter, kv.first, st)) != JT_OK) return s;
@@ -1457,11 +1433,16 @@ jt_status jt_register_coeff_textures(jt_ctx* c, int first_tex_id, int count, int
   if (c->ngid + per * count > kMaxGids) return fail(c, JT_ERR_UNSUPPORTED, "more than 2^26 MCUs in one context");
   DeviceGuard dg(c->device);
   if (!dg.ok) return fail(c, JT_ERR_CUDA, "cannot select device %d", c->device);
-  const uint64_t cap = std::min<uint64_t>(per * count, c->cap_units / 4);
+  const uint64_t total = per * count, cap = std::min<uint64_t>(total, c->cap_units / 4);
+  if (!float_configure()) return fail(c, JT_ERR_CUDA, "float kernels: %s", cudaGetErrorString(cudaGetLastError()));
+  dev_free(c->float_cursor);  // (of a registration that failed)
+  dev_free(c->float_offset);
+  dev_free(c->float_sums);
   jt_status s;
-  if ((s = dev_alloc(c, &c->bucket_cnt, (cap + 1) * 4)) != JT_OK) return s;
-  if ((s = dev_alloc(c, &c->bucket_off, (cap + 1) * 4)) != JT_OK) return s;
-  if ((s = dev_alloc(c, &c->bucket_bsum, ((cap + 1 + kBucketScan - 1) / kBucketScan) * 4)) != JT_OK) return s;
+  if ((s = dev_alloc(c, &c->float_cursor, total * 4)) != JT_OK) return s;
+  if ((s = dev_alloc(c, &c->float_offset, total * 4)) != JT_OK) return s;
+  if ((s = dev_alloc(c, &c->float_sums, (total + kFloatScan - 1) / kFloatScan * 8)) != JT_OK) return s;
+  JT_CUDA(c, cudaMemset(c->float_cursor, 0, total * 4));
   c->float_tile_cap = (uint32_t)cap;
   c->coef_gid_base = (uint32_t)c->ngid;
   for (int t = 0; t < count; ++t) {
@@ -1492,9 +1473,9 @@ jt_status jt_colorize_float(jt_ctx* c, const jt_gbuffer* g, const float* coeffs,
   a.frame = out_rgb;
   DeviceGuard dg(c->device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if ((s = enqueue_float_needed(c, a, st)) != JT_OK) return s;
+  if ((s = float_bucket(c, a, st)) != JT_OK) return s;
   JT_CUDA(c, cudaMemsetAsync(out_rgb, 0, (size_t)a.views.v[0].width * a.views.v[0].height * 3 * sizeof(float), st));
-  launch_float_forward(a, c->tuning.pixel_threads, pixel_grid(c, a.views), c->sm_count * 8, st);
+  launch_float_forward(a, c->tuning.pixel_threads, pixel_grid(c, a.views), st);
   if ((s = check_launch(c, "float forward")) != JT_OK) return s;
   c->phase = Phase::Idle;  // the work list now describes coefficient MCUs
   c->last_stream = st;
@@ -1511,8 +1492,8 @@ jt_status jt_colorize_backward(jt_ctx* c, const jt_gbuffer* g, const float* grad
   a.grad_coef = grad_coeffs;
   DeviceGuard dg(c->device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if ((s = enqueue_float_needed(c, a, st)) != JT_OK) return s;
-  launch_float_backward(a, c->tuning.pixel_threads, pixel_grid(c, a.views), c->sm_count * 8, st);
+  if ((s = float_bucket(c, a, st)) != JT_OK) return s;
+  launch_float_backward(a, c->tuning.pixel_threads, pixel_grid(c, a.views), st);
   if ((s = check_launch(c, "float backward")) != JT_OK) return s;
   c->phase = Phase::Idle;
   c->last_stream = st;

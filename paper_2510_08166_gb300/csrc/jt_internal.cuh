@@ -3,7 +3,7 @@
 //
 // HBM layout
 //   descs      DevDesc[ndesc]        one per uploaded (texture, level), sorted by gid_base
-//   desc_map   int32[ntex * 16]      (tex_id, level) -> desc index, -1 when absent
+//   pix        PixRec[(ntex + 1) * 17]  (tex_id, level) -> the screen passes' record
 //   streams    per level: uint32 words of the unstuffed entropy stream + >= 64 zero bytes
 //   index      per level: packed 10-byte {bit_offset, dc_pred[3]} entries
 //   huff       HuffSet[nh]           decode tables, deduplicated by content
@@ -197,25 +197,6 @@ struct ViewSet {
   uint32_t total_tiles;
 };
 
-// Per-(texture, level) record for the screen passes, indexed directly by
-// tex_id * JT_MAX_LEVELS + level; 16 bytes, one vector load. w == 0 marks a missing level.
-//   x: gid_base
-//   y: width (16) | height (16)
-//   z: mcus_x (16) | mcu shift (4: 4 at 4:2:0, 3 at 4:4:4) | units (4) | sampling (4) |
-//      width is a power of two (1) | height is a power of two (1)
-//   w: unused
-struct LevelRec {
-  uint32_t gid_base;
-  uint32_t wh;
-  uint32_t info;
-  uint32_t pad;
-};
-__host__ __device__ inline uint32_t level_info(uint32_t mcus_x, uint32_t shift, uint32_t units, uint32_t sampling,
-                                               bool wpow2, bool hpow2) {
-  return (mcus_x & 0xFFFF) | (shift << 16) | (units << 20) | (sampling << 24) | ((wpow2 ? 1u : 0u) << 28) |
-         ((hpow2 ? 1u : 0u) << 29);
-}
-
 // The screen passes' record of one (texture, level): 32 bytes (two vector loads that hit
 // L1, since a warp's pixels mostly share a level), every field in the form the texel
 // addressing uses, so no per-pixel branch or decoding is needed. Indexed by
@@ -235,13 +216,10 @@ struct PixRec {
 static_assert(sizeof(PixRec) == 32, "screen-pass record layout");
 constexpr uint32_t kPixLevels = JT_MAX_LEVELS + 1;
 constexpr uint32_t kPixJpeg = 1u << 16;  // an uploaded JPEG level (colourise, mark)
-constexpr uint32_t kPixCoef = 1u << 17;  // a coefficient level (mark of the float chain)
+constexpr uint32_t kPixCoef = 1u << 17;  // a coefficient level (the float chain)
 constexpr uint32_t kPixPow2 = 1u << 18;  // both sides are powers of two
 
 struct TexLookup {
-  const DevDesc* descs;
-  const int32_t* desc_map;
-  const uint4* levels;  // LevelRec per (tex, level), same indexing as desc_map
   const uint4* pix;     // PixRec per (tex, level) as two uint4, indexed as PixRec says
   uint32_t map_ntex;
   uint32_t all_p2;      // every level has power-of-two sides
@@ -256,7 +234,6 @@ struct MarkArgs {
   FrameState* state;
   int filter;
   int only_tex;   // -1: all textures; otherwise only pixels with this texture id
-  int coef_mode;  // 0: JPEG levels only; 1: coefficient textures only
 };
 void launch_mark(const MarkArgs& a, int threads, int grid, cudaStream_t s);
 
@@ -363,39 +340,39 @@ struct ColorizeArgs {
 };
 void launch_colorize(const ColorizeArgs& a, int threads, int grid, cudaStream_t s);
 
-// Float chain (differentiable colourise; not in the paper). Coefficient textures are
-// 4:2:0 level-0 textures whose MCUs are marked with 1 unit each, so after the compaction
-// slot[gid] is the MCU's position in the work list and the index of its float tile.
+// Float chain (differentiable colourise; not in the paper; float_kernels.cu). Coefficient
+// textures are 4:2:0 level-0 textures; an MCU is needed when a pixel's taps touch it, and slot[gid]
+// is then its position in the work list.
 struct FloatArgs {
   ViewSet views;          // one view
   TexLookup tl;
-  const uint32_t* slot;   // gid -> work position = float tile index
-  const uint32_t* work;
+  uint32_t* slot;
+  uint32_t* work;
+  uint32_t work_cap;
+  uint32_t cap_units;     // slots stay below it
   const float* coef;      // [T][my][mx][6][64], natural order k = v*8+u
   uint32_t coef_gid_base; // gid of coefficient texture 0, MCU 0
   uint32_t coef_mcus;     // MCUs of all coefficient textures
-  uint32_t tile_cap;      // needed coefficient MCUs a pass can serve (more: JT_DEVERR_CAPACITY)
+  uint32_t tile_cap;      // needed coefficient MCUs a pass serves (more: JT_DEVERR_CAPACITY)
   float* frame;           // [npx][3]: forward output (zero on entry), or the backward's dL/dF
   float* grad_coef;       // [T][my][mx][6][64]: backward output
   FrameState* state;
-  // the view's pixels bucketed under the needed MCUs (work positions) their taps touch
-  uint32_t* bucket_cnt;   // [tile_cap + 1] per-MCU counts, then fill cursors; zero on entry
-  uint32_t* bucket_off;   // [tile_cap + 1] exclusive offsets into bucket
-  uint32_t* bucket_bsum;  // [ceil((tile_cap + 1) / kBucketScan)] per-block sums of the counts
-  uint32_t* bucket;       // [bucket_cap][8]: the pixel's index (forward) or its colour^T terms
-                          // (3 floats, backward), its taps' texels (4 bytes), their weights
-                          // (4 floats, 0 for a tap in another MCU)
-  uint32_t bucket_cap;    // entries, >= 4 pixels of the view (a pixel's taps touch at most 4 MCUs)
+  // the view's pixels bucketed under the coefficient MCUs their taps touch
+  uint32_t* cursor;       // [coef_mcus] counts, then fill cursors; zero between passes
+  uint32_t* offset;       // [coef_mcus] first entry of each MCU
+  uint64_t* block_sum;    // [ceil(coef_mcus / kFloatScan)] needed MCUs << 32 | entries
+  uint4* bucket;          // [bucket_cap] entries
+  uint32_t bucket_cap;    // >= 4 pixels of the view (a pixel's taps touch at most 4 MCUs)
   float basis[64];        // A[x][u] = C(u)/2 cos((2x+1)u pi/16), C(0) = 1/sqrt(2); x*8+u
 };
 // JFIF colour of the float chain: R = Y + kCr2R Cr, G = Y - kCb2G Cb - kCr2G Cr, B = Y + kCb2B Cb
 constexpr float kCr2R = 1.402f, kCb2G = 0.344136f, kCr2G = 0.714136f, kCb2B = 1.772f;
-constexpr int kFloatWarps = 8;     // warps per CTA of the per-MCU float kernels
-constexpr int kBucketScan = 1024;  // counts per CTA of the bucket-offset scan (256 threads x 4)
-// count pass, offsets, fill pass, then the per-MCU gather (forward: weighted texels into the
-// pixels; backward: the adjoint into the coefficients)
-void launch_float_forward(const FloatArgs& a, int threads, int pixel_grid, int mcu_grid, cudaStream_t s);
-void launch_float_backward(const FloatArgs& a, int threads, int pixel_grid, int mcu_grid, cudaStream_t s);
+constexpr int kFloatWarps = 8;     // warps per CTA of the gathers
+constexpr int kForwardPairs = 8, kBackwardPairs = 4;  // pairs of MCUs per warp there (2: 152/152 us, 4: 115/131, 8: 104/140, 16: 107/169)
+constexpr int kFloatScan = 1024;   // counts per CTA of the scan (256 threads x 4)
+bool float_configure();
+void launch_float_forward(const FloatArgs& a, int threads, int pixel_grid, cudaStream_t s);
+void launch_float_backward(const FloatArgs& a, int threads, int pixel_grid, cudaStream_t s);
 
 // The integer IDCT constants the decode kernel is compiled with, for the host-side check
 // against round(8192 cos(k pi / 16)), k = 1..7.
