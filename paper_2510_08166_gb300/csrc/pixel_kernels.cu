@@ -26,6 +26,7 @@
 #include <cuda_runtime.h>
 
 #include <cstring>
+#include <type_traits>
 
 #include "jt_internal.cuh"
 #include "texel.cuh"
@@ -368,14 +369,12 @@ __device__ __noinline__ uint32_t colour_any(const uint32_t* slot, const uint32_t
 // wavefronts per load), and the lane's NPX pixels are independent chains (level record, slots,
 // texels) that overlap. The next NPX pixels' G-buffer is loaded before the current ones are
 // shaded. The fast path has no data-dependent branch: the level record is loaded per pixel (an
-// L1 hit), and pixels it cannot address (sides not powers of two, |u w| or |v h| >= 2^22) are
-// redone on the general path. Warps whose pixels all lack a texture skip the arithmetic. Slots
+// L1 hit), and pixels it cannot address (|u w| or |v h| >= 2^22) are redone on the general path. Warps whose pixels all lack a texture skip the arithmetic. Slots
 // are in range by construction (the compaction and the cache update never write a slot whose
 // tile would end past the cache), and the all-zero record of keys outside the table addresses
 // the first gid, so no load needs a bound check.
-// ONE: pixels of one texture only (the per-texture form). S: see shade; S >= 0 also says that
-// every level's sides are powers of two.
-template <int FILTER, bool ONE, int S, int NPX>
+// ONE: pixels of one texture only (the per-texture form). S: see shade. WRAP covers every level.
+template <int FILTER, bool ONE, int S, Wrap WRAP, int NPX>
 __device__ __forceinline__ void colour_step(const ColorizeArgs& a, const RowG<NPX>& g, uint32_t* out, int rem,
                                             bool& missing) {
   const uint32_t* __restrict__ cache = reinterpret_cast<const uint32_t*>(a.cache);
@@ -402,14 +401,14 @@ __device__ __forceinline__ void colour_step(const ColorizeArgs& a, const RowG<NP
       float fx = 0.f, fy = 0.f;
       bool fast;
       if (FILTER == JT_FILTER_NEAREST) {
-        fast = nearest_fast<(S >= 0)>(P, g.u[k], g.v[k], xa, ya);
+        fast = nearest_fast<WRAP>(P, g.u[k], g.v[k], xa, ya);
         xb = xa;
         yb = ya;
       } else {
-        fast = taps_fast<(S >= 0)>(P, g.u[k], g.v[k], xa, xb, ya, yb, fx, fy);
+        fast = taps_fast<WRAP>(P, g.u[k], g.v[k], xa, xb, ya, yb, fx, fy);
         if (FILTER == JT_FILTER_BILINEAR_CLAMP) {
           int nxp, nyp;
-          fast &= nearest_fast<(S >= 0)>(P, g.u[k], g.v[k], nxp, nyp);
+          fast &= nearest_fast<WRAP>(P, g.u[k], g.v[k], nxp, nyp);
           clamp_taps(S >= 0 ? (uint32_t)S : P.shift, nxp, nyp, xa, xb, ya, yb);
         }
       }
@@ -428,7 +427,7 @@ __device__ __forceinline__ void colour_step(const ColorizeArgs& a, const RowG<NP
     if (32 * k < rem && (!ONE || (int)(g.tm[k] & 0xFFFFu) == a.only_tex)) __stcs(out + 32 * k, px[k]);
 }
 
-template <int FILTER, bool MULTI, bool ONE, int S, int NPX>
+template <int FILTER, bool MULTI, bool ONE, int S, Wrap WRAP, int NPX>
 __global__ void __launch_bounds__(512, 2) k_colorize(const __grid_constant__ ColorizeArgs a) {
   constexpr int kSteps = 4 / NPX;
   const ViewSet& vs = a.views;
@@ -452,7 +451,7 @@ __global__ void __launch_bounds__(512, 2) k_colorize(const __grid_constant__ Col
         row = row_of(vs.v[MULTI ? it.vi : 0], it, it.valid(vs));
         load_row(vs.v[MULTI ? it.vi : 0], row, 0, ng);
       }
-      colour_step<FILTER, ONE, S, NPX>(a, g, out + 32 * NPX * h, rem - 32 * NPX * h, missing);
+      colour_step<FILTER, ONE, S, WRAP, NPX>(a, g, out + 32 * NPX * h, rem - 32 * NPX * h, missing);
       g = ng;
     }
   }
@@ -476,27 +475,36 @@ void launch_mark(const MarkArgs& a, int threads, int grid, cudaStream_t s) {
 // nearest texel, whose chains are shorter (eight 4096^2 views: 549 us, 686 with two)
 constexpr int kColorizePx = 2, kColorizePxNearest = 4;
 
-template <bool MULTI, bool ONE, int S>
+template <bool MULTI, bool ONE, int S, Wrap WRAP>
 void launch_colorize_form(const ColorizeArgs& a, int threads, int grid, cudaStream_t s) {
-  constexpr int N = kColorizePx;
+  constexpr int N = kColorizePx, kNearest = ONE && WRAP == kWrapAny ? N : kColorizePxNearest;  // (four spill there)
   if (a.filter == JT_FILTER_NEAREST)
-    k_colorize<JT_FILTER_NEAREST, MULTI, ONE, S, kColorizePxNearest><<<grid, threads, 0, s>>>(a);
+    k_colorize<JT_FILTER_NEAREST, MULTI, ONE, S, WRAP, kNearest><<<grid, threads, 0, s>>>(a);
   else if (a.filter == JT_FILTER_BILINEAR_CLAMP)
-    k_colorize<JT_FILTER_BILINEAR_CLAMP, MULTI, ONE, S, N><<<grid, threads, 0, s>>>(a);
+    k_colorize<JT_FILTER_BILINEAR_CLAMP, MULTI, ONE, S, WRAP, N><<<grid, threads, 0, s>>>(a);
   else
-    k_colorize<JT_FILTER_BILINEAR, MULTI, ONE, S, N><<<grid, threads, 0, s>>>(a);
+    k_colorize<JT_FILTER_BILINEAR, MULTI, ONE, S, WRAP, N><<<grid, threads, 0, s>>>(a);
 }
 
 // The form with a constant MCU side serves contexts whose levels are all 4:2:0 at full size
-// with power-of-two sides; the other one takes both from each pixel's record.
+// with power-of-two sides; the other ones take it from each pixel's record, and a context
+// with any other sides wraps by a remainder (twelve textures of odd sides in a 1367 x 769 frame,
+// the three calls: 63.0 us with every pixel on the general path, 55.6 so).
 void launch_colorize(const ColorizeArgs& a, int threads, int grid, cudaStream_t s) {
   const bool s4 = a.tl.all_s4 && a.tl.all_p2 && a.cap_units <= 0xFFFFFFFFu / (kUnitBytes / 4);
+  auto form = [&](auto multi) {
+    constexpr bool M = decltype(multi)::value;
+    s4 ? launch_colorize_form<M, false, 4, kWrapPow2>(a, threads, grid, s)
+       : a.tl.all_p2 ? launch_colorize_form<M, false, -1, kWrapPow2>(a, threads, grid, s)
+                     : launch_colorize_form<M, false, -1, kWrapAny>(a, threads, grid, s);
+  };
   if (a.only_tex >= 0)  // one view at a time
-    launch_colorize_form<false, true, -1>(a, threads, grid, s);
+    a.tl.all_p2 ? launch_colorize_form<false, true, -1, kWrapPow2>(a, threads, grid, s)
+                : launch_colorize_form<false, true, -1, kWrapAny>(a, threads, grid, s);
   else if (a.views.n > 1)
-    s4 ? launch_colorize_form<true, false, 4>(a, threads, grid, s) : launch_colorize_form<true, false, -1>(a, threads, grid, s);
+    form(std::true_type{});
   else
-    s4 ? launch_colorize_form<false, false, 4>(a, threads, grid, s) : launch_colorize_form<false, false, -1>(a, threads, grid, s);
+    form(std::false_type{});
 }
 
 }  // namespace jt

@@ -79,8 +79,8 @@ __device__ __forceinline__ void for_each_quad(const ViewSet& vs, F&& f) {
 // floor(x) + 1.5 * 2^23 (the sum lies in [2^23, 2^24), where floats are the integers), so
 // t - 1.5 * 2^23 is floor(x) as a float, and the bit pattern of t is that of 1.5 * 2^23
 // (a multiple of 2^22) plus floor(x): masked by w - 1 (w a power of two below 2^22) it is
-// floor(x) floor-mod w. Pixels outside that range, and levels whose sides are not powers of
-// two, take the general path (conversion instructions, which saturate, and a division).
+// floor(x) floor-mod w. Pixels outside that range take the general path (conversion
+// instructions, which saturate, and a division).
 constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
 
 // A pixel's level, from its PixRec (two vector loads; all fields zero for keys outside the
@@ -110,37 +110,68 @@ __device__ __forceinline__ PixL pix_level(const TexLookup& tl, uint32_t tm) {
   return P;
 }
 
-// Bilinear taps on the fast path: a power-of-two level and |u w|, |v h| < 2^22 (returns
-// false otherwise; every tap is then still inside the level, so loads made from it stay in
-// range, but the caller must redo the pixel on the general path). Columns xa, xb = xa + 1,
-// rows ya, yb = ya + 1 (repeat wrap), fractions fx, fy. The range test is of the round-down
-// sums' exponents: [2^23, 2^24). P2: every level is known to be a power of two.
+// The range test of the fast path is of the round-down sums' exponents: [2^23, 2^24).
 __device__ __forceinline__ bool in_range(float tx, float ty) {
   return ((__float_as_uint(tx) ^ 0x4B000000u) | (__float_as_uint(ty) ^ 0x4B000000u)) < 0x00800000u;
 }
 
-template <bool P2 = false>
+// Repeat wrap of the fast path: by the record's masks, for levels known to have power-of-two
+// sides (kWrapPow2) or with the others left to the general path (kWrapChecked), or by a
+// remainder for sides of any size (kWrapAny).
+enum Wrap { kWrapChecked, kWrapPow2, kWrapAny };
+
+template <Wrap WRAP>
+__device__ __forceinline__ bool wrap_covers(const PixL& P) {
+  return WRAP != kWrapChecked || (P.info & kPixPow2) != 0;
+}
+
+// floor-mod of the integer in t = n + kMagic by a side (a float), the largest result in m. For
+// any side: the quotient (two units in the last place), rounded down, is at most one off for |n| < 2^22, so
+// its remainder, exact by the fused step, needs one side added or taken away. Outside that
+// range the result is any number, at most m.
+template <Wrap WRAP>
+__device__ __forceinline__ int wrap_texel(float t, float side, uint32_t m) {
+  if (WRAP != kWrapAny) return __float_as_int(t) & (int)m;
+  const float n = __fsub_rn(t, kMagic);
+  const float q = __fsub_rn(__fadd_rd(__fdividef(n, side), kMagic), kMagic);
+  int r = __float_as_int(__fadd_rn(__fmaf_rn(-q, side, n), kMagic)) - 0x4B400000;
+  const int w = (int)m + 1;
+  r += r < 0 ? w : 0;
+  r -= r >= w ? w : 0;
+  return (int)min((uint32_t)r, m);
+}
+
+template <Wrap WRAP>
+__device__ __forceinline__ int next_texel(int x, uint32_t m) {
+  return WRAP == kWrapAny ? ((uint32_t)x == m ? 0 : x + 1) : (x + 1) & (int)m;
+}
+
+// Bilinear taps on the fast path: |u w|, |v h| < 2^22 and a level that WRAP covers (returns
+// false otherwise; every tap is then still inside the level, so loads made from it stay in
+// range, but the caller must redo the pixel on the general path). Columns xa, xb = xa + 1,
+// rows ya, yb = ya + 1 (repeat wrap), fractions fx, fy.
+template <Wrap WRAP = kWrapChecked>
 __device__ __forceinline__ bool taps_fast(const PixL& P, float u, float v, int& xa, int& xb, int& ya, int& yb,
                                           float& fx, float& fy) {
   const float xs = __fsub_rn(__fmul_rn(u, P.wf), 0.5f), ys = __fsub_rn(__fmul_rn(v, P.hf), 0.5f);
   const float tx = __fadd_rd(xs, kMagic), ty = __fadd_rd(ys, kMagic);
   fx = __fsub_rn(xs, __fsub_rn(tx, kMagic));
   fy = __fsub_rn(ys, __fsub_rn(ty, kMagic));
-  const int wm = (int)(P.masks & 0xFFFFu), hm = (int)(P.masks >> 16);
-  xa = __float_as_int(tx) & wm;
-  ya = __float_as_int(ty) & hm;
-  xb = (xa + 1) & wm;
-  yb = (ya + 1) & hm;
-  return (P2 || (P.info & kPixPow2)) && in_range(tx, ty);
+  const uint32_t wm = P.masks & 0xFFFFu, hm = P.masks >> 16;
+  xa = wrap_texel<WRAP>(tx, P.wf, wm);
+  ya = wrap_texel<WRAP>(ty, P.hf, hm);
+  xb = next_texel<WRAP>(xa, wm);
+  yb = next_texel<WRAP>(ya, hm);
+  return wrap_covers<WRAP>(P) && in_range(tx, ty);
 }
 
 // Nearest texel on the fast path (same conditions as taps_fast).
-template <bool P2 = false>
+template <Wrap WRAP = kWrapChecked>
 __device__ __forceinline__ bool nearest_fast(const PixL& P, float u, float v, int& x, int& y) {
   const float tx = __fadd_rd(__fmul_rn(u, P.wf), kMagic), ty = __fadd_rd(__fmul_rn(v, P.hf), kMagic);
-  x = __float_as_int(tx) & (int)(P.masks & 0xFFFFu);
-  y = __float_as_int(ty) & (int)(P.masks >> 16);
-  return (P2 || (P.info & kPixPow2)) && in_range(tx, ty);
+  x = wrap_texel<WRAP>(tx, P.wf, P.masks & 0xFFFFu);
+  y = wrap_texel<WRAP>(ty, P.hf, P.masks >> 16);
+  return wrap_covers<WRAP>(P) && in_range(tx, ty);
 }
 
 // The same taps for any level and coordinate (conversion instructions, floor-mod by
