@@ -14,8 +14,10 @@
 // instructions (it reads only the quad list and writes 11 bytes a pixel); what was taken out
 // of a pixel: the 64-bit remainder (three 32-bit ones by a precomputed reciprocal), the
 // level's loop (the exponent of the footprint), most conversions, where the camera does not roll the ray divisions
-// (one per pixel row and its two edges, instead of five per pixel), and most of the
-// tiles' listing. 4K, 200 quads: 156 -> 101 us, without quads 57 us.
+// (one per pixel row and its two edges, instead of five per pixel), most of the tiles'
+// listing, the hash of a cell the lane's pixel before lay in, and the tests of quads that do not
+// reach the 32 pixels. 4K, 200 quads, the whole call: 165 -> 108 us, with the last two 102 us (four
+// CTAs per SM at 64 registers; 105 at 74, 118 with five).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -134,11 +136,33 @@ __device__ __forceinline__ void quad_uv(const SceneQuad& q, float x, float y, fl
 
 // Conversions without the special-function unit: floor of |x| < 2^22 from the low bits of
 // x + 1.5 * 2^23 rounded down, and integers below 2^23 as the low bits of 2^23 + n.
-__device__ __forceinline__ int64_t floor_i64(float x) {
-  const uint32_t b = __float_as_uint(__fadd_rd(x, 12582912.0f));
-  return (b ^ 0x4B000000u) < 0x00800000u ? (int64_t)((int)b - 0x4B400000) : (int64_t)floorf(x);
+__device__ __forceinline__ uint32_t floor_bits(float x) { return __float_as_uint(__fadd_rd(x, 12582912.0f)); }
+__device__ __forceinline__ bool small_floor(uint32_t b) { return (b ^ 0x4B000000u) < 0x00800000u; }
+__device__ __forceinline__ int64_t floor_i64(float x, uint32_t b) {
+  return small_floor(b) ? (int64_t)((int)b - 0x4B400000) : (int64_t)floorf(x);
 }
 __device__ __forceinline__ float small_float(uint32_t n) { return fsub(__uint_as_float(0x4B000000u | n), 8388608.0f); }
+
+// A 2 m cell of the ground: its texture and uv offset, and the floors (as floor_bits) it was made
+// for, both zero, which no floor_bits are, for a cell too far out to be told by them.
+struct Cell {
+  uint32_t bu, bv;
+  int tex;
+  float ou, ov;
+  TexSize size;
+};
+__device__ __forceinline__ Cell cell_of(const RasterArgs& a, float u, float v, uint32_t bu, uint32_t bv) {
+  const uint64_t hs = cell_hash(a.cell_seed, (uint64_t)floor_i64(u, bu), (uint64_t)floor_i64(v, bv));
+  Cell c;
+  const bool known = small_floor(bu) && small_floor(bv);
+  c.bu = known ? bu : 0u;
+  c.bv = known ? bv : 0u;
+  c.tex = (int)mod_ntex(hs, a);
+  c.ou = fmul(small_float((uint32_t)(hs >> 16) & 0xFFFFu), 1.0f / 65536.0f);
+  c.ov = fmul(small_float((uint32_t)(hs >> 32) & 0xFFFFu), 1.0f / 65536.0f);
+  c.size = a.use_mips ? tex_size(a, c.tex) : TexSize{};
+  return c;
+}
 
 // A quad's containment test: four edges (corner, edge vector) and the pixel bounds.
 struct QuadEdges {
@@ -155,15 +179,14 @@ __device__ __forceinline__ QuadEdges edges_of(const SceneQuad& q) {
 }
 
 __device__ __forceinline__ bool inside(const QuadEdges& k, int x, int y, float qx, float qy) {
-  if (x < k.b.x || x > k.b.z || y < k.b.y || y > k.b.w) return false;
-  bool in = true;
+  bool in = x >= k.b.x && x <= k.b.z && y >= k.b.y && y <= k.b.w;
 #pragma unroll
   for (int i = 0; i < 4; ++i) in &= !(fsub(fmul(k.e[i].z, fsub(qy, k.e[i].y)), fmul(k.e[i].w, fsub(qx, k.e[i].x))) < 0.0f);
   return in;
 }
 
 template <bool LEVEL>
-__global__ void __launch_bounds__(kThreads) k_raster(const __grid_constant__ RasterArgs a) {
+__global__ void __launch_bounds__(kThreads, 4) k_raster(const __grid_constant__ RasterArgs a) {
   __shared__ uint16_t list[kMaxSceneQuads];
   __shared__ __align__(16) QuadEdges staged[kStagedQuads];
   __shared__ uint32_t warp_count[kThreads / 32];
@@ -204,17 +227,34 @@ __global__ void __launch_bounds__(kThreads) k_raster(const __grid_constant__ Ras
   bool hr, h0, h1;  // the rays of the row, of its upper and of its lower edge
   const RayRow r = ray_row<LEVEL>(a, fy, hr), r0 = ray_row<LEVEL>(a, (float)y, h0),
                r1 = ray_row<LEVEL>(a, fadd((float)y, 1.0f), h1);
+  // lane i's staged quad: the columns it may cover in this row (none past the list)
+  const int4 mine = lane < (int)count ? staged[lane].b : make_int4(1, 1, 0, 0);
+  const bool in_row = y >= mine.y && y <= mine.w;
+  Cell cell{};
 #pragma unroll 1
-  for (int x = tx0 + lane; x <= tx1; x += 32) {
+  for (int xc = tx0; xc <= tx1; xc += 32) {
+    uint32_t near = __ballot_sync(0xFFFFFFFFu, in_row && mine.x <= xc + 31 && mine.z >= xc);
+    const int x = xc + lane;
+    if (x > tx1) break;
     const float xf = a.width < (1 << 23) ? small_float((uint32_t)x) : (float)x;
     const float fx = fadd(xf, 0.5f), qx = fsub(fmul(fx, a.kx), a.shift);
     int hit = -1;
-#pragma unroll 1
-    for (int i = 0; i < (int)count; ++i) {  // the last quad drawn wins
-      if (i < kStagedQuads ? inside(staged[i], x, y, qx, qy)
-                           : inside(edges_of(a.quads[list[count - 1 - i]]), x, y, qx, qy)) {
+    while (near) {  // the last quad drawn wins
+      const int i = __ffs(near) - 1;
+      near &= near - 1;
+      if (inside(staged[i], x, y, qx, qy)) {
         hit = list[count - 1 - i];
         break;
+      }
+    }
+    if (hit < 0 && count > kStagedQuads) {
+#pragma unroll 1
+      for (int i = kStagedQuads; i < (int)count; ++i) {
+        const int n = list[count - 1 - i];
+        if (inside(edges_of(a.quads[n]), x, y, qx, qy)) {
+          hit = n;
+          break;
+        }
       }
     }
     float u = 0.f, v = 0.f;
@@ -238,13 +278,13 @@ __global__ void __launch_bounds__(kThreads) k_raster(const __grid_constant__ Ras
     } else {
       const RayCol c = ray_col(a, fx);
       if (hr && ground<LEVEL>(a, c, r, u, v)) {
-        const int64_t cx = floor_i64(u), cz = floor_i64(v);  // 2 m cells
-        const uint64_t hs = cell_hash(a.cell_seed, (uint64_t)cx, (uint64_t)cz);
-        t = (int)mod_ntex(hs, a);
-        u = fadd(u, fmul(small_float((uint32_t)(hs >> 16) & 0xFFFFu), 1.0f / 65536.0f));
-        v = fadd(v, fmul(small_float((uint32_t)(hs >> 32) & 0xFFFFu), 1.0f / 65536.0f));
+        const uint32_t bu = floor_bits(u), bv = floor_bits(v);
+        if (bu != cell.bu || bv != cell.bv) cell = cell_of(a, u, v, bu, bv);
+        t = cell.tex;
+        u = fadd(u, cell.ou);
+        v = fadd(v, cell.ov);
         if (a.use_mips) {
-          const TexSize z = tex_size(a, t);
+          const TexSize z = cell.size;
           float u0, v0, u1, v1, u2, v2, u3, v3;
           const bool ok = ground<LEVEL>(a, ray_col(a, xf), r, u0, v0) &&
                           ground<LEVEL>(a, ray_col(a, fadd(xf, 1.0f)), r, u1, v1) &&
