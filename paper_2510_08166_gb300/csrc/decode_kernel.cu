@@ -29,6 +29,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstddef>
 
 #include "jt_internal.cuh"
@@ -78,7 +79,9 @@ constexpr int kStageWords = 32;
 // then the staged words [M * kStageWords]. An MCU's 772 bytes are an odd number of words,
 // so that lanes storing the same coefficient of their MCUs hit different banks; a data unit
 // is 32 words, so the pixel phase's reads of one data unit never conflict.
-constexpr int kMcuBytes = 6 * 128 + 4;
+// A batch of 4:4:4 MCUs alone packs them in 388 bytes, two for one of the others.
+constexpr int kMcuBytes = 6 * 128 + 4, kMcuBytes444 = 3 * 128 + 4;
+static_assert(kMcuBytes444 / 4 % 2 == 1 && 4 * kMcuBytes444 % 16 == 0 && 2 * kMcuBytes444 < kMcuBytes + 4 * kStageWords, "as below");
 static_assert(kMcuBytes / 4 % 2 == 1 && 4 * kMcuBytes % 16 == 0, "bank spread, and 16-byte whole for M >= 4");
 __host__ __device__ constexpr size_t warp_smem(int M) { return (size_t)M * (kMcuBytes + kStageWords * 4); }
 
@@ -148,6 +151,7 @@ __device__ __forceinline__ void load_if(bool p, const char* a, uint4& t, uint4& 
 
 constexpr uint32_t kNoSet = 0xFFFFFFFFu;
 constexpr uint32_t kBusyWarps = 12;         // three per SM sub-partition
+constexpr uint32_t kLongRun = 10;           // full batches per warp from which a list is long
 constexpr uint32_t kInvalid = 0x80000000u;  // an invalid coding (bit positions stay far below)
 constexpr uint32_t kSizeMask = 15u << 5;
 constexpr uint32_t kPast = (64u << kRunShift) - (1u << (kRunShift - 1));  // k + entry past slot 63, or kNoEntry at any k
@@ -477,15 +481,14 @@ __device__ __forceinline__ void mcu_pixels(const Frag& f, uint32_t coef, uint32_
 // UNITS: the variant for contexts with data-unit starts. Each MCU of a batch then takes six
 // lanes, lane 6m + d decoding data unit d of MCU m from its own start (levels without
 // starts are decoded whole by lane 6m); MCUs per batch are at most 4.
-template <bool UNITS>
+// LONG: the variant that takes long lists in batches of twice the width.
+template <bool UNITS, bool LONG>
 __global__ void __launch_bounds__(512, 1) k_decode(const __grid_constant__ DecodeArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int M = a.mcus_per_warp;
   const uint32_t coef0 = kStagedTables + (uint32_t)warp * (uint32_t)warp_smem(M);
-  const uint32_t stage0 = coef0 + (uint32_t)(M * kMcuBytes);
   // this lane's MCU slot and data unit (the whole MCU outside the unit variant)
   const int lm = UNITS ? lane / 6 : lane, ld = UNITS ? lane % 6 : 0;
-  const uint32_t mine = coef0 + (uint32_t)((lm < M ? lm : 0) * kMcuBytes);
   const int max_batch = UNITS ? min(M, 4) : M;
 
   // stages set i of the Huffman tables when it fits; kNoSet when it does not
@@ -521,6 +524,7 @@ __global__ void __launch_bounds__(512, 1) k_decode(const __grid_constant__ Decod
   const uint32_t busy = min(warps, kBusyWarps), per_warp = (run + busy - 1) / busy;
   int meff = 1;
   while ((uint32_t)meff < per_warp && meff < max_batch) meff *= 2;
+  if (LONG && 2 * M <= 32 && run >= kLongRun * warps * (uint32_t)M) meff = 2 * M;
   const bool runs = a.nsets > 1;
   const uint32_t span = runs ? min(run, warps * (uint32_t)meff) : warps * (uint32_t)meff;
   const uint32_t first = blockIdx.x * span;
@@ -548,12 +552,13 @@ __global__ void __launch_bounds__(512, 1) k_decode(const __grid_constant__ Decod
     }
     if (base >= limit) break;
 
-    {  // clear the batch's coefficients
+    auto clear = [&](int bytes) {
       uint4* z = reinterpret_cast<uint4*>(smem + coef0);
-      const int nz = (meff * kMcuBytes + 15) / 16;
+      const int nz = (bytes + 15) / 16;
 #pragma unroll 4
       for (int i = lane; i < nz; i += 32) z[i] = make_uint4(0, 0, 0, 0);
-    }
+    };
+    clear(LONG && meff > M ? 2 * M * kMcuBytes444 : meff * kMcuBytes);  // the first part's coefficients
 
     // ---- set-up: lanes of MCU slot m < m_eff take item base + m ----
     const uint32_t item = base + lm;
@@ -629,154 +634,167 @@ __global__ void __launch_bounds__(512, 1) k_decode(const __grid_constant__ Decod
     } else {
       act = false;
     }
-    // ---- entropy phase: each active lane decodes all data units of its MCU (or, with
-    // data-unit starts, one data unit), in rounds of staging and decoding (one round unless
-    // the batch's words exceed the pool) ----
-    int nd = ndu, nl = ndu - 2, seq = s420 ? (cpt ? kSeqCompact420 : kSeq420) : (cpt ? kSeqCompact444 : kSeq444);
-    uint32_t dst = mine;
-    if (UNITS && unit) {
-      nl = ld < nl ? 1 : 0;
-      nd = 1;
-      seq = nl ? kSeqLuma : kSeqChroma;
-      dst += 128 * (uint32_t)ld;
-    }
-    Chain ch{bitpos, kFresh, 0u, (uint32_t)(seq * sizeof(HuffSeq)), (uint32_t)((seq + nd) * sizeof(HuffSeq)), dst};
-    int reached = ndu;  // data units whose DC difference was decoded
-    bool more = act;
-    const uint32_t pool = (uint32_t)(kStageWords * M);
+    // A batch of more than M (of a long list) goes as one part when all of its MCUs are 4:4:4
+    // (packed), and in parts of M otherwise.
+    const bool packed = LONG && meff > M && !__any_sync(0xFFFFFFFFu, act && s420);
+    const int part_mcus = packed || !LONG ? meff : min(meff, M);
+    const uint32_t stride = packed ? kMcuBytes444 : kMcuBytes;
+    const uint32_t stage0 = coef0 + (packed ? 2u * kMcuBytes444 : (uint32_t)kMcuBytes) * (uint32_t)M;
+    const uint32_t pool = (coef0 + (uint32_t)warp_smem(M) - stage0) / 4;
 #pragma unroll 1
-    do {
-      // the chain's words: from its next one (16 B aligned) to the next MCU's start plus the
-      // window's look-ahead (3 words)
-      const uint32_t w0 = (ch.pos >> 5) & ~3u;
-      uint32_t all = (max(endbit, ch.pos) >> 5) + 3 - w0;
-      all = (all + 3) & ~3u;
-      if (w0 + all > nwords) all = nwords > w0 ? (nwords - w0) & ~3u : 0u;
-      if (!more) all = 0;
-      // share the warp's stage pool out by a prefix sum of the lanes' word counts, in equal
-      // shares when they exceed it (at least 12 words: a group of symbols from any bit of the
-      // first four ends inside them, so the first unfinished chain always advances)
-      uint32_t want = all;
-      if (__reduce_add_sync(0xFFFFFFFFu, all) > pool)
-        want = min(all, max(pool / (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, all != 0)) & ~3u, 12u));
-      uint32_t sbeg = want;
-#pragma unroll
-      for (int dlt = 1; dlt < 32; dlt <<= 1) {
-        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, sbeg, dlt);
-        if (lane >= dlt) sbeg += o;
+    for (int part = 0; part < (LONG ? meff : 1); part += part_mcus) {
+      const bool in_part = lm >= part && lm < part + part_mcus, on = act && (!LONG || in_part);
+      const uint32_t mine = coef0 + (in_part ? (uint32_t)(lm - part) * stride : 0u);
+      if (part != 0) clear(M * kMcuBytes);
+      if (LONG) __syncwarp();  // (the packed clear ends inside the other form's stage)
+      // ---- entropy phase: each active lane decodes all data units of its MCU (or, with
+      // data-unit starts, one data unit), in rounds of staging and decoding (one round unless
+      // the batch's words exceed the pool) ----
+      int nd = ndu, nl = ndu - 2, seq = s420 ? (cpt ? kSeqCompact420 : kSeq420) : (cpt ? kSeqCompact444 : kSeq444);
+      uint32_t dst = mine;
+      if (UNITS && unit) {
+        nl = ld < nl ? 1 : 0;
+        nd = 1;
+        seq = nl ? kSeqLuma : kSeqChroma;
+        dst += 128 * (uint32_t)ld;
       }
-      sbeg -= want;  // exclusive
-      const uint32_t nst = sbeg >= pool ? 0u : min(want, pool - sbeg);
-      if (more) {
-        const uint4* src4 = reinterpret_cast<const uint4*>(words + w0);
-        uint4* dst4 = reinterpret_cast<uint4*>(smem + stage0 + 4 * sbeg);
+      Chain ch{bitpos, kFresh, 0u, (uint32_t)(seq * sizeof(HuffSeq)), (uint32_t)((seq + nd) * sizeof(HuffSeq)), dst};
+      int reached = ndu;  // data units whose DC difference was decoded
+      bool more = on;
 #pragma unroll 1
-        for (uint32_t j = 0; j < nst / 4; j += 4) {
-          uint4 r[4];
+      do {
+        // the chain's words: from its next one (16 B aligned) to the next MCU's start plus the
+        // window's look-ahead (3 words)
+        const uint32_t w0 = (ch.pos >> 5) & ~3u;
+        uint32_t all = (max(endbit, ch.pos) >> 5) + 3 - w0;
+        all = (all + 3) & ~3u;
+        if (w0 + all > nwords) all = nwords > w0 ? (nwords - w0) & ~3u : 0u;
+        if (!more) all = 0;
+        // share the warp's stage pool out by a prefix sum of the lanes' word counts, in equal
+        // shares when they exceed it (at least 12 words: a group of symbols from any bit of the
+        // first four ends inside them, so the first unfinished chain always advances)
+        uint32_t want = all;
+        if (__reduce_add_sync(0xFFFFFFFFu, all) > pool)
+          want = min(all, max(pool / (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, all != 0)) & ~3u, 12u));
+        uint32_t sbeg = want;
 #pragma unroll
-          for (int t = 0; t < 4; ++t) r[t] = j + t < nst / 4 ? __ldg(src4 + j + t) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-          for (int t = 0; t < 4; ++t)
-            if (j + t < nst / 4) dst4[j + t] = make_uint4(bswap(r[t].x), bswap(r[t].y), bswap(r[t].z), bswap(r[t].w));
+        for (int dlt = 1; dlt < 32; dlt <<= 1) {
+          const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, sbeg, dlt);
+          if (lane >= dlt) sbeg += o;
         }
-      }
-      __syncwarp();
-      const bool whole = nst >= all;  // staged to its end
-      if (more && (whole || nst >= 12)) {
-        const uint32_t st = stage0 + 4 * sbeg, limit = whole ? 0xFFFFFFFFu : 8 * st + 32 * nst - kGroupBits;
-        bool ok = all != 0;
-        if (ok)
-          ok = !staged_set  ? entropy_fast<false, true>(ch, st, w0, limit, hs)
-               : staged_cap ? entropy_fast<true, true>(ch, st, w0, limit, hs)
-                            : entropy_fast<true, false>(ch, st, w0, limit, hs);
-        more = ok && ch.q != ch.qend;
-        if (!more) {
-          uint64_t end = 32ull * w0 + (ch.pos - 32 * w0);  // after the last symbol
-          // an invalid symbol, or bits past the stage: from the start again, word by word
-          if (!ok || ch.pos - 32 * w0 + 32 > 32 * nst) {
-            const uint32_t f = (bitpos >> 5) & ~3u;
-            const uint32_t r = entropy_any(words + f, nwords > f ? nwords - f : 0u, bitpos - 32 * f, hs, nd, nl, cpt, dst);
-            ok = r < kInvalid;
-            end = 32ull * f + r;
-            if (!ok && !unit) reached = (int)(r - kInvalid);
+        sbeg -= want;  // exclusive
+        const uint32_t nst = sbeg >= pool ? 0u : min(want, pool - sbeg);
+        if (more) {
+          const uint4* src4 = reinterpret_cast<const uint4*>(words + w0);
+          uint4* dst4 = reinterpret_cast<uint4*>(smem + stage0 + 4 * sbeg);
+#pragma unroll 1
+          for (uint32_t j = 0; j < nst / 4; j += 4) {
+            uint4 r[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) r[t] = j + t < nst / 4 ? __ldg(src4 + j + t) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+              if (j + t < nst / 4) dst4[j + t] = make_uint4(bswap(r[t].x), bswap(r[t].y), bswap(r[t].z), bswap(r[t].w));
           }
-          // the coding must be valid and end inside the stream; a compact MCU inside its own
-          // bytes, a data unit at or before the next one's start
-          if (!ok || end > ((cpt || unit) ? endbit : nbits)) any_bad = true;
         }
-      }
+        __syncwarp();
+        const bool whole = nst >= all;  // staged to its end
+        if (more && (whole || nst >= 12)) {
+          const uint32_t st = stage0 + 4 * sbeg, limit = whole ? 0xFFFFFFFFu : 8 * st + 32 * nst - kGroupBits;
+          bool ok = all != 0;
+          if (ok)
+            ok = !staged_set  ? entropy_fast<false, true>(ch, st, w0, limit, hs)
+                 : staged_cap ? entropy_fast<true, true>(ch, st, w0, limit, hs)
+                              : entropy_fast<true, false>(ch, st, w0, limit, hs);
+          more = ok && ch.q != ch.qend;
+          if (!more) {
+            uint64_t end = 32ull * w0 + (ch.pos - 32 * w0);  // after the last symbol
+            // an invalid symbol, or bits past the stage: from the start again, word by word
+            if (!ok || ch.pos - 32 * w0 + 32 > 32 * nst) {
+              const uint32_t f = (bitpos >> 5) & ~3u;
+              const uint32_t r = entropy_any(words + f, nwords > f ? nwords - f : 0u, bitpos - 32 * f, hs, nd, nl, cpt, dst);
+              ok = r < kInvalid;
+              end = 32ull * f + r;
+              if (!ok && !unit) reached = (int)(r - kInvalid);
+            }
+            // the coding must be valid and end inside the stream; a compact MCU inside its own
+            // bytes, a data unit at or before the next one's start
+            if (!ok || end > ((cpt || unit) ? endbit : nbits)) any_bad = true;
+          }
+        }
+        __syncwarp();
+      } while (__any_sync(0xFFFFFFFFu, more));
       __syncwarp();
-    } while (__any_sync(0xFFFFFFFFu, more));
-    __syncwarp();
-    if (act && ld == 0) {  // chain the DC differences (modulo 2^16)
-      uint32_t o = mine;
-      int c0 = pr0;
+      if (on && ld == 0) {  // chain the DC differences (modulo 2^16)
+        uint32_t o = mine;
+        int c0 = pr0;
 #pragma unroll 1
-      for (int d = 0; d < min(ndu - 2, reached); ++d, o += 128) {
-        c0 = (int16_t)(uint16_t)(c0 + (int)sm_i16(o));
-        sm_i16(o) = (int16_t)c0;
-      }
-      if (reached > ndu - 2) sm_i16(o) = (int16_t)(uint16_t)((int)pr1 + (int)sm_i16(o));
-      if (reached > ndu - 1) sm_i16(o + 128) = (int16_t)(uint16_t)((int)pr2 + (int)sm_i16(o + 128));
-    }
-    // ---- pixel phase: the warp takes the batch's MCUs one by one ----
-    const uint32_t minfo = (act && store ? 1u : 0u) | (s420 ? 2u : 0u) | ((uint32_t)red << 2) | (qs << 8);
-    __syncwarp();  // every lane's coefficients are visible to the warp
-    Steps Q{};
-    Frag fr = f8;  // fragments of the last reduced level
-    int rcur = 0;
-    uint32_t qcur = 0xFFFFFFFFu;
-#pragma unroll 1
-    for (int m = 0; m < meff; ++m) {
-      const uint32_t im = __shfl_sync(0xFFFFFFFFu, minfo, UNITS ? 6 * m : m);
-      const uint32_t om = __shfl_sync(0xFFFFFFFFu, off, UNITS ? 6 * m : m);
-      if (!(im & 1u)) continue;
-      if (im >> 8 != qcur) {
-        qcur = im >> 8;
-        const uint16_t* q = a.quant + (size_t)qcur * 128;
-        Q.la = __ldg(q + oa / 2);
-        Q.lb = __ldg(q + ob / 2);
-        Q.ca = __ldg(q + 64 + oa / 2);
-        Q.cb = __ldg(q + 64 + ob / 2);
-        Q.l = __floats2half2_rn(fminf((float)Q.la, 32768.f), fminf((float)Q.lb, 32768.f));
-        Q.c = __floats2half2_rn(fminf((float)Q.ca, 32768.f), fminf((float)Q.cb, 32768.f));
-      }
-      const uint32_t cm = coef0 + (uint32_t)(m * kMcuBytes);
-      uint32_t* tile = reinterpret_cast<uint32_t*>(a.cache + (size_t)om * kUnitBytes);
-      const int rm = (int)((im >> 2) & 3u);
-      if (rm == 0) {
-        if (im & 2u)
-          mcu_pixels<true, false>(f8, cm, oa, ob, Q, bound, 0, tile, lane);
-        else
-          mcu_pixels<false, false>(f8, cm, oa, ob, Q, bound, 0, tile, lane);
-      } else {
-        if (rm != rcur) {
-          rcur = rm;
-          fr = idct_frag(rm, lane);
+        for (int d = 0; d < min(ndu - 2, reached); ++d, o += 128) {
+          c0 = (int16_t)(uint16_t)(c0 + (int)sm_i16(o));
+          sm_i16(o) = (int16_t)c0;
         }
-        if (im & 2u)
-          mcu_pixels<true, true>(fr, cm, oa, ob, Q, bound, rm, tile, lane);
-        else
-          mcu_pixels<false, true>(fr, cm, oa, ob, Q, bound, rm, tile, lane);
+        if (reached > ndu - 2) sm_i16(o) = (int16_t)(uint16_t)((int)pr1 + (int)sm_i16(o));
+        if (reached > ndu - 1) sm_i16(o + 128) = (int16_t)(uint16_t)((int)pr2 + (int)sm_i16(o + 128));
       }
+      // ---- pixel phase: the warp takes the batch's MCUs one by one ----
+      const uint32_t minfo = (on && store ? 1u : 0u) | (s420 ? 2u : 0u) | ((uint32_t)red << 2) | (qs << 8);
+      __syncwarp();  // every lane's coefficients are visible to the warp
+      Steps Q{};
+      Frag fr = f8;  // fragments of the last reduced level
+      int rcur = 0;
+      uint32_t qcur = 0xFFFFFFFFu;
+#pragma unroll 1
+      for (int m = 0; m < part_mcus; ++m) {
+        const uint32_t im = __shfl_sync(0xFFFFFFFFu, minfo, UNITS ? 6 * m : part + m);
+        const uint32_t om = __shfl_sync(0xFFFFFFFFu, off, UNITS ? 6 * m : part + m);
+        if (!(im & 1u)) continue;
+        if (im >> 8 != qcur) {
+          qcur = im >> 8;
+          const uint16_t* q = a.quant + (size_t)qcur * 128;
+          Q.la = __ldg(q + oa / 2);
+          Q.lb = __ldg(q + ob / 2);
+          Q.ca = __ldg(q + 64 + oa / 2);
+          Q.cb = __ldg(q + 64 + ob / 2);
+          Q.l = __floats2half2_rn(fminf((float)Q.la, 32768.f), fminf((float)Q.lb, 32768.f));
+          Q.c = __floats2half2_rn(fminf((float)Q.ca, 32768.f), fminf((float)Q.cb, 32768.f));
+        }
+        const uint32_t cm = coef0 + (uint32_t)m * stride;
+        uint32_t* tile = reinterpret_cast<uint32_t*>(a.cache + (size_t)om * kUnitBytes);
+        const int rm = (int)((im >> 2) & 3u);
+        if (rm == 0) {
+          if (im & 2u)
+            mcu_pixels<true, false>(f8, cm, oa, ob, Q, bound, 0, tile, lane);
+          else
+            mcu_pixels<false, false>(f8, cm, oa, ob, Q, bound, 0, tile, lane);
+        } else {
+          if (rm != rcur) {
+            rcur = rm;
+            fr = idct_frag(rm, lane);
+          }
+          if (im & 2u)
+            mcu_pixels<true, true>(fr, cm, oa, ob, Q, bound, rm, tile, lane);
+          else
+            mcu_pixels<false, true>(fr, cm, oa, ob, Q, bound, rm, tile, lane);
+        }
+      }
+      __syncwarp();  // the buffers are cleared for the next items
     }
-    __syncwarp();  // the buffers are cleared for the next items
   }
   if (any_bad) atomicOr(&a.state->err, JT_DEVERR_CORRUPT);
 }
 
 size_t smem_bytes(int warps, int M) { return kStagedTables + (size_t)warps * warp_smem(M) + kSlackBytes; }
 
-template <bool UNITS>
+template <bool UNITS, bool LONG>
 int occupancy_of(int warps, int M) {
   const size_t smem_b = smem_bytes(warps, M);
   if (smem_b > 227 * 1024) return 0;
-  if (cudaFuncSetAttribute(k_decode<UNITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess) {
+  if (cudaFuncSetAttribute(k_decode<UNITS, LONG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_decode<UNITS>, warps * 32, smem_b) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_decode<UNITS, LONG>, warps * 32, smem_b) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -787,19 +805,29 @@ int occupancy_of(int warps, int M) {
 
 size_t decode_smem_bytes(int warps, int mcus_per_warp) { return smem_bytes(warps, mcus_per_warp); }
 
-// The dynamic shared-memory attribute of both variants is set by decode_max_ctas_per_sm(),
+// The dynamic shared-memory attribute of the variants is set by decode_max_ctas_per_sm(),
 // which the context calls for every (warps, M) on its device before the first launch.
+//
+// The variant for long lists serves contexts whose lists can be long: as many MCUs and cache units
+// as kLongRun full batches for every warp. It takes 32 MCUs a batch, so that the set-up's dependent
+// loads serve twice as many, and packs 4:4:4 ones, so that all lanes decode: 1440 -> 1376 us for
+// eight 4096^2 textures to pixels, half of them 4:4:4 (1.3 M MCUs). It is a kernel of its own
+// because the parts cost a short list time (1080p frame 54.4 -> 54.9 us in one kernel).
 void launch_decode(const DecodeArgs& a, int warps, int grid, cudaStream_t s) {
   const size_t smem_b = smem_bytes(warps, a.mcus_per_warp);
+  const uint64_t most = std::min<uint64_t>(a.ngid, a.cap_units), batch = (uint64_t)grid * (uint32_t)(warps * a.mcus_per_warp);
   if (a.unit_mode)
-    launch_pdl(k_decode<true>, grid, warps * 32, smem_b, s, a);
+    launch_pdl(k_decode<true, false>, grid, warps * 32, smem_b, s, a);
+  else if (most >= kLongRun * batch)
+    launch_pdl(k_decode<false, true>, grid, warps * 32, smem_b, s, a);
   else
-    launch_pdl(k_decode<false>, grid, warps * 32, smem_b, s, a);
+    launch_pdl(k_decode<false, false>, grid, warps * 32, smem_b, s, a);
 }
 
-// Resident CTAs per SM that both variants reach (the launch picks one per frame).
+// Resident CTAs per SM that every variant reaches (the launch picks one per frame).
 int decode_max_ctas_per_sm(int warps, int mcus_per_warp) {
-  return min(occupancy_of<false>(warps, mcus_per_warp), occupancy_of<true>(warps, mcus_per_warp));
+  return std::min({occupancy_of<false, false>(warps, mcus_per_warp), occupancy_of<false, true>(warps, mcus_per_warp),
+                   occupancy_of<true, false>(warps, mcus_per_warp)});
 }
 
 void idct_constants(int out[8]) {

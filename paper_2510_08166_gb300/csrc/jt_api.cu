@@ -519,6 +519,7 @@ jt_status enqueue_decode(jt_ctx* c, cudaStream_t s) {
   a.quant = c->d_quant;
   a.work = c->work;
   a.work_cap = (uint32_t)c->gid_cap;
+  a.ngid = (uint32_t)c->ngid;
   a.slot = c->slot;
   a.cache = c->cache;
   a.cap_units = (uint32_t)c->cap_units;

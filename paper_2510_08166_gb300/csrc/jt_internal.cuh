@@ -319,6 +319,7 @@ struct DecodeArgs {
   const uint16_t* quant;  // [nq][2][64] zig-zag order
   const uint32_t* work;
   uint32_t work_cap;
+  uint32_t ngid;          // MCUs of the context: no list is longer
   const uint32_t* slot;
   uint8_t* cache;
   uint32_t cap_units;
