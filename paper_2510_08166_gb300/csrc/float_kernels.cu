@@ -204,32 +204,56 @@ __global__ void k_float_fill(const __grid_constant__ FloatArgs a) {
       T[i] = taps_of(a, u[i], v[i], t[i], m[i], missing);
       if (check && T[i].ok) T[i].ok = served(a, T[i]);
     }
-    // one kind of entry of the four pixels at a time: their cursors' atomics overlap
-    auto visit = [&](auto second_x, auto second_y) {
+    // places of the four kinds of entries (by the pixel's first or second tap of each axis), all
+    // asked for before the first entry is written: the pass is bound by the atomics' round trips
+    uint32_t pos[4][4];
+    auto take = [&](auto second_x, auto second_y) {
       constexpr bool SX = decltype(second_x)::value, SY = decltype(second_y)::value;
-      uint32_t pos[4];
-      bool on[4];
+      uint32_t(&at)[4] = pos[2 * SY + SX];
+      uint32_t mcu[4], run[4];
+      bool on[4], with_last[4];  // neighbours with one MCU take their places by one atomic
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         on[i] = T[i].ok && (!SX || T[i].xa >> 4 != T[i].xb >> 4) && (!SY || T[i].ya >> 4 != T[i].yb >> 4);
-        pos[i] = a.bucket_cap;
-        if (on[i]) pos[i] = atomicAdd(a.cursor + mcu_of(T[i], SX ? T[i].xb : T[i].xa, SY ? T[i].yb : T[i].ya), 1u);
+        mcu[i] = mcu_of(T[i], SX ? T[i].xb : T[i].xa, SY ? T[i].yb : T[i].ya);
+        with_last[i] = i > 0 && on[i] && on[i - 1] && mcu[i] == mcu[i - 1];
       }
 #pragma unroll
+      for (int i = 3; i >= 0; --i) {
+        run[i] = 1 + (i < 3 && with_last[i + 1] ? run[i + 1] : 0u);
+        at[i] = a.bucket_cap;
+        if (on[i] && !with_last[i]) at[i] = atomicAdd(a.cursor + mcu[i], run[i]);
+      }
+    };
+    auto write = [&](auto second_x, auto second_y) {
+      constexpr bool SX = decltype(second_x)::value, SY = decltype(second_y)::value;
+      uint32_t(&at)[4] = pos[2 * SY + SX];
+      uint32_t last = 0;  // the MCU of the pixel before, and whether it has an entry of the kind
+      bool last_on = false;
+#pragma unroll
       for (int i = 0; i < 4; ++i) {
-        if (pos[i] >= a.bucket_cap) continue;
         const int tx = SX ? T[i].xb : T[i].xa, ty = SY ? T[i].yb : T[i].ya;
+        const bool on = T[i].ok && (!SX || T[i].xa >> 4 != T[i].xb >> 4) && (!SY || T[i].ya >> 4 != T[i].yb >> 4);
+        const uint32_t mcu = mcu_of(T[i], tx, ty);
+        if (i > 0) at[i] = on && last_on && mcu == last ? at[i - 1] + 1 : at[i];
+        last = mcu;
+        last_on = on;
+        if (at[i] >= a.bucket_cap) continue;
         const bool bx = !SX && T[i].xa >> 4 == T[i].xb >> 4, by = !SY && T[i].ya >> 4 == T[i].yb >> 4;
         const int lx = bx ? T[i].xb : tx, ly = by ? T[i].yb : ty;
         const uint32_t info = (uint32_t)((ty & 15) << 4 | (tx & 15)) | (SX ? kLastX : bx ? kBothX : 0u) |
                               (SY ? kLastY : by ? kBothY : 0u) | (uint32_t)((ly & 15) << 16 | (lx & 15) << 12);
-        a.bucket[pos[i]] = make_uint4(p0 + (uint32_t)i, info, __float_as_uint(T[i].fx), __float_as_uint(T[i].fy));
+        a.bucket[at[i]] = make_uint4(p0 + (uint32_t)i, info, __float_as_uint(T[i].fx), __float_as_uint(T[i].fy));
       }
     };
-    visit(std::false_type{}, std::false_type{});
-    visit(std::true_type{}, std::false_type{});
-    visit(std::false_type{}, std::true_type{});
-    visit(std::true_type{}, std::true_type{});
+    auto each = [](auto&& f) {
+      f(std::false_type{}, std::false_type{});
+      f(std::true_type{}, std::false_type{});
+      f(std::false_type{}, std::true_type{});
+      f(std::true_type{}, std::true_type{});
+    };
+    each(take);
+    each(write);
   });
 }
 
