@@ -31,6 +31,7 @@
 // pairs on a persistent grid (248 us forward), loads through the first-level cache.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "jt_internal.cuh"
@@ -557,7 +558,7 @@ void launch_inversion(const FloatArgs& a, int threads, int pixel_grid, cudaStrea
   k_float_count<<<pixel_grid, threads, 0, s>>>(a);
   k_float_sums<<<blocks, 256, 0, s>>>(a);
   k_float_offsets<<<blocks, 256, 0, s>>>(a);
-  k_float_fill<<<pixel_grid, threads, 0, s>>>(a);
+  k_float_fill<<<pixel_grid, std::min(threads, 512), 0, s>>>(a);  // (its registers allow no more)
 }
 
 int gather_grid(const FloatArgs& a, int pairs) {
