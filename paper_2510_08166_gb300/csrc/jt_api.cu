@@ -376,7 +376,13 @@ jt_status check_gbuffer(jt_ctx* c, const jt_gbuffer* g) {
 jt_status make_views(jt_ctx* c, const jt_view* views, int n, bool need_out, ViewSet& vs) {
   if (!views || n <= 0 || n > JT_MAX_VIEWS) return fail(c, JT_ERR_INVALID_ARG, "need 1..%d views", JT_MAX_VIEWS);
   std::memset(&vs, 0, sizeof vs);
-  uint64_t quads = 0, tiles = 0;
+  uint64_t quads = 0, tiles = 0, high = 0;
+  auto tiles_of = [](const jt_gbuffer& g, int rows) {
+    return (uint64_t)((g.width + kTileW - 1) / kTileW) * (uint64_t)((g.height + rows - 1) / rows);
+  };
+  for (int i = 0; i < n; ++i)
+    if (views[i].g.width > 0 && views[i].g.height > 0) high += tiles_of(views[i].g, kTileHigh);
+  vs.tile_h = high >= kFewTiles ? kTileHigh : std::min(kTileHigh, std::max(kTileLow, c->tuning.pixel_threads / 32));
   for (int i = 0; i < n; ++i) {
     jt_status s = check_gbuffer(c, &views[i].g);
     if (s != JT_OK) return s;
@@ -394,7 +400,7 @@ jt_status make_views(jt_ctx* c, const jt_view* views, int n, bool need_out, View
     v.height = views[i].g.height;
     v.tiles_x = (uint32_t)((v.width + kTileW - 1) / kTileW);
     v.tile_begin = (uint32_t)tiles;
-    tiles += (uint64_t)v.tiles_x * ((v.height + kTileH - 1) / kTileH);
+    tiles += tiles_of(views[i].g, vs.tile_h);
   }
   if (quads >= (1ull << 31)) return fail(c, JT_ERR_INVALID_ARG, "views too large");
   vs.n = n;

@@ -173,9 +173,14 @@ struct FrameState {
   uint32_t pad[3];
 };
 
-// Screen passes walk each view in tiles of kTileW x kTileH pixels (one CTA per tile at a
-// time, one warp per 128-pixel row segment), so a CTA's pixels share MCUs.
-constexpr int kTileW = 128, kTileH = 32;
+// Screen passes walk each view in tiles of kTileW x tile_h pixels (one CTA per tile at a
+// time, one warp per 128-pixel row segment), so a CTA's pixels share MCUs. High tiles share
+// more of them; low ones spread a small frame over the SMs, whose 510 tiles of 1080p leave a
+// quarter of the warps idle (frame with 32 rows, 16 and 8: 1080p 55.9, 53.9 and 52.3 us, 4K
+// 110.6, 115.1 and 117.5; 1440p with 32 and 8: 68.5 and 72.1). So views of fewer than kFewTiles
+// high tiles, four CTAs for each SM, get low ones.
+constexpr int kTileW = 128, kTileHigh = 32, kTileLow = 8;
+constexpr uint64_t kFewTiles = 4 * 152, kManyTiles = 8 * 152;
 
 // One view of a (possibly batched) frame, passed by value in the kernel parameters.
 struct View {
@@ -195,6 +200,7 @@ struct ViewSet {
   int n;
   uint32_t total_quads;
   uint32_t total_tiles;
+  int tile_h;  // rows of a tile
 };
 
 // The screen passes' record of one (texture, level): 32 bytes (two vector loads that hit

@@ -2,8 +2,8 @@
 // colourise (Sec. 4.4), for one or several views in one launch.
 //
 // Both stream the G-buffer (11 B/px read; colourise also writes 4 B/px and gathers texels
-// from the block cache). A persistent grid walks the views in 128 x 32 pixel tiles, one warp
-// per 128-pixel row.
+// from the block cache). A persistent grid walks the views in tiles of 128 pixels by 32 or 8
+// rows, one warp per 128-pixel row.
 //
 // Mark: one quad of 4 pixels per lane (32 B + 8 B + 4 B vector loads). Pixels of a tile
 // share MCUs, so Mark keeps a 1024-entry table of the gids its CTA already flagged in shared
@@ -25,6 +25,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <type_traits>
 
@@ -51,18 +52,19 @@ struct RowWalk {
     const uint32_t lt = tile - V.tile_begin;
     const uint32_t ty = lt / V.tiles_x;
     x0 = (int)(lt - ty * V.tiles_x) * kTileW;
-    y0 = (int)ty * kTileH;
+    y0 = (int)ty * vs.tile_h;
   }
   __device__ __forceinline__ void start(const ViewSet& vs) {
     tile = blockIdx.x;
     r = threadIdx.x >> 5;
     vi = 0;
     x0 = y0 = 0;
+    if (r >= vs.tile_h) tile = 0xFFFFFFFFu;  // a warp without a row
     set_tile(vs);
   }
   __device__ __forceinline__ void advance(const ViewSet& vs) {
     r += blockDim.x >> 5;
-    if (r >= kTileH) {
+    if (r >= vs.tile_h) {
       r = threadIdx.x >> 5;
       tile += gridDim.x;
       set_tile(vs);
@@ -151,8 +153,11 @@ __device__ __forceinline__ void mark_pixel(const PixL& P, float u, float v, F&& 
 
 constexpr int kMarkQueue = 8 + 32;  // quads waiting in a warp: fewer than eight, and one row segment's
 
-template <int FILTER>
-__global__ void k_mark(const __grid_constant__ MarkArgs a) {
+// MANY: enough tiles for eight CTAs of 256 threads on every SM (32 registers), whose loads then
+// overlap (passes: 4K 113.3 -> 111.3 us, VR pair 119.5 -> 114.0, eight 4096^2 textures 1393 -> 1356);
+// with fewer tiles there is nothing to fill the SMs with, and six CTAs' 40 registers spill none.
+template <int FILTER, bool MANY>
+__global__ void __launch_bounds__(512, MANY ? 4 : 3) k_mark(const __grid_constant__ MarkArgs a) {
   constexpr int kTap = FILTER == JT_FILTER_NEAREST ? 0 : 1;  // the second tap's distance
   extern __shared__ uint2 queue[];  // [warps][kMarkQueue]: first pixel in the view; view | pixels << 8
   __shared__ uint32_t seen[kSeen];
@@ -461,12 +466,17 @@ __global__ void __launch_bounds__(512, 2) k_colorize(const __grid_constant__ Col
 }  // namespace
 
 void launch_mark(const MarkArgs& a, int threads, int grid, cudaStream_t s) {
-  // the clamped filter reads only the nearest texel's MCU
+  threads = std::min(threads, 512);
   const size_t smem = (size_t)(threads / 32) * kMarkQueue * sizeof(uint2);
+  const bool many = a.views.tile_h == kTileHigh && a.views.total_tiles >= kManyTiles;
+  if (many) grid = (int)std::min<uint64_t>(a.views.total_tiles, 2 * (uint64_t)grid);
+  // the clamped filter reads only the nearest texel's MCU
   if (a.filter == JT_FILTER_NEAREST || a.filter == JT_FILTER_BILINEAR_CLAMP)
-    k_mark<JT_FILTER_NEAREST><<<grid, threads, smem, s>>>(a);
+    many ? k_mark<JT_FILTER_NEAREST, true><<<grid, threads, smem, s>>>(a)
+         : k_mark<JT_FILTER_NEAREST, false><<<grid, threads, smem, s>>>(a);
   else
-    k_mark<JT_FILTER_BILINEAR><<<grid, threads, smem, s>>>(a);
+    many ? k_mark<JT_FILTER_BILINEAR, true><<<grid, threads, smem, s>>>(a)
+         : k_mark<JT_FILTER_BILINEAR, false><<<grid, threads, smem, s>>>(a);
 }
 
 // pixels per lane per step: of one, two and four with three to five 256-thread CTAs per SM, two
@@ -491,6 +501,7 @@ void launch_colorize_form(const ColorizeArgs& a, int threads, int grid, cudaStre
 // with any other sides wraps by a remainder (twelve textures of odd sides in a 1367 x 769 frame,
 // the three calls: 63.0 us with every pixel on the general path, 55.6 so).
 void launch_colorize(const ColorizeArgs& a, int threads, int grid, cudaStream_t s) {
+  threads = std::min(threads, 512);
   const bool s4 = a.tl.all_s4 && a.tl.all_p2 && a.cap_units <= 0xFFFFFFFFu / (kUnitBytes / 4);
   auto form = [&](auto multi) {
     constexpr bool M = decltype(multi)::value;

@@ -66,9 +66,9 @@ __device__ __forceinline__ void for_each_quad(const ViewSet& vs, F&& f) {
     const View& V = vs.v[vi];
     const uint32_t lt = tile - V.tile_begin;
     const int x = (int)(lt % V.tiles_x) * kTileW + lane * 4;
-    const int y0 = (int)(lt / V.tiles_x) * kTileH;
+    const int y0 = (int)(lt / V.tiles_x) * vs.tile_h;
 #pragma unroll 1
-    for (int r = warp; r < kTileH; r += nwarps) f(V, y0 + r, x);
+    for (int r = warp; r < vs.tile_h; r += nwarps) f(V, y0 + r, x);
   }
 }
 
