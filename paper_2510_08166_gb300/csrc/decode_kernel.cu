@@ -192,13 +192,6 @@ struct Chain {
 };
 constexpr uint32_t kFresh = 0xFFFFFFFFu;
 
-// Byte offset in a table of the entry for window w (see HuffSet).
-template <bool CAP>
-__device__ __forceinline__ uint32_t table_index(uint32_t w, int d, int cap) {
-  const int t = (int)(w >> 16), i = (int)(w >> (32 - kLutBits));
-  return 2u * (uint32_t)(CAP ? max(__viaddmin_s32(t, d, cap), i) : __viaddmax_s32(t, d, i));
-}
-
 // SH: the tables staged in shared memory; CAP: a set that needs its tables' caps.
 template <bool SH, bool CAP>
 __device__ __forceinline__ bool entropy_fast(Chain& ch, uint32_t st, uint32_t w0, uint32_t limit, const HuffSet* set) {
@@ -221,7 +214,7 @@ __device__ __forceinline__ bool entropy_fast(Chain& ch, uint32_t st, uint32_t w0
   if (e == kFresh) {
     const uint4 t0 = rec(q + 32);
     k = t0.z;
-    e = entry(t0.x + table_index<CAP>(b0, (int)t0.y, (int)t0.w));
+    e = entry(t0.x + 2u * table_index<CAP>(b0, (int)t0.y, (int)t0.w));
   }
   uint32_t bad = 0;
 #pragma unroll 1
@@ -234,7 +227,7 @@ __device__ __forceinline__ bool entropy_fast(Chain& ch, uint32_t st, uint32_t w0
       const uint32_t w = b0;
       b0 = __funnelshift_l(b1, b0, e);
       const uint32_t en = entry((done ? t.z : t.x) +
-                                table_index<CAP>(b0, (int)(done ? t.w : t.y), (int)(done ? c.z : c.y)));
+                                2u * table_index<CAP>(b0, (int)(done ? t.w : t.y), (int)(done ? c.z : c.y)));
       p += e & 31u;
       o = (p >> 3) & ~3u;
       b1 = __funnelshift_l(sm_u32(o + 8), sm_u32(o + 4), p);
@@ -276,7 +269,7 @@ __device__ __noinline__ uint32_t entropy_any(const uint32_t* gw, uint32_t ngw, u
   for (int it = 0; it < 64 * 6; ++it) {  // at most 64 symbols per data unit: each advances k
     const HuffWalk* t = set->walk + (k == 0 ? 0 : 1) + (du < nl ? 0 : 2);
     const uint32_t w = __funnelshift_l(word((pos >> 5) + 1), word(pos >> 5), pos & 31u);
-    const uint32_t x = (uint32_t)max(min((int)(w >> 16) + __ldg(&t->d), __ldg(&t->cap)), (int)(w >> (32 - kLutBits)));
+    const uint32_t x = table_index<true>(w, __ldg(&t->d), __ldg(&t->cap));
     uint32_t e = __ldg(reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(set) + __ldg(&t->base)) + x);
     if (e == kNoEntry) e = walk_symbol(t, w, k == 0);
     if (e == kNoEntry) return kInvalid + (uint32_t)(du + (k > 0 ? 1 : 0));

@@ -89,9 +89,22 @@ constexpr uint32_t kRunEob = 63;
 constexpr int kRunShift = 10;
 constexpr uint16_t kNoEntry = 0xFFE0;
 
+// Index in a table of the entry for window w. CAP: a table that needs its cap (see below).
+template <bool CAP>
+__host__ __device__ __forceinline__ uint32_t table_index(uint32_t w, int d, int cap) {
+  const int t = (int)(w >> 16), i = (int)(w >> (32 - kLutBits));
+#ifdef __CUDA_ARCH__
+  const int x = __viaddmax_s32(t, d, i);
+#else
+  const int x = t + d > i ? t + d : i;
+#endif
+  return (uint32_t)(CAP && x > cap ? cap : x);
+}
+
 // A code that leaves prefixes unused above its last one (`end`, 65536 for a complete code) has
-// entries up to there only, and the index of a longer code is also capped, at the table's
-// last entry (kNoEntry).
+// entries up to there only, and the index is also capped, at the table's last entry
+// (kNoEntry): the index as a whole, because past `end` a table of few long codes is
+// shorter than 1 << kLutBits, and there w >> 22 lies beyond it too.
 //
 // The MAXCODE walk's tables of one spec, and where its entries are (byte offset in the set).
 struct HuffWalk {

@@ -1,0 +1,108 @@
+"""Host logic of the library on a CUDA runtime of host memory (fake_runtime.cpp): decode tables,
+and what the calls keep and leave behind. No GPU needed."""
+
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+import synth
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CUDA_INCLUDE = "/usr/local/cuda/include"
+
+
+@pytest.fixture(scope="module")
+def fake_library(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None or not os.path.exists(os.path.join(CUDA_INCLUDE, "cuda_runtime.h")):
+        pytest.skip("no host C++ compiler or no CUDA headers")
+    import paper_2510_08166_gb300 as jt
+    so = str(tmp_path_factory.mktemp("fake") / "libjt_fake.so")
+    subprocess.check_call([cxx, "-std=c++17", "-O1", "-w", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", CUDA_INCLUDE,
+                           "-I", os.path.join(ROOT, "include"), "-I",
+                           os.path.join(ROOT, "paper_2510_08166_gb300", "csrc"),
+                           os.path.join(ROOT, "tests", "fake_runtime.cpp"), "-o", so])
+    lib = ctypes.CDLL(so)
+    for name, argtypes in jt._SIGS.items():
+        if hasattr(lib, name):
+            f = getattr(lib, name)
+            f.argtypes = argtypes
+            f.restype = ctypes.c_char_p if name in ("jt_last_error", "jt_status_string") else ctypes.c_int
+    lib.fake_begin_capture.restype = ctypes.c_void_p
+    lib.fake_scene_tables.restype = ctypes.c_size_t
+    return lib
+
+
+@pytest.fixture
+def fake(fake_library, monkeypatch):
+    """The package's binding over the fake library."""
+    import paper_2510_08166_gb300 as jt
+    monkeypatch.setattr(jt, "lib", lambda: fake_library)
+    return fake_library
+
+
+def spec(lengths, symbols):
+    """(bits[16], vals[256]) of canonical codes of the given lengths (ascending)."""
+    bits, vals = np.zeros(16, np.uint8), np.zeros(256, np.uint8)
+    for l in lengths:
+        bits[l - 1] += 1
+    vals[:len(symbols)] = symbols
+    return bits, vals
+
+
+def naive_entries(bits, vals, dc):
+    """Per 16-bit prefix: (code length, symbol) of T.81 Annex C's code assignment, else None."""
+    out, code, k = [None] * 65536, 0, 0
+    for l in range(1, 17):
+        for _ in range(int(bits[l - 1])):
+            s = int(vals[k])
+            size = s if dc else s & 15
+            valid = size <= (11 if dc else 10) and (dc or size or s in (0x00, 0xF0))
+            for p in range(code << (16 - l), (code + 1) << (16 - l)):
+                out[p] = (l, s) if valid else None
+            code, k = code + 1, k + 1
+        code <<= 1
+    return out
+
+
+def entry(l, s, dc):
+    run, size = (0, s) if dc else (s >> 4, s & 15)
+    if not dc and s == 0:
+        run = 63
+    return (l + size) | (size << 5) | (run << 10)
+
+
+DC, AC = list(range(12)), [0x00, 0x01, 0x02, 0x11, 0x03, 0x21, 0x12, 0x31, 0xF0, 0x04, 0x41, 0x05]
+SHAPES = {
+    "one short, one long": [1, 16],                # 514 entries: w >> 22 alone reaches past them
+    "a few short, one long": [4] * 11 + [12],
+    "one long": [11],
+    "short only": [4] * 12,
+    "complete but for one prefix": list(range(1, 12)) + [16],
+    "long only": [13] * 12,
+}
+
+
+@pytest.mark.parametrize("name", SHAPES)
+@pytest.mark.parametrize("at", [(0, 1, 2, 3), (3,), (0,)])
+def test_every_prefix_finds_its_entry(fake, name, at):
+    import paper_2510_08166_gb300 as jt
+    std_bits, std_vals, _ = synth.standard_huffman()
+    enc = synth.encode(synth.texture(1, 16, 16), 80, 420)
+    lengths = SHAPES[name]
+    bits, vals = std_bits.copy(), std_vals.copy()
+    for t in at:
+        bits[t], vals[t] = spec(lengths, np.resize(AC if t & 1 else DC, len(lengths)))
+    enc.huff_bits, enc.huff_vals = bits, vals
+    ctx = jt.Context(0, 64)
+    ctx.upload(0, 0, enc)
+    got = np.empty((1, 4, 65536), np.int32)
+    fake.fake_table_entries(ctx._h, ctypes.c_void_p(got.ctypes.data))
+    for t in range(4):
+        want = np.array([0xFFE0 if e is None else entry(*e, t % 2 == 0) for e in naive_entries(bits[t], vals[t], t % 2 == 0)])
+        assert np.array_equal(got[0, t], want), (t, np.flatnonzero(got[0, t] != want)[:4])
+    ctx.close()
