@@ -20,6 +20,8 @@ namespace {
 
 enum class Phase { Idle, Marked, Decoded };
 
+constexpr uint32_t kSceneHosts = 16;
+
 struct Level {
   int tex, level;
   void* stream_mem = nullptr;
@@ -93,9 +95,15 @@ struct jt_ctx {
   uint64_t bucket_cap = 0;
   cudaStream_t capture_stream = nullptr;
 
-  // scene rasteriser inputs (jt_raster_scene)
+  // scene rasteriser inputs (jt_raster_scene): the device copy, and the host memory that the calls
+  // copy it from, in turn; scene_read[h] follows the copies of half h
   uint8_t* raster_buf = nullptr;
   size_t raster_cap = 0;
+  bool raster_captured = false;          // a graph copies to raster_buf
+  std::vector<uint8_t*> raster_retired;  // outgrown, but graphs may copy to them
+  std::vector<uint8_t> scene_host[kSceneHosts];
+  cudaEvent_t scene_read[2] = {};
+  uint32_t scene_calls = 0;
 
   // pass timing (jt_profile)
   bool profiling = false;
@@ -637,6 +645,53 @@ jt_status float_bucket(jt_ctx* c, FloatArgs& a, cudaStream_t st) {
   return JT_OK;
 }
 
+// The host memory of jt_raster_scene's next copy. Calls take kSceneHosts vectors in turn, and an event
+// after each half of them says that their copies are done: one wait and one record for eight
+// calls, and up to eight calls ahead of the stream without waiting.
+jt_status scene_host_of_call(jt_ctx* c, std::vector<uint8_t>*& host) {
+  const uint32_t n = c->scene_calls % kSceneHosts;
+  if (n % (kSceneHosts / 2) == 0) {
+    cudaEvent_t& read = c->scene_read[n / (kSceneHosts / 2)];
+    if (!read) {
+      JT_CUDA(c, cudaEventCreateWithFlags(&read, cudaEventDisableTiming));
+    } else {  // (another stream of the program may be capturing)
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      JT_CUDA(c, cudaThreadExchangeStreamCaptureMode(&mode));
+      const cudaError_t e = cudaEventSynchronize(read);
+      JT_CUDA(c, cudaThreadExchangeStreamCaptureMode(&mode));
+      JT_CUDA(c, e);
+    }
+  }
+  host = &c->scene_host[n];
+  return JT_OK;
+}
+
+// After that copy was enqueued on st.
+jt_status scene_copied(jt_ctx* c, cudaStream_t st) {
+  const uint32_t n = c->scene_calls++ % kSceneHosts;
+  if ((n + 1) % (kSceneHosts / 2) == 0) JT_CUDA(c, cudaEventRecord(c->scene_read[n / (kSceneHosts / 2)], st));
+  return JT_OK;
+}
+
+// In a capture: memory that the graph owns, as each of its launches copies from it again.
+jt_status scene_host_of_graph(jt_ctx* c, cudaGraph_t graph, std::vector<uint8_t>*& host) {
+  auto* mem = new std::vector<uint8_t>();
+  auto destroy = [](void* p) { delete static_cast<std::vector<uint8_t>*>(p); };
+  cudaUserObject_t owner = nullptr;
+  cudaError_t e = cudaUserObjectCreate(&owner, mem, destroy, 1, cudaUserObjectNoDestructorSync);
+  if (e != cudaSuccess) {
+    delete mem;
+    return fail(c, JT_ERR_CUDA, "graph memory: %s", cudaGetErrorString(e));
+  }
+  e = cudaGraphRetainUserObject(graph, owner, 1, cudaGraphUserObjectMove);
+  if (e != cudaSuccess) {
+    cudaUserObjectRelease(owner, 1);
+    return fail(c, JT_ERR_CUDA, "graph memory: %s", cudaGetErrorString(e));
+  }
+  host = mem;
+  return JT_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -739,6 +794,9 @@ jt_status jt_destroy(jt_ctx* c) {
   dev_free(c->float_sums);
   dev_free(c->bucket);
   dev_free(c->raster_buf);
+  for (uint8_t*& p : c->raster_retired) dev_free(p);
+  for (cudaEvent_t& e : c->scene_read)
+    if (e) cudaEventDestroy(e);
   if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
   for (cudaEvent_t& e : c->prof)
     if (e) cudaEventDestroy(e);
@@ -1038,24 +1096,39 @@ jt_status jt_raster_scene(jt_ctx* c, const jt_scene* sc, const jt_gbuffer* out, 
   // device copies of the texture table ([w, h, levels] as 16-byte records) and the quads
   const size_t qoff = (size_t)sc->ntex * 16;
   const size_t need = qoff + (size_t)sc->nquads * sizeof(SceneQuad);
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaGraph_t graph = nullptr;
+  JT_CUDA(c, cudaStreamGetCaptureInfo(st, &cap, nullptr, &graph, nullptr, nullptr, nullptr));
   if (need > c->raster_cap) {
-    dev_free(c->raster_buf);
+    if (c->raster_captured)
+      c->raster_retired.push_back(c->raster_buf);
+    else
+      dev_free(c->raster_buf);
     c->raster_buf = nullptr;
     c->raster_cap = 0;
+    c->raster_captured = false;
     jt_status s = dev_alloc(c, &c->raster_buf, need);
     if (s != JT_OK) return s;
     c->raster_cap = need;
   }
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // one copy of them all (pageable memory is staged before the call returns)
-  std::vector<uint8_t> host(need);
+  // one copy of them all, from memory that outlives it (nothing says that a copy from pageable memory
+  // has read it when the call returns)
+  std::vector<uint8_t>* host = nullptr;
+  jt_status s = cap == cudaStreamCaptureStatusActive ? scene_host_of_graph(c, graph, host) : scene_host_of_call(c, host);
+  if (s != JT_OK) return s;
+  host->assign(need, 0);
   for (int t = 0; t < sc->ntex; ++t) {
     const float wh[2] = {(float)sc->tex_w[t], (float)sc->tex_h[t]};
-    std::memcpy(host.data() + (size_t)t * 16, wh, 8);
-    std::memcpy(host.data() + (size_t)t * 16 + 8, &sc->tex_levels[t], 4);
+    std::memcpy(host->data() + (size_t)t * 16, wh, 8);
+    std::memcpy(host->data() + (size_t)t * 16 + 8, &sc->tex_levels[t], 4);
   }
-  if (sc->nquads) std::memcpy(host.data() + qoff, sc->quads, (size_t)sc->nquads * sizeof(SceneQuad));
-  JT_CUDA(c, cudaMemcpyAsync(c->raster_buf, host.data(), need, cudaMemcpyHostToDevice, st));
+  if (sc->nquads) std::memcpy(host->data() + qoff, sc->quads, (size_t)sc->nquads * sizeof(SceneQuad));
+  JT_CUDA(c, cudaMemcpyAsync(c->raster_buf, host->data(), need, cudaMemcpyHostToDevice, st));
+  if (cap == cudaStreamCaptureStatusActive)
+    c->raster_captured = true;
+  else if ((s = scene_copied(c, st)) != JT_OK)
+    return s;
   RasterArgs a{};
   a.width = sc->width;
   a.height = sc->height;

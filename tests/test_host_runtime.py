@@ -106,3 +106,84 @@ def test_every_prefix_finds_its_entry(fake, name, at):
         want = np.array([0xFFE0 if e is None else entry(*e, t % 2 == 0) for e in naive_entries(bits[t], vals[t], t % 2 == 0)])
         assert np.array_equal(got[0, t], want), (t, np.flatnonzero(got[0, t] != want)[:4])
     ctx.close()
+
+
+def device(a):
+    """A host array as the fake runtime's device memory, with what the binding asks of a tensor."""
+    a.data_ptr = lambda: a.ctypes.data
+    return a
+
+
+class Array(np.ndarray):
+    """An array that can carry a data_ptr (16-byte aligned, as numpy's larger arrays are)."""
+
+
+def zeros(*shape, dtype=np.float32):
+    return device(np.zeros(shape, dtype).view(Array))
+
+
+class GBuffer:
+    def __init__(self, w, h):
+        self.width, self.height = w, h
+        self.uv, self.tex_id, self.mip = zeros(h, w, 2), zeros(h, w, dtype=np.uint16), zeros(h, w, dtype=np.uint8)
+
+    def c(self):
+        import paper_2510_08166_gb300 as jt
+        return jt.jt_gbuffer(self.uv.data_ptr(), self.tex_id.data_ptr(), self.mip.data_ptr(), self.width, self.height)
+
+
+class Scene:
+    """What raster_scene takes: `n` textures of sides of their own and three quads."""
+
+    def __init__(self, seed, n):
+        self.width = self.height = 16
+        self.cam, self.rot = [0, 1, 0], [1, 0, 0, 0, 1, 0, 0, 0, 1]
+        self.ax = self.ay = self.tan_x = self.tan_y = self.max_t = self.kx = self.ky = 1.0
+        self.shift, self.cell_seed, self.use_mips = 0.0, 1, 1
+        self.tex_w = np.arange(1, n + 1, dtype=np.int32) + seed * 1000
+        self.tex_h, self.tex_levels = self.tex_w + 5, np.full(n, 1 + seed % 4, np.int32)
+        self.quads = np.zeros(3, synth.QUAD_DTYPE)
+        self.quads["tex"], self.quads["rep"] = np.arange(3) % n, seed
+
+    def tables(self):
+        t = np.zeros((len(self.tex_w), 4), np.float32)
+        t[:, 0], t[:, 1], t[:, 2] = self.tex_w, self.tex_h, self.tex_levels.view(np.float32)
+        return t.tobytes() + self.quads.tobytes()
+
+
+def scene_tables(fake):
+    out = np.zeros(fake.fake_scene_tables(None), np.uint8)
+    fake.fake_scene_tables(ctypes.c_void_p(out.ctypes.data))
+    return out.tobytes()
+
+
+def test_a_scene_is_copied_from_memory_that_outlives_the_call(fake):
+    import paper_2510_08166_gb300 as jt
+    ctx, gb = jt.Context(0, 64), GBuffer(16, 16)
+    for seed in range(40):  # more calls than the host memory has turns, the copies read late
+        s = Scene(seed, 1 + seed * 7 % 50)
+        ctx.raster_scene(s, gb, 0)
+        if seed % 3 == 0:
+            assert scene_tables(fake) == s.tables()
+    assert scene_tables(fake) == s.tables()
+    ctx.close()
+
+
+def test_a_captured_scene_keeps_its_tables(fake):
+    import paper_2510_08166_gb300 as jt
+    ctx, gb = jt.Context(0, 64), GBuffer(16, 16)
+    ctx.raster_scene(Scene(0, 9), gb, 0)
+    graph = fake.fake_begin_capture()
+    s = Scene(1, 9)
+    ctx.raster_scene(s, gb, 0)
+    fake.fake_end_capture()
+    for seed in range(2, 30):  # others come between its launches, larger ones too
+        other = Scene(seed, 9 if seed < 20 else 400)
+        ctx.raster_scene(other, gb, 0)
+        assert scene_tables(fake) == other.tables()
+        fake.fake_launch_graph(ctypes.c_void_p(graph))
+        assert scene_tables(fake) == s.tables()
+    assert fake.fake_owned(ctypes.c_void_p(graph)) == 1
+    fake.fake_destroy_graph(ctypes.c_void_p(graph))
+    assert fake.fake_owned(ctypes.c_void_p(graph)) == 0
+    ctx.close()
