@@ -574,7 +574,8 @@ bool float_configure() {
          cudaFuncSetAttribute(k_float_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem) == cudaSuccess;
 }
 
-// The cursors must be zero on entry (the gathers leave them so), and the forward's frame.
+// The cursors must be zero on entry (the gathers leave them so; after a failed launch the caller
+// clears them), and the forward's frame.
 void launch_float_forward(const FloatArgs& a, int threads, int pixel_grid, cudaStream_t s) {
   launch_inversion(a, threads, pixel_grid, s);
   k_float_forward<<<gather_grid(a, kForwardPairs), kFloatWarps * 32, kForwardSmem, s>>>(a);

@@ -89,6 +89,7 @@ struct jt_ctx {
   uint32_t coef_gid_base = 0;
   uint32_t float_tile_cap = 0;     // needed coefficient MCUs a float pass can serve
   uint32_t* float_cursor = nullptr;   // [coefficient MCUs], zero between passes
+  bool float_stale = false;           // except after a pass that stopped before its gather
   uint32_t* float_offset = nullptr;   // [coefficient MCUs]
   uint64_t* float_sums = nullptr;     // one per kFloatScan counts
   uint4* bucket = nullptr;            // [bucket_cap] entries
@@ -643,6 +644,23 @@ jt_status float_bucket(jt_ctx* c, FloatArgs& a, cudaStream_t st) {
   a.bucket = c->bucket;
   a.bucket_cap = (uint32_t)std::min<uint64_t>(c->bucket_cap, 0xFFFFFFFFull);
   return JT_OK;
+}
+
+// Launches a pass of the float chain. Its last kernel leaves the cursors at zero for the next one;
+// if a launch failed they may hold counts, and the next pass clears them first (in a capture
+// that clears nothing yet, so the one after it does so again).
+jt_status float_pass(jt_ctx* c, const FloatArgs& a, cudaStream_t st, const char* what,
+                     void (*launch)(const FloatArgs&, int, int, cudaStream_t)) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (c->float_stale) {
+    JT_CUDA(c, cudaStreamIsCapturing(st, &cap));
+    JT_CUDA(c, cudaMemsetAsync(c->float_cursor, 0, (size_t)a.coef_mcus * 4, st));
+  }
+  c->float_stale = true;
+  launch(a, c->tuning.pixel_threads, pixel_grid(c, a.views), st);
+  jt_status s = check_launch(c, what);
+  if (s == JT_OK) c->float_stale = cap == cudaStreamCaptureStatusActive;
+  return s;
 }
 
 // The host memory of jt_raster_scene's next copy. Calls take kSceneHosts vectors in turn, and an event
@@ -1555,8 +1573,7 @@ jt_status jt_colorize_float(jt_ctx* c, const jt_gbuffer* g, const float* coeffs,
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if ((s = float_bucket(c, a, st)) != JT_OK) return s;
   JT_CUDA(c, cudaMemsetAsync(out_rgb, 0, (size_t)a.views.v[0].width * a.views.v[0].height * 3 * sizeof(float), st));
-  launch_float_forward(a, c->tuning.pixel_threads, pixel_grid(c, a.views), st);
-  if ((s = check_launch(c, "float forward")) != JT_OK) return s;
+  if ((s = float_pass(c, a, st, "float forward", launch_float_forward)) != JT_OK) return s;
   c->phase = Phase::Idle;  // the work list now describes coefficient MCUs
   c->last_stream = st;
   return JT_OK;
@@ -1573,8 +1590,7 @@ jt_status jt_colorize_backward(jt_ctx* c, const jt_gbuffer* g, const float* grad
   DeviceGuard dg(c->device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if ((s = float_bucket(c, a, st)) != JT_OK) return s;
-  launch_float_backward(a, c->tuning.pixel_threads, pixel_grid(c, a.views), st);
-  if ((s = check_launch(c, "float backward")) != JT_OK) return s;
+  if ((s = float_pass(c, a, st, "float backward", launch_float_backward)) != JT_OK) return s;
   c->phase = Phase::Idle;
   c->last_stream = st;
   return JT_OK;
