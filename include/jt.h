@@ -311,8 +311,9 @@ jt_status jt_get_tuning(const jt_ctx* ctx, jt_tuning* out);
 jt_status jt_set_tuning(jt_ctx* ctx, const jt_tuning* t);
 
 /* Times `reps` graph replays of the frame for each candidate launch configuration (decode
- * MCUs per warp x warps per CTA x CTAs per SM, then the pixel-kernel shape), keeps the
- * fastest in the context and returns it with its median frame time in milliseconds. */
+ * MCUs per warp x warps per CTA x CTAs per SM, then the pixel-kernel shape) and for the one in
+ * use, keeps the fastest in the context and returns it with its median frame time in
+ * milliseconds. */
 jt_status jt_autotune(jt_ctx* ctx, const jt_view* views, int nviews, int filter, jt_stream stream, int reps,
                       jt_tuning* best, float* best_ms);
 

@@ -585,9 +585,9 @@ bool valid_filter(int f) {
 }
 
 const int kMcusPerWarp[] = {4, 8, 16, 32};
-// warps per decode CTA the autotuner tries (any 1..16 is valid); the odd counts let the
-// 32-MCU shape fill an SM's shared memory (seven warps of 28 KiB)
-const int kDecodeWarps[] = {2, 3, 4, 5, 6, 7, 8, 12, 16};
+// warps per decode CTA the autotuner tries (any 1..16 is valid); seven let the 32-MCU shape fill an
+// SM's shared memory, fourteen the 16-MCU one (the default)
+const int kDecodeWarps[] = {2, 3, 4, 5, 6, 7, 8, 12, 14, 16};
 
 bool valid_tuning(const jt_ctx* c, const jt_tuning& t) {
   const int M = t.decode_mcus_per_warp, W = t.decode_warps;
@@ -1422,7 +1422,8 @@ jt_status jt_autotune(jt_ctx* c, const jt_view* views, int nviews, int filter, j
   };
   jt_tuning cur = saved, top = saved;
   float top_ms = 1e30f;
-  jt_status s = JT_OK;
+  jt_status s = measure(saved, top_ms);  // the shape in use is the first candidate
+  if (s != JT_OK) goto done;
   // stage 1: decode shape (MCUs per warp x warps per CTA at full occupancy, then fewer CTAs)
   for (int M : kMcusPerWarp) {
     for (int W : kDecodeWarps) {

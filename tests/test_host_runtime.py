@@ -210,3 +210,20 @@ def test_a_failed_float_pass_leaves_no_counts_to_the_next(fake):
         ctx.stats()
         assert not fake.fake_cursors_dirty()
     ctx.close()
+
+
+@pytest.mark.parametrize("mcus,warps", [(16, 14), (32, 7), (8, 9), (4, 1)])  # the default, a listed one, two of neither
+def test_autotune_times_the_shape_in_use(fake, mcus, warps):
+    import paper_2510_08166_gb300 as jt
+    ctx, gb, out = jt.Context(0, 64), GBuffer(64, 64), zeros(64, 64, 4, dtype=np.uint8)
+    ctx.upload(0, 0, synth.encode(synth.texture(1, 64, 64), 80, 420))
+    used = {**ctx.tuning(), "decode_mcus_per_warp": mcus, "decode_warps": warps, "decode_ctas_per_sm": 1}
+    ctx.set_tuning(**used)
+    fake.fake_fast_shape(mcus, warps)
+    best, ms = ctx.autotune([(gb, out)], jt.FILTER_BILINEAR, reps=2, stream=0)
+    assert ms == 1.0 and (best["decode_mcus_per_warp"], best["decode_warps"]) == (mcus, warps)
+    # the default is found from any other shape too
+    fake.fake_fast_shape(16, 14)
+    best, ms = ctx.autotune([(gb, out)], jt.FILTER_BILINEAR, reps=2, stream=0)
+    assert ms == 1.0 and (best["decode_mcus_per_warp"], best["decode_warps"]) == (16, 14)
+    ctx.close()
