@@ -190,10 +190,10 @@ struct FrameState {
 // time, one warp per 128-pixel row segment), so a CTA's pixels share MCUs. High tiles share
 // more of them; low ones spread a small frame over the SMs, whose 510 tiles of 1080p leave a
 // quarter of the warps idle (frame with 32 rows, 16 and 8: 1080p 55.9, 53.9 and 52.3 us, 4K
-// 110.6, 115.1 and 117.5; 1440p with 32 and 8: 68.5 and 72.1). So views of fewer than kFewTiles
-// high tiles, four CTAs for each SM, get low ones.
+// 110.6, 115.1 and 117.5; 1440p with 32 and 8: 68.5 and 72.1). So views of fewer high tiles than
+// kFewTilesPerSm CTAs for each SM get low ones.
 constexpr int kTileW = 128, kTileHigh = 32, kTileLow = 8;
-constexpr uint64_t kFewTiles = 4 * 152, kManyTiles = 8 * 152;
+constexpr uint64_t kFewTilesPerSm = 4, kManyTilesPerSm = 8;
 
 // One view of a (possibly batched) frame, passed by value in the kernel parameters.
 struct View {
@@ -253,6 +253,7 @@ struct MarkArgs {
   FrameState* state;
   int filter;
   int only_tex;   // -1: all textures; otherwise only pixels with this texture id
+  bool many;      // high tiles, at least kManyTilesPerSm for each SM
 };
 void launch_mark(const MarkArgs& a, int threads, int grid, cudaStream_t s);
 
@@ -317,7 +318,7 @@ struct RasterArgs {
   float ax, ay, tan_x, tan_y, max_t, kx, ky, shift;
   uint64_t cell_seed;
   int32_t ntex, use_mips, nquads;
-  int32_t tile_x;             // columns of a CTA's tile (chosen by the launcher)
+  int32_t tile_x;             // columns of a CTA's tile
   uint32_t mod_m;             // floor(2^32 / ntex), or 2^32 - 1 for one texture
   const float4* sizes;        // device copies: per texture its level-0 sides and (bits of) its level count,
   const SceneQuad* quads;     // then the quads
@@ -325,6 +326,7 @@ struct RasterArgs {
   uint16_t* tex;
   uint8_t* mip;
 };
+constexpr int kRasterTileY = 8;  // rows of a CTA's tile
 void launch_raster(const RasterArgs& a, cudaStream_t s);
 
 struct DecodeArgs {

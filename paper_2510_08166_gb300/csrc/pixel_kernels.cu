@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(512, 2) k_colorize(const __grid_constant__ Col
 void launch_mark(const MarkArgs& a, int threads, int grid, cudaStream_t s) {
   threads = std::min(threads, 512);
   const size_t smem = (size_t)(threads / 32) * kMarkQueue * sizeof(uint2);
-  const bool many = a.views.tile_h == kTileHigh && a.views.total_tiles >= kManyTiles;
+  const bool many = a.many;
   if (many) grid = (int)std::min<uint64_t>(a.views.total_tiles, 2 * (uint64_t)grid);
   // the clamped filter reads only the nearest texel's MCU
   if (a.filter == JT_FILTER_NEAREST || a.filter == JT_FILTER_BILINEAR_CLAMP)

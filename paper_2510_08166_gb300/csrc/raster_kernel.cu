@@ -27,7 +27,7 @@
 namespace jt {
 namespace {
 
-constexpr int kTileY = 8, kThreads = 32 * kTileY;
+constexpr int kThreads = 32 * kRasterTileY;
 constexpr int kStagedQuads = 32;
 
 __device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b); }
@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_raster(const __grid_constant__ 
   __shared__ __align__(16) QuadEdges staged[kStagedQuads];
   __shared__ uint32_t warp_count[kThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int tx0 = blockIdx.x * a.tile_x, ty0 = blockIdx.y * kTileY;
-  const int tx1 = min(tx0 + a.tile_x, a.width) - 1, ty1 = min(ty0 + kTileY, a.height) - 1;
+  const int tx0 = blockIdx.x * a.tile_x, ty0 = blockIdx.y * kRasterTileY;
+  const int tx1 = min(tx0 + a.tile_x, a.width) - 1, ty1 = min(ty0 + kRasterTileY, a.height) - 1;
 
   // the quads that may cover the tile, in drawing order
   uint32_t count = 0;
@@ -308,14 +308,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_raster(const __grid_constant__ 
 
 }  // namespace
 
-void launch_raster(const RasterArgs& args, cudaStream_t s) {
-  RasterArgs a = args;
-  // wide tiles share the quads' listing and a row's rays among more pixels (4K, 200 quads: 104 us
-  // with 128 columns, 101 with 256), narrow ones keep a small frame's SMs busy: eight CTAs each
-  const int rows = (a.height + kTileY - 1) / kTileY;
-  for (a.tile_x = 256; a.tile_x > 32 && (int64_t)((a.width + a.tile_x - 1) / a.tile_x) * rows < 8 * 152; a.tile_x /= 2) {
-  }
-  const dim3 grid((a.width + a.tile_x - 1) / a.tile_x, rows);
+void launch_raster(const RasterArgs& a, cudaStream_t s) {
+  const dim3 grid((a.width + a.tile_x - 1) / a.tile_x, (a.height + kRasterTileY - 1) / kRasterTileY);
   // a finite column factor times zero adds nothing to dy: the camera does not roll
   if (a.rot[3] == 0.0f && std::isfinite(a.ax * (a.width + 1.0f)) && std::isfinite(a.tan_x) &&
       std::isfinite((a.ax * (a.width + 1.0f) - 1.0f) * a.tan_x))

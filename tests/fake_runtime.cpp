@@ -29,7 +29,7 @@ cudaError_t last_error = cudaSuccess;
 int sm_count = 152, fast_mcus = 0, fast_warps = 0, run_mcus = 0, run_warps = 0;
 bool fail_gather = false, cursors_dirty = false;
 std::vector<uint8_t> scene_tables;
-int tile_x = 0, tile_h = 0;
+int tile_x = 0, tile_h = 0, many = 0;
 
 void put(std::function<void()> f) { (capture ? capture->ops : pending).push_back(std::move(f)); }
 cudaError_t wait() {
@@ -141,6 +141,7 @@ void fake_fail_gather(int on) { fail_gather = on != 0; }
 int fake_cursors_dirty() { return cursors_dirty; }
 int fake_tile_h() { return tile_h; }
 int fake_tile_x() { return tile_x; }
+int fake_many() { return many; }
 size_t fake_scene_tables(uint8_t* out) {  // the tables the last rasteriser pass that ran has read
   wait();
   if (out) memcpy(out, scene_tables.data(), scene_tables.size());
@@ -172,7 +173,10 @@ void fake_table_entries(jt_ctx* c, int32_t* out) {
 
 // ---- the kernels ----
 namespace jt {
-void launch_mark(const MarkArgs& a, int, int, cudaStream_t) { tile_h = a.views.tile_h; }
+void launch_mark(const MarkArgs& a, int, int, cudaStream_t) {
+  tile_h = a.views.tile_h;
+  many = a.many;
+}
 void launch_scan(const ScanArgs&, cudaStream_t) {}
 void launch_cache_update(const CacheArgs&, int, cudaStream_t) {}
 void launch_decode(const DecodeArgs& a, int warps, int, cudaStream_t) {

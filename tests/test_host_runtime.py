@@ -227,3 +227,29 @@ def test_autotune_times_the_shape_in_use(fake, mcus, warps):
     best, ms = ctx.autotune([(gb, out)], jt.FILTER_BILINEAR, reps=2, stream=0)
     assert ms == 1.0 and (best["decode_mcus_per_warp"], best["decode_warps"]) == (16, 14)
     ctx.close()
+
+
+@pytest.mark.parametrize("sms", [40, 152])
+def test_tiles_go_by_the_device_s_sm_count(fake, sms):
+    import paper_2510_08166_gb300 as jt
+    fake.fake_sm_count(sms)
+    try:
+        ctx = jt.Context(0, 64)
+    finally:
+        fake.fake_sm_count(152)
+    ctx.upload(0, 0, synth.encode(synth.texture(1, 64, 64), 80, 420))
+    for tiles in (4 * sms - 1, 4 * sms, 8 * sms - 1, 8 * sms):  # high tiles of 128 x 32 pixels in a column
+        gb = GBuffer.__new__(GBuffer)
+        one = zeros(16)
+        gb.uv = gb.tex_id = gb.mip = one
+        gb.width, gb.height = 128, 32 * tiles
+        ctx.mark(gb, jt.FILTER_NEAREST, 0)
+        assert fake.fake_tile_h() == (8 if tiles < 4 * sms else 32)
+        assert fake.fake_many() == (tiles >= 8 * sms)
+        ctx.decode(0)
+        s = Scene(1, 2)
+        s.width, s.height = gb.width, gb.height = 1024, 2 * tiles
+        ctx.raster_scene(s, gb, 0)
+        rows = -(-2 * tiles // 8)
+        assert fake.fake_tile_x() == next(x for x in (256, 128, 64, 32) if x == 32 or 1024 // x * rows >= 8 * sms)
+    ctx.close()
