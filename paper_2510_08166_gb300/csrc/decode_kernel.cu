@@ -90,26 +90,6 @@ __device__ __forceinline__ uint32_t bswap(uint32_t w) { return __byte_perm(w, 0,
 __device__ __forceinline__ uint32_t sm_u32(uint32_t off) { return *reinterpret_cast<const uint32_t*>(smem + off); }
 __device__ __forceinline__ int16_t& sm_i16(uint32_t off) { return *reinterpret_cast<int16_t*>(smem + off); }
 
-// Symbol entry by the MAXCODE walk (T.81 F.2.2.3), or kNoEntry for an invalid code or a symbol
-// invalid for the table's class. Only codes without a table entry come here.
-__device__ __noinline__ uint32_t walk_symbol(const HuffWalk* t, uint32_t w, bool dc) {
-  const uint32_t top = w >> 16;
-#pragma unroll 1
-  for (int l = 1; l <= 16; ++l) {
-    const int code = (int)(top >> (16 - l));
-    if (code <= t->maxcode[l]) {
-      const int vi = code + t->valoff[l];
-      if (vi < 0 || vi > 255) return kNoEntry;
-      const uint32_t sym = t->vals[vi];
-      const uint32_t r = dc ? 0 : sym >> 4, s = dc ? sym : sym & 15;
-      if (s > (dc ? 11u : 10u)) return kNoEntry;
-      if (!dc && s == 0) return r == 0 ? huff_entry(l, 0, kRunEob) : (r == 15 ? huff_entry(l, 0, 15) : kNoEntry);
-      return huff_entry(l, s, r);
-    }
-  }
-  return kNoEntry;
-}
-
 // Signed value of a symbol with entry e whose code starts at the top of w (T.81 EXTEND; 0
 // without value bits).
 __device__ __forceinline__ int symbol_value(uint32_t w, uint32_t e) {
@@ -267,11 +247,10 @@ __device__ __noinline__ uint32_t entropy_any(const uint32_t* gw, uint32_t ngw, u
   int du = 0, k = cpt ? 1 : 0;
 #pragma unroll 1
   for (int it = 0; it < 64 * 6; ++it) {  // at most 64 symbols per data unit: each advances k
-    const HuffWalk* t = set->walk + (k == 0 ? 0 : 1) + (du < nl ? 0 : 2);
+    const HuffTable* t = set->table + (k == 0 ? 0 : 1) + (du < nl ? 0 : 2);
     const uint32_t w = __funnelshift_l(word((pos >> 5) + 1), word(pos >> 5), pos & 31u);
     const uint32_t x = table_index<true>(w, __ldg(&t->d), __ldg(&t->cap));
-    uint32_t e = __ldg(reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(set) + __ldg(&t->base)) + x);
-    if (e == kNoEntry) e = walk_symbol(t, w, k == 0);
+    const uint32_t e = __ldg(reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(set) + __ldg(&t->base)) + x);
     if (e == kNoEntry) return kInvalid + (uint32_t)(du + (k > 0 ? 1 : 0));
     const bool val = (e & kSizeMask) != 0;
     const int kst = k + (int)(e >> kRunShift);

@@ -185,7 +185,7 @@ void zigzag_natural(int nat[64]) {
 }
 
 // Table entry of symbol `sym` with a code of length l (kNoEntry when the symbol is invalid for the
-// table's class; the decoder's MAXCODE walk then rejects it).
+// table's class).
 uint16_t symbol_entry(bool dc, int l, uint8_t sym) {
   const int r = dc ? 0 : sym >> 4, s = dc ? sym : sym & 15;
   if ((dc && s > 11) || (!dc && s > 10) || (!dc && s == 0 && r != 0 && r != 15)) return kNoEntry;
@@ -193,9 +193,9 @@ uint16_t symbol_entry(bool dc, int l, uint8_t sym) {
   return huff_entry((uint32_t)l, (uint32_t)s, (uint32_t)r);
 }
 
-// Canonical decode tables of one Huffman spec (T.81 Annex C code assignment): its entries at
-// `lut`, their count, and the walk's tables.
-bool build_table(const jt_huff_spec& spec, bool dc, uint16_t* lut, uint32_t& entries, HuffWalk& t, std::string& why) {
+// Entries of one Huffman spec (T.81 Annex C code assignment) at `lut`, their count, and the table's
+// d and cap.
+bool build_table(const jt_huff_spec& spec, bool dc, uint16_t* lut, uint32_t& entries, HuffTable& t, std::string& why) {
   int n = 0;
   uint64_t kraft = 0;
   for (int l = 1; l <= 16; ++l) {
@@ -210,40 +210,23 @@ bool build_table(const jt_huff_spec& spec, bool dc, uint16_t* lut, uint32_t& ent
     why = "Huffman code lengths violate the Kraft inequality";
     return false;
   }
-  std::memcpy(t.vals, spec.vals, n);
-  // left-aligned start of the codes longer than kLutBits = Kraft mass of the shorter ones;
-  // 65536 (no second granularity) when they take too many prefixes
+  // left-aligned start of the codes longer than kLutBits = Kraft mass of the shorter ones; 65536
+  // (no second granularity) when there are none
   uint32_t first = 0;
   for (int l = 1; l <= kLutBits; ++l) first += (uint32_t)spec.bits[l - 1] << (16 - l);
   const uint32_t end = std::min<uint32_t>((uint32_t)kraft + 1, 65536u);  // one entry past the last code stays empty
-  if (kraft <= first || end - first > (uint32_t)kLut2Size) first = 65536u;
+  if (kraft <= first) first = 65536u;
   t.d = (int32_t)(first >> 6) - (int32_t)first;
   entries = (first >> 6) + (first < 65536u ? end - first : 0u);
   t.cap = (int32_t)entries - 1;
   std::fill(lut, lut + entries, kNoEntry);
-  int code = 0, k = 0;
-  for (int l = 1; l <= 16; ++l) {
-    const int nl = spec.bits[l - 1];
-    if (nl == 0) {
-      t.maxcode[l] = -1;
-      t.valoff[l] = 0;
-    } else {
-      t.valoff[l] = k - code;
-      for (int i = 0; i < nl; ++i, ++k, ++code) {
-        const uint16_t e = symbol_entry(dc, l, spec.vals[k]);
-        if (l <= kLutBits) {
-          const uint32_t at = (uint32_t)code << (kLutBits - l), cnt = 1u << (kLutBits - l);
-          for (uint32_t j = 0; j < cnt; ++j) lut[at + j] = e;
-        } else if (first < 65536u) {
-          const uint32_t at = (uint32_t)((int32_t)((uint32_t)code << (16 - l)) + t.d), cnt = 1u << (16 - l);
-          for (uint32_t j = 0; j < cnt; ++j) lut[at + j] = e;
-        }
-      }
-      t.maxcode[l] = code - 1;
+  uint32_t at16 = 0;  // left-aligned code
+  for (int l = 1, k = 0; l <= 16; ++l)
+    for (int i = 0; i < spec.bits[l - 1]; ++i, ++k, at16 += 1u << (16 - l)) {
+      const uint32_t at = l <= kLutBits ? at16 >> (16 - kLutBits) : (uint32_t)((int32_t)at16 + t.d);
+      const uint32_t cnt = l <= kLutBits ? 1u << (kLutBits - l) : 1u << (16 - l);
+      std::fill(lut + at, lut + at + cnt, symbol_entry(dc, l, spec.vals[k]));
     }
-    code <<= 1;
-  }
-  t.maxcode[0] = -1;
   return true;
 }
 
@@ -253,17 +236,17 @@ bool build_set(const jt_huff_spec huff[4], HuffSet& hs, std::string& why) {
   uint32_t at = 0;
   for (int t = 0; t < 4; ++t) {
     uint32_t entries = 0;
-    if (!build_table(huff[t], t % 2 == 0, hs.lut + at, entries, hs.walk[t], why)) {
+    if (!build_table(huff[t], t % 2 == 0, hs.lut + at, entries, hs.table[t], why)) {
       why = "Huffman table " + std::to_string(t) + ": " + why;
       return false;
     }
-    hs.walk[t].base = (uint32_t)offsetof(HuffSet, lut) + 2 * at;
+    hs.table[t].base = (uint32_t)offsetof(HuffSet, lut) + 2 * at;
     at += entries;
   }
   hs.used = (uint32_t)offsetof(HuffSet, lut) + 2 * at;
-  for (const HuffWalk& w : hs.walk) hs.capped |= 65535 + w.d > w.cap ? 1u : 0u;
+  for (const HuffTable& w : hs.table) hs.capped |= 65535 + w.d > w.cap ? 1u : 0u;
   // data unit i of a chain of nl luma and nc chroma units, then the record past the end
-  HuffWalk none{};
+  HuffTable none{};
   none.base = (uint32_t)offsetof(HuffSet, none);
   none.d = (65536 >> 6) - 65536;
   none.cap = kLutSize - 1;
@@ -274,7 +257,7 @@ bool build_set(const jt_huff_spec huff[4], HuffSet& hs, std::string& why) {
     for (int i = 0; i <= nl + nc; ++i) {
       HuffSeq& q = hs.seq[first + i];
       const bool over = i == nl + nc, final = i + 1 >= nl + nc;
-      const HuffWalk &a = over ? none : hs.walk[ac(i)], &n = final ? none : hs.walk[head(i + 1)], &o = hs.walk[head(i)];
+      const HuffTable &a = over ? none : hs.table[ac(i)], &n = final ? none : hs.table[head(i + 1)], &o = hs.table[head(i)];
       q = HuffSeq{a.base, a.d, n.base, n.d, (!final && apart(i + 1) ? 1u : 0u) << kRunShift, a.cap, n.cap, 0u,
                   o.base, o.d, (apart(i) ? 1u : 0u) << kRunShift, o.cap};
     }

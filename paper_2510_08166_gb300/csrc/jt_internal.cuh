@@ -55,7 +55,7 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 
 constexpr int kLutBits = 10;                 // first-level Huffman LUT: next 10 bits
 constexpr int kLutSize = 1 << kLutBits;
-constexpr int kLut2Size = 4096;              // entries for longer codes, at most
+constexpr int kLut2Size = 256 * 32 + 8;      // entries for longer codes: 256 codes of up to 32 prefixes, one empty
 constexpr int kStreamPadBytes = 64;          // zero padding after each entropy stream
 constexpr uint32_t kUnitBytes = 256;         // cache unit
 constexpr int kSampling420 = 0, kSampling444 = 1, kSamplingCoef = 2;
@@ -77,11 +77,11 @@ constexpr int kSampling420 = 0, kSampling444 = 1, kSamplingCoef = 2;
 // 64), and their entries, one per 16-bit prefix, start where the short ones end, at
 // first >> 6. The index of any code is then max(w >> 22, (w >> 16) + d) with
 // d = (first >> 6) - first: the second term grows 64 times as fast and passes the first one
-// exactly at `first`. So a symbol is one read, without a branch or a select. Codes without
-// an entry (invalid codes, the long codes of a table where they take more than kLut2Size
-// prefixes) and symbols invalid for the table's class (DC category > 11, AC size > 10, AC
-// size 0 with a run other than 0 or 15) go to the MAXCODE walk of T.81 F.2.2.3, which decodes
-// or rejects them.
+// exactly at `first`. So a symbol is one read, without a branch or a select. Every code has its
+// entry, kNoEntry in the place of invalid codes and of symbols invalid for the table's class (DC
+// category > 11, AC size > 10, AC size 0 with a run other than 0 or 15). With room for 4096 entries
+// of longer codes, MCUs that met one of a table with more went through the general chain: 154
+// codes of 11 bits, decode of 576 MCUs 53.4 us (now 17.4), of 23,040 90.5 us (33.6).
 __host__ __device__ constexpr uint16_t huff_entry(uint32_t l, uint32_t s, uint32_t r) {
   return (uint16_t)((l + s) | (s << 5) | (r << 10));
 }
@@ -106,11 +106,8 @@ __host__ __device__ __forceinline__ uint32_t table_index(uint32_t w, int d, int 
 // (kNoEntry): the index as a whole, because past `end` a table of few long codes is
 // shorter than 1 << kLutBits, and there w >> 22 lies beyond it too.
 //
-// The MAXCODE walk's tables of one spec, and where its entries are (byte offset in the set).
-struct HuffWalk {
-  int32_t maxcode[17];  // -1 when no code of length l
-  int32_t valoff[17];
-  uint8_t vals[256];
+// Where one spec's entries are: the byte offset of the first one in the set, d and the last one's index.
+struct HuffTable {
   uint32_t base;
   int32_t d, cap;
   uint32_t pad;
@@ -147,11 +144,11 @@ struct HuffSet {
   uint32_t pad[2];
   uint16_t none[kLutSize];               // zeros: a symbol without value, run or length
   uint16_t lut[4 * kMaxTableEntries];  // the four tables' entries, back to back
-  HuffWalk walk[4];
+  HuffTable table[4];
 };
 static_assert(sizeof(HuffSet) % 16 == 0 && offsetof(HuffSet, lut) % 16 == 0, "copied in 16-byte words");
 // A decode CTA stages one set in shared memory when it is at most this long (the typical tables
-// of the standard take 13,144 bytes).
+// of the standard take 12,828 bytes).
 constexpr uint32_t kStagedTables = 18432;
 
 struct DevDesc {

@@ -159,7 +159,7 @@ void fake_table_entries(jt_ctx* c, int32_t* out) {
   for (auto& v : c->hsets) {
     const HuffSet& hs = v[0];
     for (int t = 0; t < 4; ++t) {
-      const HuffWalk& w = hs.walk[t];
+      const HuffTable& w = hs.table[t];
       const uint32_t first = (w.base - (uint32_t)offsetof(HuffSet, lut)) / 2;
       for (uint32_t p = 0; p < 65536; ++p) {
         const uint32_t x = hs.capped ? table_index<true>(p << 16, w.d, w.cap) : table_index<false>(p << 16, w.d, w.cap);

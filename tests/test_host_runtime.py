@@ -84,6 +84,8 @@ SHAPES = {
     "short only": [4] * 12,
     "complete but for one prefix": list(range(1, 12)) + [16],
     "long only": [13] * 12,
+    "every code long": [11] * 255 + [12],          # (almost) the most prefixes that long codes can take
+    "half of them long": [4] * 8 + [11] * 154,
 }
 
 
@@ -130,6 +132,29 @@ class GBuffer:
     def c(self):
         import paper_2510_08166_gb300 as jt
         return jt.jt_gbuffer(self.uv.data_ptr(), self.tex_id.data_ptr(), self.mip.data_ptr(), self.width, self.height)
+
+
+def test_a_failed_float_pass_leaves_no_counts_to_the_next(fake):
+    import paper_2510_08166_gb300 as jt
+    ctx = jt.Context(0, 1 << 10)
+    ctx.register_coeff_textures(0, 1, 64, 64)
+    gb, coef, out = GBuffer(64, 16), zeros(1, 4, 4, 6, 64), zeros(16, 64, 3)
+    for _ in range(2):
+        ctx.colorize_float(gb, coef, out, 0)
+    for run in (lambda: ctx.colorize_float(gb, coef, out, 0), lambda: ctx.colorize_backward(gb, out, coef, 0)):
+        fake.fake_fail_gather(1)
+        with pytest.raises(jt.JTError):
+            run()
+        fake.fake_fail_gather(0)
+        # a pass that is only captured clears nothing: the eager one after it still has to
+        fake.fake_begin_capture()
+        run()
+        fake.fake_end_capture()
+        run()
+        run()
+        ctx.stats()
+        assert not fake.fake_cursors_dirty()
+    ctx.close()
 
 
 class Scene:
@@ -186,29 +211,6 @@ def test_a_captured_scene_keeps_its_tables(fake):
     assert fake.fake_owned(ctypes.c_void_p(graph)) == 1
     fake.fake_destroy_graph(ctypes.c_void_p(graph))
     assert fake.fake_owned(ctypes.c_void_p(graph)) == 0
-    ctx.close()
-
-
-def test_a_failed_float_pass_leaves_no_counts_to_the_next(fake):
-    import paper_2510_08166_gb300 as jt
-    ctx = jt.Context(0, 1 << 10)
-    ctx.register_coeff_textures(0, 1, 64, 64)
-    gb, coef, out = GBuffer(64, 16), zeros(1, 4, 4, 6, 64), zeros(16, 64, 3)
-    for _ in range(2):
-        ctx.colorize_float(gb, coef, out, 0)
-    for run in (lambda: ctx.colorize_float(gb, coef, out, 0), lambda: ctx.colorize_backward(gb, out, coef, 0)):
-        fake.fake_fail_gather(1)
-        with pytest.raises(jt.JTError):
-            run()
-        fake.fake_fail_gather(0)
-        # a pass that is only captured clears nothing: the eager one after it still has to
-        fake.fake_begin_capture()
-        run()
-        fake.fake_end_capture()
-        run()
-        run()
-        ctx.stats()
-        assert not fake.fake_cursors_dirty()
     ctx.close()
 
 
