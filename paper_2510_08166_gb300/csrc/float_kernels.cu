@@ -26,7 +26,7 @@
 // first-level cache out), entries and gradients are under way while this one is worked on.
 // Measured on sixteen 2048^2 textures under a 1920x1080 plane (244 K MCUs needed, 2.3 M entries,
 // 375 MB of coefficients each way: 55 us): k_float_forward 170 -> 104 us, k_float_backward
-// 198 -> 131 us, the inversion of both passes 275 -> 104 us; both passes 626 -> 384 us. Tried and slower:
+// 198 -> 131 us, the inversion of both passes 275 -> 104 us; both passes 626 -> 365 us. Tried and slower:
 // each entry straight from the coefficients (341 us backward: 48 16-byte shared reads per entry),
 // pairs on a persistent grid (248 us forward), loads through the first-level cache.
 #include <cuda_runtime.h>
@@ -317,15 +317,19 @@ __device__ __forceinline__ void get_row(const float* row, int v, float (&r)[8]) 
   r[4] = hi.x; r[5] = hi.y; r[6] = hi.z; r[7] = hi.w;
 }
 
-// A warp takes kPairs pairs of neighbouring MCUs, one pair at a time; the grid covers all pairs
+// A warp takes a.pairs pairs of neighbouring MCUs, one pair at a time; the grid covers all pairs
 // (a persistent grid waited for its slowest warps: 560 K cycles against 330 K on average).
-// Entry range of lane k < 2 kPairs's MCU m0 + k, whose cursor is zeroed for the next pass's
+// First MCU of this warp.
+__device__ __forceinline__ uint32_t first_mcu(const FloatArgs& a) {
+  return (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (2u * (uint32_t)a.pairs);
+}
+
+// Entry range of lane k < 2 a.pairs's MCU m0 + k, whose cursor is zeroed for the next pass's
 // count: x its first entry, y how many.
-template <int kPairs>
 __device__ __forceinline__ uint2 load_ranges(const FloatArgs& a, uint32_t m0) {
   const uint32_t lane = threadIdx.x & 31, m = m0 + lane;
   uint2 r = make_uint2(0, 0);
-  if (lane < 2 * kPairs && m < a.coef_mcus) {
+  if (lane < 2u * (uint32_t)a.pairs && m < a.coef_mcus) {
     r = make_uint2(a.offset[m], min(a.cursor[m], a.bucket_cap));
     a.cursor[m] = 0;
   }
@@ -341,6 +345,20 @@ struct Pair {
     return j < total() ? __ldcs(a.bucket + (j < n0 ? b0 + j : b1 + (j - n0))) : make_uint4(0, 0, 0, 0);
   }
 };
+
+// The backward's walk of a lane over n entries: from first on by step up to end. Neighbouring entries are
+// mostly neighbouring pixels, so where many pixels fall on a texel (kDense entries in a pair), 32
+// of them at a time would add into one or two addresses: there each lane takes a run of its own
+// (backward, sixteen pixels a texel each way in 40 MCUs: 63.8 ms by 32 neighbours, 5.6 by runs;
+// one pixel a texel, 580 entries in a pair: 91 us, and 123 by runs).
+constexpr uint32_t kDense = 1024;
+struct Walk {
+  uint32_t first, step, end;
+};
+__device__ __forceinline__ Walk walk_of(uint32_t n) {
+  const uint32_t lane = threadIdx.x & 31, run = (n + 31) / 32;
+  return n < kDense ? Walk{lane, 32u, n} : Walk{lane * run, 1u, min(n, lane * run + run)};
+}
 __device__ __forceinline__ Pair pair_of(uint2 r, int p) {
   return Pair{__shfl_sync(0xFFFFFFFFu, r.x, 2 * p), __shfl_sync(0xFFFFFFFFu, r.y, 2 * p), __shfl_sync(0xFFFFFFFFu, r.x, 2 * p + 1), __shfl_sync(0xFFFFFFFFu, r.y, 2 * p + 1)};
 }
@@ -366,13 +384,13 @@ __device__ __forceinline__ void copy16_async(float* to, const float* from) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from) : "memory");
 }
 
-__global__ void __launch_bounds__(kFloatWarps * 32, 4) k_float_forward(const __grid_constant__ FloatArgs a) {
+__global__ void __launch_bounds__(kFloatWarps * 32, kForwardCtas) k_float_forward(const __grid_constant__ FloatArgs a) {
   extern __shared__ __align__(16) float pair_mem[];  // [warps][2][kMcu] texels, [warps][768] coefficients
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* f = pair_mem + warp * (2 * kMcu);
-  float* raw = pair_mem + kFloatWarps * (2 * kMcu) + warp * 768;
-  const uint32_t m0 = (blockIdx.x * kFloatWarps + warp) * (2 * kForwardPairs);
-  const uint2 ranges = load_ranges<kForwardPairs>(a, m0);
+  float* raw = pair_mem + (blockDim.x >> 5) * (2 * kMcu) + warp * 768;
+  const uint32_t m0 = first_mcu(a);
+  const uint2 ranges = load_ranges(a, m0);
   // the next pair's coefficients and first entries are fetched while this one is worked on
   auto fetch = [&](const Pair& r, int p) {
     const float* src = a.coef + (size_t)(m0 + 2u * (uint32_t)p) * 384 + lane * 4;
@@ -385,7 +403,7 @@ __global__ void __launch_bounds__(kFloatWarps * 32, 4) k_float_forward(const __g
   fetch(next, 0);
   uint4 first = next.entry(a, (uint32_t)lane);
 #pragma unroll 1
-  for (int p = 0; p < kForwardPairs; ++p) {
+  for (int p = 0; p < a.pairs; ++p) {
     const Pair r = next;
     uint4 ent = first;
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -401,7 +419,7 @@ __global__ void __launch_bounds__(kFloatWarps * 32, 4) k_float_forward(const __g
       }
       __syncwarp();
     }
-    if (p + 1 < kForwardPairs) {
+    if (p + 1 < a.pairs) {
       next = pair_of(ranges, p + 1);
       fetch(next, p + 1);
       first = next.entry(a, (uint32_t)lane);
@@ -421,6 +439,7 @@ __global__ void __launch_bounds__(kFloatWarps * 32, 4) k_float_forward(const __g
     __syncwarp();
 #pragma unroll 1
     for (uint32_t j = (uint32_t)lane; j < r.total(); j += 32) {
+      const uint4 after = r.entry(a, j + 32);
       const float2 wx = axis_weights(ent.y, kBothX, kLastX, __uint_as_float(ent.z));
       const float2 wy = axis_weights(ent.y, kBothY, kLastY, __uint_as_float(ent.w));
       const EntryPlaces q = places_of(ent.y);
@@ -441,22 +460,22 @@ __global__ void __launch_bounds__(kFloatWarps * 32, 4) k_float_forward(const __g
         atomicAdd(out + 1, grn);
         atomicAdd(out + 2, blu);
       }
-      ent = r.entry(a, j + 32);
+      ent = after;
     }
     __syncwarp();  // the pair's memory is written again
   }
 }
 
-__global__ void __launch_bounds__(kFloatWarps * 32, 5) k_float_backward(const __grid_constant__ FloatArgs a) {
+__global__ void __launch_bounds__(kFloatWarps * 32, kBackwardCtas) k_float_backward(const __grid_constant__ FloatArgs a) {
   extern __shared__ __align__(16) float pair_mem[];  // [warps][2][kMcu]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* f = pair_mem + warp * (2 * kMcu);
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-  const uint32_t m0 = (blockIdx.x * kFloatWarps + warp) * (2 * kBackwardPairs);
-  const uint2 ranges = load_ranges<kBackwardPairs>(a, m0);
+  const uint32_t m0 = first_mcu(a);
+  const uint2 ranges = load_ranges(a, m0);
   // the next pair's first entries and their pixels' gradients are fetched ahead
   Pair next = pair_of(ranges, 0);
-  uint4 first = next.entry(a, (uint32_t)lane);
+  uint4 first = next.entry(a, walk_of(next.total()).first);
   float3 grad;
   auto fetch = [&](uint32_t px) {
     const float* gf = a.frame + 3 * (size_t)px;
@@ -464,14 +483,15 @@ __global__ void __launch_bounds__(kFloatWarps * 32, 5) k_float_backward(const __
   };
   fetch(first.x);
 #pragma unroll 1
-  for (int p = 0; p < kBackwardPairs; ++p) {
+  for (int p = 0; p < a.pairs; ++p) {
     const uint32_t m = m0 + 2u * (uint32_t)p;
     if (m >= a.coef_mcus) break;
     const Pair r = next;
-    uint4 ent = first;
-    if (p + 1 < kBackwardPairs) {
+    const Walk w = walk_of(r.total());
+    uint4 ent = first, after = r.entry(a, w.first + w.step);
+    if (p + 1 < a.pairs) {
       next = pair_of(ranges, p + 1);
-      first = next.entry(a, (uint32_t)lane);
+      first = next.entry(a, walk_of(next.total()).first);
     }
     if (r.total()) {
 #pragma unroll
@@ -480,17 +500,18 @@ __global__ void __launch_bounds__(kFloatWarps * 32, 5) k_float_backward(const __
       }
       __syncwarp();
 #pragma unroll 1
-      for (uint32_t j = (uint32_t)lane; j < r.total(); j += 32) {
+      for (uint32_t j = w.first; j < w.end; j += w.step) {
         const float gy = grad.x + grad.y + grad.z, gcb = kCb2B * grad.z - kCb2G * grad.y, gcr = kCr2R * grad.x - kCr2G * grad.y;
         float2 wx = axis_weights(ent.y, kBothX, kLastX, __uint_as_float(ent.z));
         float2 wy = axis_weights(ent.y, kBothY, kLastY, __uint_as_float(ent.w));
         const EntryPlaces q = places_of(ent.y);
         float* g = f + (j < r.n0 ? 0 : kMcu);
         const bool bx = (ent.y & kBothX) != 0, by = (ent.y & kBothY) != 0;
-        if (j + 32 < r.total()) {
-          ent = r.entry(a, j + 32);
-          fetch(ent.x);
-        }
+        // the next entry's gradient and the entry after it are under way during this one's sums (one
+        // after the other at the head of the loop they took longer than the sums)
+        ent = after;
+        fetch(ent.x);
+        after = r.entry(a, j + 2 * w.step);
         atomicAdd(g + q.y[0] + q.x[0], wx.x * wy.x * gy);
         if (bx) atomicAdd(g + q.y[0] + q.x[1], wx.y * wy.x * gy);
         if (by) atomicAdd(g + q.y[1] + q.x[0], wx.x * wy.y * gy);
@@ -550,8 +571,7 @@ __global__ void __launch_bounds__(kFloatWarps * 32, 5) k_float_backward(const __
   }
 }
 
-constexpr size_t kPairSmem = (size_t)kFloatWarps * 2 * kMcu * sizeof(float);
-constexpr size_t kForwardSmem = kPairSmem + (size_t)kFloatWarps * 768 * sizeof(float);
+constexpr size_t kBackwardSmem = 2 * kMcu * sizeof(float), kForwardSmem = kBackwardSmem + 768 * sizeof(float);  // a warp
 
 void launch_inversion(const FloatArgs& a, int threads, int pixel_grid, cudaStream_t s) {
   const int blocks = (int)((a.coef_mcus + kFloatScan - 1) / kFloatScan);
@@ -561,29 +581,39 @@ void launch_inversion(const FloatArgs& a, int threads, int pixel_grid, cudaStrea
   k_float_fill<<<pixel_grid, std::min(threads, 512), 0, s>>>(a);  // (its registers allow no more)
 }
 
-int gather_grid(const FloatArgs& a, int pairs) {
-  const uint32_t mcus = (uint32_t)(kFloatWarps * 2 * pairs);
-  return (int)((a.coef_mcus + mcus - 1) / mcus);
+// Launches a gather of `ctas` resident CTAs per SM with up to `most` pairs for each warp: fewer where
+// there are not enough to fill the chip, then smaller CTAs, so that few MCUs (which then hold many
+// entries) spread over its SMs. One 1080p frame, forward / backward: one 128^2 texture (64 MCUs)
+// 7.9 / 29.1 ms with the most pairs and whole CTAs, 1.7 / 3.9 so; one of 512^2 723 / 1430 us, 246 / 402;
+// two of 1024^2 184 / 262 us, 108 / 143.
+void launch_gather(void (*gather)(FloatArgs), FloatArgs a, int most, int ctas, size_t warp_smem, cudaStream_t s) {
+  const uint64_t pairs = ((uint64_t)a.coef_mcus + 1) / 2, sms = (uint64_t)a.sms;
+  for (a.pairs = most; a.pairs > 1 && pairs < sms * ctas * kFloatWarps * a.pairs; a.pairs /= 2) {
+  }
+  const uint64_t tasks = (pairs + a.pairs - 1) / a.pairs;
+  int warps = kFloatWarps;
+  while (warps > 1 && tasks < sms * warps) warps /= 2;
+  gather<<<(int)((tasks + warps - 1) / warps), warps * 32, warps * warp_smem, s>>>(a);
 }
 
 }  // namespace
 
 // Sets the gather kernels' shared-memory attributes on the current device.
 bool float_configure() {
-  return cudaFuncSetAttribute(k_float_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kForwardSmem) == cudaSuccess &&
-         cudaFuncSetAttribute(k_float_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem) == cudaSuccess;
+  return cudaFuncSetAttribute(k_float_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kFloatWarps * kForwardSmem)) == cudaSuccess &&
+         cudaFuncSetAttribute(k_float_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kFloatWarps * kBackwardSmem)) == cudaSuccess;
 }
 
 // The cursors must be zero on entry (the gathers leave them so; after a failed launch the caller
 // clears them), and the forward's frame.
 void launch_float_forward(const FloatArgs& a, int threads, int pixel_grid, cudaStream_t s) {
   launch_inversion(a, threads, pixel_grid, s);
-  k_float_forward<<<gather_grid(a, kForwardPairs), kFloatWarps * 32, kForwardSmem, s>>>(a);
+  launch_gather(k_float_forward, a, kForwardPairs, kForwardCtas, kForwardSmem, s);
 }
 
 void launch_float_backward(const FloatArgs& a, int threads, int pixel_grid, cudaStream_t s) {
   launch_inversion(a, threads, pixel_grid, s);
-  k_float_backward<<<gather_grid(a, kBackwardPairs), kFloatWarps * 32, kPairSmem, s>>>(a);
+  launch_gather(k_float_backward, a, kBackwardPairs, kBackwardCtas, kBackwardSmem, s);
 }
 
 }  // namespace jt

@@ -604,6 +604,7 @@ jt_status float_setup(jt_ctx* c, const jt_gbuffer* g, const float* in, const flo
   a.cursor = c->float_cursor;
   a.offset = c->float_offset;
   a.block_sum = c->float_sums;
+  a.sms = c->sm_count;
   a.state = c->state;
   // orthonormal 8-point DCT-III basis, A[x][u] = C(u)/2 cos((2x+1) u pi / 16)
   const double pi = 3.14159265358979323846;

@@ -382,12 +382,15 @@ struct FloatArgs {
   uint64_t* block_sum;    // [ceil(coef_mcus / kFloatScan)] needed MCUs << 32 | entries
   uint4* bucket;          // [bucket_cap] entries
   uint32_t bucket_cap;    // >= 4 pixels of the view (a pixel's taps touch at most 4 MCUs)
+  int sms;                // SMs of the device
+  int pairs;              // pairs of MCUs per warp of a gather (chosen by its launcher)
   float basis[64];        // A[x][u] = C(u)/2 cos((2x+1)u pi/16), C(0) = 1/sqrt(2); x*8+u
 };
 // JFIF colour of the float chain: R = Y + kCr2R Cr, G = Y - kCb2G Cb - kCr2G Cr, B = Y + kCb2B Cb
 constexpr float kCr2R = 1.402f, kCb2G = 0.344136f, kCr2G = 0.714136f, kCb2B = 1.772f;
 constexpr int kFloatWarps = 8;     // warps per CTA of the gathers
-constexpr int kForwardPairs = 8, kBackwardPairs = 4;  // pairs of MCUs per warp there (2: 152/152 us, 4: 115/131, 8: 104/140, 16: 107/169)
+constexpr int kForwardCtas = 4, kBackwardCtas = 5;    // CTAs per SM there
+constexpr int kForwardPairs = 8, kBackwardPairs = 4;  // pairs of MCUs per warp there, at most (2: 152/152 us, 4: 115/131, 8: 104/140, 16: 107/169)
 constexpr int kFloatScan = 1024;   // counts per CTA of the scan (256 threads x 4)
 bool float_configure();
 void launch_float_forward(const FloatArgs& a, int threads, int pixel_grid, cudaStream_t s);
