@@ -380,6 +380,12 @@ __device__ __forceinline__ EntryPlaces places_of(uint32_t info) {
   return q;
 }
 
+// Values that are not finite spread by the taps of weight zero (0 * inf), which the sums below add as they
+// are: where one is met, the sum is taken tap by tap.
+__device__ __forceinline__ bool finite3(float a, float b, float c) {
+  return fabsf(a) + fabsf(b) + fabsf(c) < __int_as_float(0x7F800000);
+}
+
 __device__ __forceinline__ void copy16_async(float* to, const float* from) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from) : "memory");
 }
@@ -449,7 +455,20 @@ __global__ void __launch_bounds__(kFloatWarps * 32, kForwardCtas) k_float_forwar
       };
       const float Y = fmaf(128.f, (wx.x + wx.y) * (wy.x + wy.y), sum(t, q.x, q.y));
       const float cb = sum(t, q.cx, q.cy), cr = sum(t + kDu, q.cx, q.cy);
-      const float red = fmaf(kCr2R, cr, Y), grn = fmaf(-kCr2G, cr, fmaf(-kCb2G, cb, Y)), blu = fmaf(kCb2B, cb, Y);
+      float red = fmaf(kCr2R, cr, Y), grn = fmaf(-kCr2G, cr, fmaf(-kCb2G, cb, Y)), blu = fmaf(kCb2B, cb, Y);
+      if (!finite3(red, grn, blu)) {  // tap by tap, without those of weight zero
+        red = grn = blu = 0.f;
+#pragma unroll 1
+        for (int k = 0; k < 4; ++k) {
+          const float w = (k & 1 ? wx.y : wx.x) * (k & 2 ? wy.y : wy.x);
+          if (w == 0.f) continue;
+          const float* c = t + (k & 1 ? q.cx[1] : q.cx[0]) + (k & 2 ? q.cy[1] : q.cy[0]);
+          const float y = t[(k & 1 ? q.x[1] : q.x[0]) + (k & 2 ? q.y[1] : q.y[0])] + 128.f;
+          red = fmaf(w, fmaf(kCr2R, c[kDu], y), red);
+          grn = fmaf(w, fmaf(-kCr2G, c[kDu], fmaf(-kCb2G, c[0], y)), grn);
+          blu = fmaf(w, fmaf(kCb2B, c[0], y), blu);
+        }
+      }
       float* out = a.frame + 3 * (size_t)ent.x;
       if ((ent.y & (kBothX | kBothY)) == (kBothX | kBothY)) {  // the pixel's only entry
         out[0] = red;
@@ -512,6 +531,18 @@ __global__ void __launch_bounds__(kFloatWarps * 32, kBackwardCtas) k_float_backw
         ent = after;
         fetch(ent.x);
         after = r.entry(a, j + 2 * w.step);
+        if (!finite3(gy, gcb, gcr)) {
+#pragma unroll 1
+          for (int k = 0; k < 4; ++k) {
+            const float v = (k & 1 ? wx.y : wx.x) * (k & 2 ? wy.y : wy.x);
+            if (v == 0.f) continue;
+            float* c = g + (k & 1 ? q.cx[1] : q.cx[0]) + (k & 2 ? q.cy[1] : q.cy[0]);
+            atomicAdd(g + (k & 1 ? q.x[1] : q.x[0]) + (k & 2 ? q.y[1] : q.y[0]), v * gy);
+            atomicAdd(c, v * gcb);
+            atomicAdd(c + kDu, v * gcr);
+          }
+          continue;
+        }
         atomicAdd(g + q.y[0] + q.x[0], wx.x * wy.x * gy);
         if (bx) atomicAdd(g + q.y[0] + q.x[1], wx.y * wy.x * gy);
         if (by) atomicAdd(g + q.y[1] + q.x[0], wx.x * wy.y * gy);
