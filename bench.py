@@ -752,6 +752,12 @@ def run_motion(jt, ts, dev, flush, stream, reps=100, stereo=False):
     return res
 
 
+def bucket_bytes(npx: int) -> float:
+    """Bytes of the float chain's bucket entries in one pass over npx pixels, at most: up to four
+    a pixel of 16 bytes each, written once and read once."""
+    return 4 * npx * 2 * 16.0
+
+
 def run_adjoint(jt, dev, flush, stream, steps, peak):
     """Differentiable colourise: 16 coefficient textures 2048^2 (float32 dequantised DCT,
     403 MB), 1920x1080 perspective plane, bilinear; forward F, then the adjoint of
@@ -779,9 +785,9 @@ def run_adjoint(jt, dev, flush, stream, steps, peak):
     # G-buffer twice, each needed MCU's coefficients once and writes the frame.
     bwd_bytes = 4.0 * c.numel() + 2 * 11.0 * npx + 12.0 * npx
     fwd_bytes = 2 * 11.0 * npx + needed * 1536.0 + 12.0 * npx
-    # intermediate traffic, kept out of the method's bytes: both passes' bucket entries (32 B
+    # intermediate traffic, kept out of the method's bytes: both passes' bucket entries (16 B
     # per pixel and needed MCU its taps touch, written and read once; at most four per pixel)
-    bucket_bytes_max = 4 * npx * 2 * 32.0
+    bucket_bytes_max = bucket_bytes(npx)
     ctx.close()
     ach = bwd_bytes / (ms_bwd * 1e-3) / 1e9
     return {"workload": "16 coefficient textures 2048^2 4:2:0 (float32 [16,128,128,6,64]), 1920x1080 plane, "

@@ -30,6 +30,7 @@ int sm_count = 152, fast_mcus = 0, fast_warps = 0, run_mcus = 0, run_warps = 0;
 bool fail_gather = false, cursors_dirty = false;
 std::vector<uint8_t> scene_tables;
 int tile_x = 0, tile_h = 0, many = 0;
+size_t last_malloc = 0;
 
 void put(std::function<void()> f) { (capture ? capture->ops : pending).push_back(std::move(f)); }
 cudaError_t wait() {
@@ -75,7 +76,7 @@ cudaError_t cudaGetLastError() {
   last_error = cudaSuccess;
   return e;
 }
-cudaError_t cudaMalloc(void** p, size_t n) { return *p = calloc(n, 1), cudaSuccess; }
+cudaError_t cudaMalloc(void** p, size_t n) { return *p = calloc(last_malloc = n, 1), cudaSuccess; }
 cudaError_t cudaFree(void* p) { return wait(), free(p), cudaSuccess; }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { return wait(), memcpy(d, s, n), cudaSuccess; }
 cudaError_t cudaMemset(void* d, int v, size_t n) { return wait(), memset(d, v, n), cudaSuccess; }
@@ -142,6 +143,7 @@ int fake_cursors_dirty() { return cursors_dirty; }
 int fake_tile_h() { return tile_h; }
 int fake_tile_x() { return tile_x; }
 int fake_many() { return many; }
+size_t fake_last_malloc() { return last_malloc; }
 size_t fake_scene_tables(uint8_t* out) {  // the tables the last rasteriser pass that ran has read
   wait();
   if (out) memcpy(out, scene_tables.data(), scene_tables.size());

@@ -33,7 +33,7 @@ def fake_library(tmp_path_factory):
             f.argtypes = argtypes
             f.restype = ctypes.c_char_p if name in ("jt_last_error", "jt_status_string") else ctypes.c_int
     lib.fake_begin_capture.restype = ctypes.c_void_p
-    lib.fake_scene_tables.restype = ctypes.c_size_t
+    lib.fake_scene_tables.restype = lib.fake_last_malloc.restype = ctypes.c_size_t
     return lib
 
 
@@ -254,4 +254,15 @@ def test_tiles_go_by_the_device_s_sm_count(fake, sms):
         ctx.raster_scene(s, gb, 0)
         rows = -(-2 * tiles // 8)
         assert fake.fake_tile_x() == next(x for x in (256, 128, 64, 32) if x == 32 or 1024 // x * rows >= 8 * sms)
+    ctx.close()
+
+
+def test_the_bench_counts_the_bucket_that_the_library_allocates(fake, monkeypatch):
+    import paper_2510_08166_gb300 as jt
+    monkeypatch.syspath_prepend(ROOT)
+    import bench
+    ctx = jt.Context(0, 1 << 10)
+    ctx.register_coeff_textures(0, 1, 64, 64)
+    ctx.colorize_float(GBuffer(64, 16), zeros(1, 4, 4, 6, 64), zeros(16, 64, 3), 0)
+    assert bench.bucket_bytes(64 * 16) == 2 * fake.fake_last_malloc()  # written once and read once
     ctx.close()
