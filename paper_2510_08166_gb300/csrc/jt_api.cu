@@ -315,21 +315,22 @@ jt_status sync_descs(jt_ctx* c) {
 }
 
 // Device copies of the Huffman sets and quantisation tables: grown by doubling, and only the
-// sets added since the last call are copied.
+// sets added since the last call are copied. When memory runs out the copies stay as they were, for the
+// levels that use them.
 template <typename T, typename V>
 jt_status sync_sets(jt_ctx* c, T*& dev, size_t& cap, size_t& have, const V& sets, size_t bytes) {
   const size_t n = sets.size();
   if (dev && have == n) return JT_OK;
   ++c->generation;
   if (!dev || n > cap) {
+    T* grown = nullptr;
+    const size_t grown_cap = std::max<size_t>({n, 2 * cap, 1});
+    jt_status s = dev_alloc(c, &grown, grown_cap * bytes);
+    if (s != JT_OK) return s;
     dev_free(dev);
+    dev = grown;
+    cap = grown_cap;
     have = 0;
-    cap = std::max<size_t>({n, 2 * cap, 1});
-    jt_status s = dev_alloc(c, &dev, cap * bytes);
-    if (s != JT_OK) {
-      cap = 0;
-      return s;
-    }
   }
   for (; have < n; ++have)
     JT_CUDA(c, cudaMemcpy(reinterpret_cast<uint8_t*>(dev) + have * bytes, sets[have].data(), bytes,
@@ -922,29 +923,23 @@ static jt_status upload_level(jt_ctx* c, int tex_id, int level, int width, int h
   int qset = -1;
   for (size_t i = 0; i < c->qsets.size(); ++i)
     if (c->qsets[i] == qz) qset = (int)i;
-  bool tables_changed = false;
   if (hset < 0) {
     if (c->hsets.size() >= 255) return fail(c, JT_ERR_UNSUPPORTED, "more than 255 distinct Huffman table sets");
     c->hsets.push_back(std::move(hs));
     c->huff_specs.push_back(specs);
     hset = (int)c->hsets.size() - 1;
-    tables_changed = true;
   }
   if (qset < 0) {
     if (c->qsets.size() >= 255) return fail(c, JT_ERR_UNSUPPORTED, "more than 255 distinct quantisation tables");
     c->qsets.push_back(qz);
     qset = (int)c->qsets.size() - 1;
-    tables_changed = true;
   }
-  if (tables_changed) {
-    jt_status s = sync_tables(c);
-    if (s != JT_OK) return s;
-  }
+  jt_status s = sync_tables(c);
+  if (s != JT_OK) return s;
 
   // stream words (zero padded) and side table
   Level L{tex_id, level};
   const uint64_t words = (nbytes + 3) / 4 + kStreamPadBytes / 4;
-  jt_status s;
   if ((s = dev_alloc(c, reinterpret_cast<uint8_t**>(&L.stream_mem), words * 4)) != JT_OK) return s;
   if ((s = dev_alloc(c, reinterpret_cast<uint8_t**>(&L.index_mem), side_bytes + 16)) != JT_OK) {
     cudaFree(L.stream_mem);

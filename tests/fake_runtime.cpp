@@ -30,7 +30,8 @@ int sm_count = 152, fast_mcus = 0, fast_warps = 0, run_mcus = 0, run_warps = 0;
 bool fail_gather = false, cursors_dirty = false;
 std::vector<uint8_t> scene_tables;
 int tile_x = 0, tile_h = 0, many = 0;
-size_t last_malloc = 0;
+size_t last_malloc = 0, fail_malloc = 0;
+int tables_on_device = 0;
 
 void put(std::function<void()> f) { (capture ? capture->ops : pending).push_back(std::move(f)); }
 cudaError_t wait() {
@@ -76,7 +77,10 @@ cudaError_t cudaGetLastError() {
   last_error = cudaSuccess;
   return e;
 }
-cudaError_t cudaMalloc(void** p, size_t n) { return *p = calloc(last_malloc = n, 1), cudaSuccess; }
+cudaError_t cudaMalloc(void** p, size_t n) {
+  if (fail_malloc && n >= fail_malloc) return fail_malloc = 0, last_error = cudaErrorMemoryAllocation;
+  return *p = calloc(last_malloc = n, 1), cudaSuccess;
+}
 cudaError_t cudaFree(void* p) { return wait(), free(p), cudaSuccess; }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { return wait(), memcpy(d, s, n), cudaSuccess; }
 cudaError_t cudaMemset(void* d, int v, size_t n) { return wait(), memset(d, v, n), cudaSuccess; }
@@ -144,6 +148,9 @@ int fake_tile_h() { return tile_h; }
 int fake_tile_x() { return tile_x; }
 int fake_many() { return many; }
 size_t fake_last_malloc() { return last_malloc; }
+void fake_fail_malloc(size_t n) { fail_malloc = n; }  // the next allocation of n bytes or more
+size_t fake_set_bytes() { return sizeof(HuffSet); }
+int fake_tables_on_device() { return wait(), tables_on_device; }
 size_t fake_scene_tables(uint8_t* out) {  // the tables the last rasteriser pass that ran has read
   wait();
   if (out) memcpy(out, scene_tables.data(), scene_tables.size());
@@ -182,7 +189,12 @@ void launch_mark(const MarkArgs& a, int, int, cudaStream_t) {
 void launch_scan(const ScanArgs&, cudaStream_t) {}
 void launch_cache_update(const CacheArgs&, int, cudaStream_t) {}
 void launch_decode(const DecodeArgs& a, int warps, int, cudaStream_t) {
-  put([m = a.mcus_per_warp, warps] { run_mcus = m, run_warps = warps; });
+  put([a, m = a.mcus_per_warp, warps] {
+    run_mcus = m, run_warps = warps;
+    tables_on_device = 0;  // of the levels' sets, those that the decoder finds
+    for (uint32_t d = 0, seen = 0; a.huff && a.quant && d < a.ndesc; ++d)
+      if (!(seen >> a.descs[d].hset & 1) && a.huff[a.descs[d].hset].used != 0) ++tables_on_device, seen |= 1u << a.descs[d].hset;
+  });
 }
 void launch_colorize(const ColorizeArgs&, int, int, cudaStream_t) {}
 void launch_raster(const RasterArgs& a, cudaStream_t) {

@@ -33,7 +33,7 @@ def fake_library(tmp_path_factory):
             f.argtypes = argtypes
             f.restype = ctypes.c_char_p if name in ("jt_last_error", "jt_status_string") else ctypes.c_int
     lib.fake_begin_capture.restype = ctypes.c_void_p
-    lib.fake_scene_tables.restype = lib.fake_last_malloc.restype = ctypes.c_size_t
+    lib.fake_scene_tables.restype = lib.fake_last_malloc.restype = lib.fake_set_bytes.restype = ctypes.c_size_t
     return lib
 
 
@@ -265,4 +265,22 @@ def test_the_bench_counts_the_bucket_that_the_library_allocates(fake, monkeypatc
     ctx.register_coeff_textures(0, 1, 64, 64)
     ctx.colorize_float(GBuffer(64, 16), zeros(1, 4, 4, 6, 64), zeros(16, 64, 3), 0)
     assert bench.bucket_bytes(64 * 16) == 2 * fake.fake_last_malloc()  # written once and read once
+    ctx.close()
+
+
+def test_an_upload_after_one_that_ran_out_of_memory_has_its_tables(fake):
+    import paper_2510_08166_gb300 as jt
+    ctx, gb = jt.Context(0, 64), GBuffer(64, 64)
+    encs = [synth.encode(synth.texture(1, 64, 64), q, 420) for q in (80, 50)]
+    encs[1].huff_bits, encs[1].huff_vals = encs[1].huff_bits.copy(), encs[1].huff_vals.copy()
+    encs[1].huff_bits[0], encs[1].huff_vals[0] = spec([4] * 12, DC)
+    ctx.upload(0, 0, encs[0])
+    fake.fake_fail_malloc(ctypes.c_size_t(fake.fake_set_bytes()))  # the tables grow for the second set
+    with pytest.raises(jt.JTError):
+        ctx.upload(1, 0, encs[1])
+    for t in range(2):  # the first texture is as it was, and the second one can be uploaded again
+        ctx.mark(gb, jt.FILTER_NEAREST, 0)
+        ctx.decode(0)
+        assert fake.fake_tables_on_device() == t + 1
+        ctx.upload(1 + t, 0, encs[1])
     ctx.close()
