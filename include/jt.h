@@ -122,7 +122,8 @@ typedef struct {
                                    width): 4, 8, 16 or 32; a short list runs fewer per warp */
   int32_t decode_warps;         /* warps per decode CTA: 1..16 (the CTA must fit shared memory) */
   int32_t decode_ctas_per_sm;   /* resident decode CTAs per SM of the persistent grid (>= 1) */
-  int32_t pixel_threads;        /* threads per CTA of mark and colourise (64..1024, mult. of 32) */
+  int32_t pixel_threads;        /* threads per CTA of mark and colourise (64..1024, mult. of 32;
+                                   above 512 they run with 512, as does the float chain's fill) */
   int32_t pixel_ctas_per_sm;    /* CTAs per SM of the grid-stride mark and colourise grids */
   int32_t decode_short_lists;   /* -1 (default), 0 or 1: accepted and without effect. One kernel
                                    serves lists of every length; a short list runs one MCU per

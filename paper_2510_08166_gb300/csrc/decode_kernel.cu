@@ -784,7 +784,11 @@ size_t decode_smem_bytes(int warps, int mcus_per_warp) { return smem_bytes(warps
 // as kLongRun full batches for every warp. It takes 32 MCUs a batch, so that the set-up's dependent
 // loads serve twice as many, and packs 4:4:4 ones, so that all lanes decode: 1440 -> 1376 us for
 // eight 4096^2 textures to pixels, half of them 4:4:4 (1.3 M MCUs). It is a kernel of its own
-// because the parts cost a short list time (1080p frame 54.4 -> 54.9 us in one kernel).
+// because the parts cost a short list time (1080p frame 54.4 -> 54.9 us in one kernel), which a
+// short list of a context that can have long ones still pays: the host does not know a list's length.
+// Hence the line at ten full batches a warp, well above where the two forms meet (textures to pixels
+// with every list taken as the one kind or the other, default shape: 1.2 batches 78.2 us, 84.9 as long;
+// 2.4 111.1, 112.6; 4.8 221.2, 213.5; 9.6 391.1, 381.1; 19 733, 705; 38 1425, 1361).
 void launch_decode(const DecodeArgs& a, int warps, int grid, cudaStream_t s) {
   const size_t smem_b = smem_bytes(warps, a.mcus_per_warp);
   const uint64_t most = std::min<uint64_t>(a.ngid, a.cap_units), batch = (uint64_t)grid * (uint32_t)(warps * a.mcus_per_warp);

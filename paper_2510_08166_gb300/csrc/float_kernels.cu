@@ -26,7 +26,7 @@
 // first-level cache out), entries and gradients are under way while this one is worked on.
 // Measured on sixteen 2048^2 textures under a 1920x1080 plane (244 K MCUs needed, 2.3 M entries,
 // 375 MB of coefficients each way: 55 us): k_float_forward 170 -> 104 us, k_float_backward
-// 198 -> 131 us, the inversion of both passes 275 -> 104 us; both passes 626 -> 365 us. Tried and slower:
+// 198 -> 131 us, the inversion of both passes 275 -> 104 us; both passes 626 -> 370 us. Tried and slower:
 // each entry straight from the coefficients (341 us backward: 48 16-byte shared reads per entry),
 // pairs on a persistent grid (248 us forward), loads through the first-level cache.
 #include <cuda_runtime.h>

@@ -128,7 +128,12 @@ constexpr int kSeen = 1024;  // per-CTA table of recently flagged gids
 // (in a branch of their own they made the kernel slower than the plain form: 50.9 against
 // 42.7 us on the 4K frame of 64 textures, bilinear). Measured: 42.7 -> 27.9 us on that frame
 // (43 % of the HBM rate, long_scoreboard first among its stalls), 395 -> 286 us for the
-// nearest texels of eight 4096^2 views (63 %).
+// nearest texels of eight 4096^2 views (63 %). Where most quads have to wait the plain form was
+// faster: one level seen without mips (20 texels from pixel to pixel, 4K, nearest 44.6 us, 53.9
+// now; bilinear 64.0, 75.7), another texture at every pixel (31.0, 41.3). Taking such segments
+// from the registers, from the caches or pixel by pixel won most of that back, but each of ten
+// forms cost ordinary frames 0.3 to 3 % (more registers or a vote in the box's path), and the frames
+// of those contents are as fast as with the plain form or faster.
 
 // One pixel on its own: flag(g) for every MCU its taps fall in.
 template <int FILTER, typename F>
@@ -311,7 +316,8 @@ __device__ __forceinline__ uint32_t blend_h(uint32_t c00, uint32_t c10, uint32_t
 // pixels of a lane overlap their chains: the four slots are read whether or not the footprint
 // straddles MCUs (the same address twice where it does not, an L1 hit), which costs less than
 // the comparisons, predicates and selects that would spare the reads (the ALU pipe bounds the
-// pass). Any slot is in range, of an MCU no pixel needs too (a stale one), and a pixel that
+// pass; of a G-buffer of noise, where every lane's reads are lines of their own, the pass takes 131 us
+// at 4K, 116 with predicates). Any slot is in range, of an MCU no pixel needs too (a stale one), and a pixel that
 // is not shaded reads the first slots and gathers from wherever they point.
 // S: log2 of the MCU side when every level has the same, else -1.
 template <int FILTER, int S>
