@@ -41,12 +41,12 @@ WORKLOAD = "4K frame 3840x2160, 64 JPEG textures 1024-4096^2 Q50-95 4:2:0 full m
 # DRAM bytes (read + write) per launch of each pass's kernel in an ncu capture of this workload
 # with the current kernel code (the summaries under profiles/). A kernel changed since its
 # capture must be set back to None.
-NCU_TRAFFIC = {"mark": None, "compact": 5.45e6, "decode": None, "colorize": None}
-# From one ncu capture of k_decode on the 4K frame in the decode shape the autotuner picks
-# (16 MCUs per warp, 12 warps per CTA, 1 CTA per SM): warp instructions executed, issue
-# slots busy (% of active cycles) and the frame's symbols; None until captured for the
-# current kernel code (see profiles/).
-NCU_DECODE = {"warp_instructions": None, "issue_active_pct": None, "symbols": 1257771}
+NCU_TRAFFIC = {"mark": 93.54e6, "compact": 5.45e6, "decode": 2.08e6, "colorize": 122.06e6}
+# From one ncu capture of k_decode on the 4K frame in a decode shape the autotuner picked (16
+# MCUs per warp, 6 warps per CTA, 2 CTAs per SM): warp instructions executed, issue slots busy
+# (% of active cycles) and the frame's symbols; None until captured for the current kernel
+# code (see profiles/).
+NCU_DECODE = {"warp_instructions": 16895493, "issue_active_pct": 52.4, "symbols": 1257771}
 
 
 # kernels one frame launches: mark, the compaction's two passes, decode, colourise
