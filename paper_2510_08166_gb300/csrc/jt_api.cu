@@ -1115,11 +1115,12 @@ jt_status jt_raster_scene(jt_ctx* c, const jt_scene* sc, const jt_gbuffer* out, 
   std::vector<uint8_t>* host = nullptr;
   jt_status s = cap == cudaStreamCaptureStatusActive ? scene_host_of_graph(c, graph, host) : scene_host_of_call(c, host);
   if (s != JT_OK) return s;
-  host->assign(need, 0);
+  host->resize(need);  // (every byte is written below)
   for (int t = 0; t < sc->ntex; ++t) {
     const float wh[2] = {(float)sc->tex_w[t], (float)sc->tex_h[t]};
+    const int32_t levels[2] = {sc->tex_levels[t], 0};
     std::memcpy(host->data() + (size_t)t * 16, wh, 8);
-    std::memcpy(host->data() + (size_t)t * 16 + 8, &sc->tex_levels[t], 4);
+    std::memcpy(host->data() + (size_t)t * 16 + 8, levels, 8);
   }
   if (sc->nquads) std::memcpy(host->data() + qoff, sc->quads, (size_t)sc->nquads * sizeof(SceneQuad));
   JT_CUDA(c, cudaMemcpyAsync(c->raster_buf, host->data(), need, cudaMemcpyHostToDevice, st));
