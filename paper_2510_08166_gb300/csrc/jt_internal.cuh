@@ -94,13 +94,11 @@ template <bool CAP>
 __host__ __device__ __forceinline__ uint32_t table_index(uint32_t w, int d, int cap) {
   const int t = (int)(w >> 16), i = (int)(w >> (32 - kLutBits));
 #ifdef __CUDA_ARCH__
-  // (both terms capped, side by side: the cap after the maximum is one step longer on the symbols' chain,
-  // 1 % of a small frame with tables of its own)
-  return (uint32_t)(CAP ? max(__viaddmin_s32(t, d, cap), min(i, cap)) : __viaddmax_s32(t, d, i));
+  const int x = __viaddmax_s32(t, d, i);
 #else
-  const int x = CAP && t + d > cap ? cap : t + d, y = CAP && i > cap ? cap : i;
-  return (uint32_t)(x > y ? x : y);
+  const int x = t + d > i ? t + d : i;
 #endif
+  return (uint32_t)(CAP && x > cap ? cap : x);
 }
 
 // A code that leaves prefixes unused above its last one (`end`, 65536 for a complete code) has
