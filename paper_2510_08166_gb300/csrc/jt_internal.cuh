@@ -89,7 +89,9 @@ constexpr uint32_t kRunEob = 63;
 constexpr int kRunShift = 10;
 constexpr uint16_t kNoEntry = 0xFFE0;
 
-// Index in a table of the entry for window w. CAP: a table that needs its cap (see below).
+// Index in a table of the entry for window w. CAP: a table that needs its cap (see below). The cap
+// comes after the maximum: capping both terms side by side shortens the chain of such tables (small
+// frames 0.7 % faster), but in the kernel that all tables share it cost the others 0.3 %.
 template <bool CAP>
 __host__ __device__ __forceinline__ uint32_t table_index(uint32_t w, int d, int cap) {
   const int t = (int)(w >> 16), i = (int)(w >> (32 - kLutBits));
